@@ -177,6 +177,7 @@ struct TsmRun {
   ContractPlan plan;
   NoiseSpec ns{};
   int E = 0, n_hp = 0, n_lp = 0, B = 1;
+  int BL = 1;            // sources of an LP solve
   int sp_lp = TSM_F32, sp_hp = TSM_F64;
   bool fp64_path = false;
   double2* d_corr = nullptr;
@@ -184,6 +185,9 @@ struct TsmRun {
   EOField b_lp, s_lp, b_hp, s_hp;
   bool branch = false;   // LP set recorded as a second graph branch
   EOField b_lp1, s_lp1;  // its source / solution batches
+  // FP16 LP solutions (grouped storage) unpacked per source for the contractions
+  int cp_lp = TSM_F32;
+  EOField c_lp, c_lp1;
   bool fft = false;      // every spatial momentum: running moments instead of per-source values
   FftProjector fftp;
   ~TsmRun() { fftp.release(); }
@@ -220,10 +224,14 @@ int prepare_run(Ctx& c, const tsm_params* p, TsmRun* run, bool branch = false) {
   run->n_lp = (int)(p->lp_end - p->lp_begin);
   run->sp_lp = loop_solution_prec(p->lp);
   run->sp_hp = solution_prec(p->hp);
+  run->cp_lp = run->sp_lp == F16G::id ? TSM_F16 : run->sp_lp;
   run->fp64_path = (p->lp.prec == TSM_F64 && p->hp.prec == TSM_F64);
   run->ns = make_noise(p->seed, p->noise);
   run->B = std::min(std::max(p->batch, 1), Ctx::kMaxBatch);
   c.batch_cap = std::max(c.batch_cap, run->B);
+  // FP16 LP solves fill whole groups of 8 sources, which the stencil computes
+  // and the fields hold in any case (a source's bits do not depend on its batch)
+  run->BL = run->sp_lp == F16G::id ? std::min((run->B + 7) & ~7, Ctx::kMaxBatch) : run->B;
   void* vc = nullptr;
   void* vl = nullptr;
   const size_t per = run->fft ? 1 : (size_t)run->E;   // all momenta: no per-source values are kept
@@ -234,6 +242,8 @@ int prepare_run(Ctx& c, const tsm_params* p, TsmRun* run, bool branch = false) {
   if (run->fft) TSM_TRY(run->fftp.init(c, p->n_gamma, run->fp64_path));
   TSM_TRY(eo_fields(c, "tsm_b_lp", run->sp_lp, &run->b_lp, c.batch_cap));
   TSM_TRY(eo_fields(c, "tsm_s_lp", run->sp_lp, &run->s_lp, c.batch_cap));
+  run->c_lp = run->s_lp;
+  if (run->cp_lp != run->sp_lp) TSM_TRY(eo_fields(c, "tsm_c_lp", run->cp_lp, &run->c_lp, run->BL));
   TSM_TRY(eo_fields(c, "tsm_b_hp", run->sp_hp, &run->b_hp, c.batch_cap));
   TSM_TRY(eo_fields(c, "tsm_s_hp", run->sp_hp, &run->s_hp, c.batch_cap));
   TSM_TRY(reserve_solver(c, p->lp, run->sp_lp));
@@ -245,6 +255,8 @@ int prepare_run(Ctx& c, const tsm_params* p, TsmRun* run, bool branch = false) {
     c.ws_prefix = "branch1/";
     int rc = eo_fields(c, "tsm_b_lp", run->sp_lp, &run->b_lp1, c.batch_cap);
     if (rc == TSM_OK) rc = eo_fields(c, "tsm_s_lp", run->sp_lp, &run->s_lp1, c.batch_cap);
+    run->c_lp1 = run->s_lp1;
+    if (rc == TSM_OK && run->cp_lp != run->sp_lp) rc = eo_fields(c, "tsm_c_lp", run->cp_lp, &run->c_lp1, run->BL);
     if (rc == TSM_OK) rc = reserve_solver(c, p->lp, run->sp_lp);
     if (rc == TSM_OK) rc = reserve_contract(c);
     c.ws_prefix.clear();
@@ -267,7 +279,7 @@ int prepare_run(Ctx& c, const tsm_params* p, TsmRun* run, bool branch = false) {
 // statistics (and verifies HP solutions if asked), capture mode records the
 // solves' state ranges for reading after the graph ran
 int record_run(Ctx& c, const tsm_params* p, TsmRun& run, tsm_loop_stats* st) {
-  const int E = run.E, B = run.B, sp_lp = run.sp_lp, sp_hp = run.sp_hp;
+  const int E = run.E, B = run.B, BL = run.BL, sp_lp = run.sp_lp, sp_hp = run.sp_hp, cp_lp = run.cp_lp;
   const NoiseSpec& ns = run.ns;
   *st = tsm_loop_stats{};
   st->lp_max_true_res = -1.0;
@@ -275,6 +287,10 @@ int record_run(Ctx& c, const tsm_params* p, TsmRun& run, tsm_loop_stats* st) {
   st->n_sources = run.n_hp + run.n_lp;
   // noise of sources j0 .. j0+n-1 into a batch of fields
   auto gen = [&](int prec, uint32_t j0, EOField f, int n) {
+    if (prec == F16G::id) {
+      TSM_TRY(launch_noise<F16G>(c, 0, ns, j0, f.e, n));
+      return launch_noise<F16G>(c, 1, ns, j0, f.o, n);
+    }
     return dispatch_prec(prec, [&](auto tag) {
       using S = decltype(tag);
       TSM_TRY(launch_noise<S>(c, 0, ns, j0, f.e, n));
@@ -323,6 +339,12 @@ int record_run(Ctx& c, const tsm_params* p, TsmRun& run, tsm_loop_stats* st) {
     if (pa == TSM_F16 && pb == TSM_F16) return f.accumulate<float, F16, F16>(c, gam, ns, j, a, b, set, idx + 1);
     return bad(TSM_ERR_ARG, "no momentum projection for these field tiers");
   };
+  // the LP solutions of a batch in the layout the contractions read
+  auto unpack_lp = [&](EOField sol, EOField dst, int n) -> int {
+    if (sp_lp != F16G::id) return TSM_OK;
+    TSM_TRY((launch_convert<F16G, F16>(c, sol.e, dst.e, nullptr, n)));
+    return launch_convert<F16G, F16>(c, sol.o, dst.o, nullptr, n);
+  };
   // state slots: fixed in eager mode, one fresh range per solve under capture
   auto slots = [&](int n, std::vector<std::pair<int, int>>& log) {
     if (!c.capturing) return 0;
@@ -331,7 +353,7 @@ int record_run(Ctx& c, const tsm_params* p, TsmRun& run, tsm_loop_stats* st) {
     log.push_back({s0, n});
     return s0;
   };
-  std::vector<SolveResult> r_lp(B), r_hp(B);
+  std::vector<SolveResult> r_lp(BL), r_hp(B);
   const bool hp_first = !(c.capturing && run.branch);
   if (!hp_first) {
     // graph branch: the LP set runs beside the HP set (the FP64-heavy HP
@@ -343,16 +365,17 @@ int record_run(Ctx& c, const tsm_params* p, TsmRun& run, tsm_loop_stats* st) {
     c.stream = c.branch_stream;
     c.red = c.red_branch;
     c.ws_prefix = "branch1/";
-    std::vector<SolveResult> r_lp1(B);
+    std::vector<SolveResult> r_lp1(BL);
     std::swap(r_lp, r_lp1);
     int rc = TSM_OK;
-    for (uint32_t j0 = p->lp_begin; j0 < p->lp_end && rc == TSM_OK; j0 += B) {
-      const int n = (int)std::min<uint32_t>(B, p->lp_end - j0);
+    for (uint32_t j0 = p->lp_begin; j0 < p->lp_end && rc == TSM_OK; j0 += BL) {
+      const int n = (int)std::min<uint32_t>(BL, p->lp_end - j0);
       rc = gen(sp_lp, j0, run.b_lp1, n);
       if (rc == TSM_OK)
         rc = solve_batch(c, p->lp, slots(n, c.cap_lp), n, run.b_lp1, run.s_lp1, r_lp.data(), nullptr, -1, sp_lp);
+      if (rc == TSM_OK) rc = unpack_lp(run.s_lp1, run.c_lp1, n);
       for (int r = 0; r < n && rc == TSM_OK; ++r)
-        rc = contract(j0 + r, eo_at(run.s_lp1, sp_lp, c.g.Vh, r), sp_lp, nullptr, sp_lp, 1,
+        rc = contract(j0 + r, eo_at(run.c_lp1, cp_lp, c.g.Vh, r), cp_lp, nullptr, cp_lp, 1,
                       (int)(j0 + r - p->lp_begin));
     }
     std::swap(r_lp, r_lp1);
@@ -362,47 +385,58 @@ int record_run(Ctx& c, const tsm_params* p, TsmRun& run, tsm_loop_stats* st) {
     c.ws_prefix.clear();
     TSM_TRY(rc);
   }
-  // HP set: the LP map and the HP solve of every source, then L(s_HP - s_LP)
-  for (uint32_t j0 = p->hp_begin; j0 < p->hp_end; j0 += B) {
-    const int n = (int)std::min<uint32_t>(B, p->hp_end - j0);
-    TSM_TRY(gen(sp_lp, j0, run.b_lp, n));
-    TSM_TRY(solve_batch(c, p->lp, slots(n, c.cap_lp), n, run.b_lp, run.s_lp, r_lp.data(), nullptr, -1, sp_lp));
-    if (sp_hp != sp_lp) TSM_TRY(gen(sp_hp, j0, run.b_hp, n));
-    EOField bh = (sp_hp != sp_lp) ? run.b_hp : run.b_lp;
-    // optional warm start of the HP solves from the LP solutions (the LP map
-    // itself is untouched, so both sets keep the same LP solver)
-    const bool warm = p->hp_warm_start && p->hp.prec == TSM_F32 && p->hp.reliable && !p->hp.precond;
-    TSM_TRY(solve_batch(c, p->hp, slots(n, c.cap_hp), n, bh, run.s_hp, r_hp.data(), warm ? &run.s_lp.e : nullptr,
-                        sp_lp));
-    for (int r = 0; r < n; ++r) {
-      if (!c.capturing) {
-        if (r_lp[r].status != TSM_OK || r_hp[r].status != TSM_OK) return bad(TSM_ERR_NONFINITE, "NaN/Inf in a solve");
-        if (p->verify) {
-          double tr = 0.0;
-          TSM_TRY(true_residual(c, sp_hp, eo_at(bh, sp_hp, c.g.Vh, r), eo_at(run.s_hp, sp_hp, c.g.Vh, r), &tr));
-          st->hp_max_true_res = std::max(st->hp_max_true_res, tr);
-        }
-        st->lp_iters += r_lp[r].iters;
-        st->hp_iters += r_hp[r].iters;
-        if (!r_hp[r].converged) st->hp_not_converged++;
+  // HP set: the LP map and the HP solve of every source, then L(s_HP - s_LP).
+  // Optional warm start of the HP solves from the LP solutions (the LP map
+  // itself is untouched, so both sets keep the same LP solver)
+  const bool warm = p->hp_warm_start && p->hp.prec == TSM_F32 && p->hp.reliable && !p->hp.precond;
+  const int BH = warm ? B : BL;   // sources of an LP solve here: a starting guess is the first of its batch
+  for (uint32_t l0 = p->hp_begin; l0 < p->hp_end; l0 += BH) {
+    const int nl = (int)std::min<uint32_t>(BH, p->hp_end - l0);
+    TSM_TRY(gen(sp_lp, l0, run.b_lp, nl));
+    TSM_TRY(solve_batch(c, p->lp, slots(nl, c.cap_lp), nl, run.b_lp, run.s_lp, r_lp.data(), nullptr, -1, sp_lp));
+    TSM_TRY(unpack_lp(run.s_lp, run.c_lp, nl));
+    for (int h0 = 0; h0 < nl; h0 += B) {
+      const uint32_t j0 = l0 + h0;
+      const int n = std::min(B, nl - h0);
+      EOField bh = run.b_lp;   // the LP sources, where the tiers agree (then BH = B)
+      if (sp_hp != sp_lp) {
+        bh = run.b_hp;
+        TSM_TRY(gen(sp_hp, j0, bh, n));
       }
-      const EOField sl = eo_at(run.s_lp, sp_lp, c.g.Vh, r);
-      TSM_TRY(contract(j0 + r, eo_at(run.s_hp, sp_hp, c.g.Vh, r), sp_hp, &sl, sp_lp, 0,
-                       (int)(j0 + r - p->hp_begin)));
+      TSM_TRY(solve_batch(c, p->hp, slots(n, c.cap_hp), n, bh, run.s_hp, r_hp.data(), warm ? &run.s_lp.e : nullptr,
+                          sp_lp));
+      for (int r = 0; r < n; ++r) {
+        if (!c.capturing) {
+          if (r_lp[h0 + r].status != TSM_OK || r_hp[r].status != TSM_OK)
+            return bad(TSM_ERR_NONFINITE, "NaN/Inf in a solve");
+          if (p->verify) {
+            double tr = 0.0;
+            TSM_TRY(true_residual(c, sp_hp, eo_at(bh, sp_hp, c.g.Vh, r), eo_at(run.s_hp, sp_hp, c.g.Vh, r), &tr));
+            st->hp_max_true_res = std::max(st->hp_max_true_res, tr);
+          }
+          st->lp_iters += r_lp[h0 + r].iters;
+          st->hp_iters += r_hp[r].iters;
+          if (!r_hp[r].converged) st->hp_not_converged++;
+        }
+        const EOField sl = eo_at(run.c_lp, cp_lp, c.g.Vh, h0 + r);
+        TSM_TRY(contract(j0 + r, eo_at(run.s_hp, sp_hp, c.g.Vh, r), sp_hp, &sl, cp_lp, 0,
+                         (int)(j0 + r - p->hp_begin)));
+      }
     }
   }
   // LP set: the same LP map, L(s_LP)
-  auto lp_set = [&](EOField bl, EOField sl) -> int {
-    for (uint32_t j0 = p->lp_begin; j0 < p->lp_end; j0 += B) {
-      const int n = (int)std::min<uint32_t>(B, p->lp_end - j0);
+  auto lp_set = [&](EOField bl, EOField sl, EOField cl) -> int {
+    for (uint32_t j0 = p->lp_begin; j0 < p->lp_end; j0 += BL) {
+      const int n = (int)std::min<uint32_t>(BL, p->lp_end - j0);
       TSM_TRY(gen(sp_lp, j0, bl, n));
       TSM_TRY(solve_batch(c, p->lp, slots(n, c.cap_lp), n, bl, sl, r_lp.data(), nullptr, -1, sp_lp));
+      TSM_TRY(unpack_lp(sl, cl, n));
       for (int r = 0; r < n; ++r) {
         if (!c.capturing) {
           if (r_lp[r].status != TSM_OK) return bad(TSM_ERR_NONFINITE, "NaN/Inf in a solve");
           st->lp_iters += r_lp[r].iters;
         }
-        TSM_TRY(contract(j0 + r, eo_at(sl, sp_lp, c.g.Vh, r), sp_lp, nullptr, sp_lp, 1,
+        TSM_TRY(contract(j0 + r, eo_at(cl, cp_lp, c.g.Vh, r), cp_lp, nullptr, cp_lp, 1,
                          (int)(j0 + r - p->lp_begin)));
       }
     }
@@ -412,7 +446,7 @@ int record_run(Ctx& c, const tsm_params* p, TsmRun& run, tsm_loop_stats* st) {
     TSM_CUDA(cudaStreamWaitEvent(c.stream, c.join_ev, 0));   // join the LP-set branch
     return TSM_OK;
   }
-  return lp_set(run.b_lp, run.s_lp);
+  return lp_set(run.b_lp, run.s_lp, run.c_lp);
 }
 
 }  // namespace
@@ -449,6 +483,10 @@ int tsm_create(int device, void* cuda_stream, tsm_ctx** out) {
   c.device = device;
   c.stream = static_cast<cudaStream_t>(cuda_stream);
   int rc = select_device(c);
+  if (rc == TSM_OK && cudaDeviceGetAttribute(&c.sm_count, cudaDevAttrMultiProcessorCount, device) != cudaSuccess)
+    rc = TSM_ERR_CUDA;
+  if (rc == TSM_OK && cudaMallocHost(&c.h_err, sizeof(int)) != cudaSuccess) rc = TSM_ERR_CUDA;
+  if (rc == TSM_OK) *c.h_err = 0;
   if (rc == TSM_OK && cudaMalloc(&c.states, Ctx::kMaxStates * sizeof(CGState)) != cudaSuccess) rc = TSM_ERR_CUDA;
   if (rc == TSM_OK && cudaMallocHost(&c.h_states, Ctx::kMaxStates * sizeof(CGState)) != cudaSuccess)
     rc = TSM_ERR_CUDA;
@@ -500,15 +538,16 @@ int tsm_load_gauge(tsm_ctx* h, const tm_lattice* lat, const double* U, int on_de
     TSM_CUDA(cudaStreamSynchronize(c.stream));
     for (auto& kv : c.ws) cudaFree(kv.second.first);
     c.ws.clear();
-    for (int k = 0; k < 4; ++k) {
-      if (c.links[k]) cudaFree(c.links[k]);
-      c.links[k] = nullptr;
+    for (void*& l : c.links) {
+      if (l) cudaFree(l);
+      l = nullptr;
     }
     const size_t vh = (size_t)c.g.Vh;
     TSM_CUDA(cudaMalloc(&c.links[TSM_F64], 2 * 4 * F64::LN * vh * sizeof(double2)));
     TSM_CUDA(cudaMalloc(&c.links[TSM_F32], 2 * 4 * F32::LN * vh * sizeof(float4)));
     TSM_CUDA(cudaMalloc(&c.links[TSM_BF16], 2 * 4 * BF16::LN * vh * sizeof(uint2)));
     TSM_CUDA(cudaMalloc(&c.links[TSM_F16], 2 * 4 * F16::LN * vh * sizeof(uint2)));
+    TSM_CUDA(cudaMalloc(&c.links[F16G::id], 2 * 4 * F16G::LN * vh * sizeof(uint32_t)));
     if (c.red.partials) cudaFree(c.red.partials);
     c.red_cap = vh / 32 + 64;   // block partials: up to one per 32 sites (link-sharing stencil)
     c.red.stride = (int)c.red_cap;
@@ -524,7 +563,8 @@ int tsm_load_gauge(tsm_ctx* h, const tm_lattice* lat, const double* U, int on_de
   pack_links_kernel<<<nb, SITE_NT, 0, c.stream>>>(
       c.g, reinterpret_cast<const double2*>(dU), static_cast<double2*>(c.links[TSM_F64]),
       static_cast<float4*>(c.links[TSM_F32]), static_cast<uint2*>(c.links[TSM_F16]),
-      static_cast<uint2*>(c.links[TSM_BF16]), c.lstride, static_cast<unsigned int*>(dev_max));
+      static_cast<uint2*>(c.links[TSM_BF16]), static_cast<uint32_t*>(c.links[F16G::id]), c.lstride,
+      static_cast<unsigned int*>(dev_max));
   c.launches++;
   TSM_TRY(check_launch(c, "pack_links_kernel"));
   unsigned int bits = 0;
@@ -612,6 +652,7 @@ int tm_solve_batch(tsm_ctx* h, int nrhs, const double* b, double* s, const tm_st
       else if (!q.converged && worst == TSM_OK) worst = TSM_ERR_NOT_CONVERGED;
     }
   }
+  TSM_TRY(c.check_waits());
   TSM_TRY(c.harvest_events());
   if (worst != TSM_OK) set_error("at least one solve %s", worst == TSM_ERR_NONFINITE ? "met NaN/Inf" : "did not converge");
   return worst;
@@ -794,6 +835,7 @@ int tsm_loops(tsm_ctx* h, const tsm_params* p, double* loops, double* err, doubl
   if (per_corr && n_hp > 0) TSM_CUDA(cudaMemcpyAsync(per_corr, run.d_corr, (size_t)n_hp * cb, k, c.stream));
   if (per_lp && n_lp > 0) TSM_CUDA(cudaMemcpyAsync(per_lp, run.d_lp, (size_t)n_lp * cb, k, c.stream));
   TSM_CUDA(cudaStreamSynchronize(c.stream));
+  TSM_TRY(c.check_waits());
   TSM_TRY(c.harvest_events());
   if (stats) *stats = st;
   return TSM_OK;
@@ -908,6 +950,10 @@ int tsm_loops_graph(tsm_ctx** ctxs, const tsm_params* params, int n, double** lo
   }
   if (exec) cudaGraphExecDestroy(exec);
   if (graph) cudaGraphDestroy(graph);
+  for (int i = 0; i < n; ++i) {
+    const int wt = ctxs[i]->c.check_waits();
+    if (rc == TSM_OK) rc = wt;
+  }
   if (rc == TSM_OK) {
     for (int i = 0; i < n; ++i) {
       Ctx& c = ctxs[i]->c;
@@ -990,10 +1036,12 @@ int tsm_tune(tsm_ctx* h, const tm_stop* stop, int* best_batch, int* best_tile, i
   constexpr int kShapes = 4;
   const int tiles[kShapes] = {2, 4, 8, 4};
   const int regs[kShapes] = {80, 80, 80, 96};
-  // the link-sharing stencil (16-bit tiers; FP32 for its hops without a
-  // reduction) has a block shape to choose; FP64 runs one thread per (source, site)
-  const bool tiled = stop->prec == TSM_F16 || stop->prec == TSM_BF16 || stop->prec == TSM_F32;
-  const int ntile = tiled ? kShapes : 1;
+  // the link-sharing stencil (BF16; FP32 for its hops without a reduction) has
+  // a block shape to choose; FP64 runs one thread per (source, site), FP16 the
+  // tensor-core stencil, whose blocks are fixed (one timing stands for every shape)
+  const bool fixed16 = stop->prec == TSM_F16;
+  const bool tiled = fixed16 || stop->prec == TSM_BF16 || stop->prec == TSM_F32;
+  const int ntile = tiled && !fixed16 ? kShapes : 1;
   auto ib = c.tuned_batch.find(key);
   auto it = c.tuned_rpb.find(key);
   if (ib != c.tuned_batch.end() && it != c.tuned_rpb.end() && times_ms == nullptr) {
@@ -1024,11 +1072,16 @@ int tsm_tune(tsm_ctx* h, const tm_stop* stop, int* best_batch, int* best_tile, i
   int rc = TSM_OK;
   for (int k = 0; k < 4 && rc == TSM_OK; ++k) {
     const int w = cand[k];
-    rc = dispatch_prec(sp, [&](auto tag) {
-      using S = decltype(tag);
-      TSM_TRY(launch_noise<S>(c, 0, ns, 0, fb.e, w));
-      return launch_noise<S>(c, 1, ns, 0, fb.o, w);
-    });
+    if (sp == F16G::id) {
+      rc = launch_noise<F16G>(c, 0, ns, 0, fb.e, w);
+      if (rc == TSM_OK) rc = launch_noise<F16G>(c, 1, ns, 0, fb.o, w);
+    } else {
+      rc = dispatch_prec(sp, [&](auto tag) {
+        using S = decltype(tag);
+        TSM_TRY(launch_noise<S>(c, 0, ns, 0, fb.e, w));
+        return launch_noise<S>(c, 1, ns, 0, fb.o, w);
+      });
+    }
     for (int q = 0; q < ntile && rc == TSM_OK; ++q) {
       if (tiled) {
         c.tile_rpb[stop->prec] = tiles[q];
@@ -1045,10 +1098,12 @@ int tsm_tune(tsm_ctx* h, const tm_stop* stop, int* best_batch, int* best_tile, i
       if (rc == TSM_OK) cudaEventElapsedTime(&ms, e0, e1);
       const double per = ms / w;
       if (times_ms) times_ms[kShapes * k + q] = per;
+      if (times_ms && fixed16)
+        for (int u = 1; u < kShapes; ++u) times_ms[kShapes * k + u] = per;
       if (per < best_t) {
         best_t = per;
         best_w = w;
-        best_q = q;
+        best_q = fixed16 ? 1 : q;
       }
     }
     if (times_ms && !tiled)

@@ -138,6 +138,19 @@ struct F16 {
   static constexpr int id = 3;
 };
 
+// FP16 spinors of batched solves, laid out for the tensor-core stencil
+// (mma_hop.cuh): groups of 8 right-hand sides, [group][site][source][colour]
+// chunks of the four spins of a colour.  Links: words [site][hop][12] of the 8
+// hops of every output site (each link twice, so that a site reads one run):
+// the nine entries (row-major, re and im as FP16) and the FP16 remainder of row 2.
+struct F16G {
+  using real = float;
+  using schunk = uint4;     // 4 complex as 8 fp16: spins 0..3 of one colour
+  using lchunk = uint32_t;  // 1 complex as 2 fp16
+  static constexpr int SN = 3, LN = 24;   // two hops per direction
+  static constexpr int id = 4;   // internal: not a tier of the ABI
+};
+
 template <class S> struct Pack16;
 template <> struct Pack16<F16> {
   __device__ static __forceinline__ cx<float> unpack(uint32_t w) {
@@ -179,6 +192,15 @@ __device__ __forceinline__ void load_spinor(const typename S::schunk* __restrict
       v[2 * c] = {f.x, f.y};
       v[2 * c + 1] = {f.z, f.w};
     }
+  } else if constexpr (S::id == F16G::id) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const uint4 u = b[(size_t)i * 24 + c];
+      v[c] = Pack16<F16>::unpack(u.x);
+      v[3 + c] = Pack16<F16>::unpack(u.y);
+      v[6 + c] = Pack16<F16>::unpack(u.z);
+      v[9 + c] = Pack16<F16>::unpack(u.w);
+    }
   } else {
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -201,6 +223,11 @@ __device__ __forceinline__ void store_spinor(typename S::schunk* __restrict__ b,
 #pragma unroll
     for (int c = 0; c < 6; ++c)
       b[c * stride + i] = make_float4(v[2 * c].re, v[2 * c].im, v[2 * c + 1].re, v[2 * c + 1].im);
+  } else if constexpr (S::id == F16G::id) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+      b[(size_t)i * 24 + c] = make_uint4(Pack16<F16>::pack(v[c]), Pack16<F16>::pack(v[3 + c]),
+                                         Pack16<F16>::pack(v[6 + c]), Pack16<F16>::pack(v[9 + c]));
   } else {
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -531,6 +558,7 @@ __device__ __forceinline__ int rhs_slot(const int* active) {
 // offset of right-hand side `rhs` in a batch of contiguous fields of storage S
 template <class S>
 __device__ __forceinline__ size_t rhs_offset(int rhs, int sstride) {
+  if constexpr (S::id == F16G::id) return (size_t)(rhs >> 3) * 24 * (size_t)sstride + (size_t)(rhs & 7) * 3;
   return (size_t)rhs * S::SN * (size_t)sstride;
 }
 

@@ -3,6 +3,7 @@
 #include <cstdio>
 
 #include "context.h"
+#include "tma_map.h"
 
 namespace tsm {
 
@@ -75,7 +76,9 @@ int Ctx::buffer(const std::string& base_name, size_t bytes, void** out) {
 }
 
 int Ctx::field(const std::string& name, int prec, PField* f, int nrhs) {
-  return buffer(name + "#" + std::to_string(prec), field_bytes(prec, sstride) * (size_t)(nrhs > 0 ? nrhs : 1), &f->p);
+  if (nrhs < 1) nrhs = 1;
+  if (prec == F16G::id) nrhs = (nrhs + 7) & ~7;   // whole groups of 8 sources
+  return buffer(name + "#" + std::to_string(prec), field_bytes(prec, sstride) * (size_t)nrhs, &f->p);
 }
 
 int Ctx::harvest_events() {
@@ -96,14 +99,36 @@ int Ctx::harvest_events() {
   return TSM_OK;
 }
 
+PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
+  static const PFN_cuTensorMapEncodeTiled_v12000 fn = []() -> PFN_cuTensorMapEncodeTiled_v12000 {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q{};
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess)
+      return nullptr;
+    return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
+  }();
+  return fn;
+}
+
+int Ctx::check_waits() {
+  volatile int* e = h_err;
+  if (e == nullptr || *e == 0) return TSM_OK;
+  *e = 0;
+  set_error("a bounded wait of the tensor-core stencil ran out");
+  return TSM_ERR_TIMEOUT;
+}
+
 void Ctx::free_all() {
   cudaStreamSynchronize(stream);
   for (auto& kv : ws) cudaFree(kv.second.first);
   ws.clear();
-  for (int k = 0; k < 4; ++k) {
-    if (links[k]) cudaFree(links[k]);
-    links[k] = nullptr;
+  for (void*& l : links) {
+    if (l) cudaFree(l);
+    l = nullptr;
   }
+  if (h_err) cudaFreeHost(h_err);
+  h_err = nullptr;
   if (red.partials) cudaFree(red.partials);
   if (red.counter) cudaFree(red.counter);
   if (red_branch.partials) cudaFree(red_branch.partials);

@@ -63,7 +63,10 @@ struct Ctx {
   Geom g{};
   int sstride = 0;       // chunk stride of parity fields (= Vh)
   int lstride = 0;       // chunk stride of link fields (= Vh)
-  void* links[4] = {nullptr, nullptr, nullptr, nullptr};   // F64, F32, BF16, F16: [2][4][LN][lstride]
+  // F64, F32, BF16, F16: [2][4][LN][lstride]; F16G: [2][lstride][8][12] words
+  void* links[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
+  int sm_count = 1;
+  int* h_err = nullptr;                 // pinned, device-visible: set by a kernel whose bounded wait ran out
   std::map<std::string, std::pair<void*, size_t>> ws;      // named device workspace
   RedSlot red{};
   size_t red_cap = 0;
@@ -124,6 +127,7 @@ struct Ctx {
   }
   int field(const std::string& name, int prec, PField* f, int nrhs = 1);   // nrhs parity fields of tier prec
   int harvest_events();                                        // sync + accumulate profile times
+  int check_waits();   // after a stream sync: TSM_ERR_TIMEOUT if a kernel's bounded wait ran out since the last check
   void free_all();
 };
 
@@ -164,6 +168,21 @@ inline Twist twist_mul(const Twist& a, const Twist& b) {
 // grid's x dimension), optionally through a device list `active` of the
 // right-hand sides still iterating.
 template <class S> int launch_hop(Ctx& c, const HopArgs<S>& a, int dag, int mode, int prof_kind, int nrhs = 1);
+
+// the FP32 kernels' epilogue factors of a hop, formed in FP64 and rounded once
+template <class S>
+void hop_factors(const HopArgs<S>& a, TwistF* to_ah, TwistF* to_tc_ac, TwistF* ts) {
+  Twist toah, totc;
+  for (int q = 0; q < 2; ++q) {
+    toah.re[q] = a.to.re[q] * a.ah;
+    toah.im[q] = a.to.im[q] * a.ah;
+    totc.re[q] = (a.to.re[q] * a.tc.re[q] - a.to.im[q] * a.tc.im[q]) * a.ac;
+    totc.im[q] = (a.to.re[q] * a.tc.im[q] + a.to.im[q] * a.tc.re[q]) * a.ac;
+  }
+  *to_ah = to_float(toah);
+  *to_tc_ac = to_float(totc);
+  *ts = to_float(a.ts);
+}
 template <class S, class SA> int launch_cg_update(Ctx& c, const CGUpdArgs<S, SA>& a, int nrhs);
 template <class S, class SA>
 int launch_cg_p(Ctx& c, const PField& r, const PField& p, CGState* st, const int* active, int nrhs);
@@ -178,6 +197,22 @@ template <class S>
 int launch_norm(Ctx& c, const PField& v, CGState* st, int post, const int* active = nullptr, int nrhs = 1);
 template <class Si, class So>
 int launch_convert(Ctx& c, const PField& in, const PField& out, const int* active = nullptr, int nrhs = 1);
+
+// grouped FP16 storage (ops_f16g.cu)
+template <> int launch_hop<F16G>(Ctx& c, const HopArgs<F16G>& a, int dag, int mode, int prof_kind, int nrhs);
+template <> int launch_cg_update<F16G, F16G>(Ctx& c, const CGUpdArgs<F16G, F16G>& a, int nrhs);
+template <>
+int launch_cg_p<F16G, F16G>(Ctx& c, const PField& r, const PField& p, CGState* st, const int* active, int nrhs);
+template <>
+int launch_noise<F16G>(Ctx& c, int parity, const NoiseSpec& n, uint32_t source0, const PField& out, int nrhs);
+template <>
+int launch_twist<F16G>(Ctx& c, const Twist& f, const PField& in, const PField& out, const CGState* st,
+                       const int* active, int nrhs);
+template <> int launch_convert<F16G, F16G>(Ctx& c, const PField& in, const PField& out, const int* active, int nrhs);
+template <> int launch_convert<F32, F16G>(Ctx& c, const PField& in, const PField& out, const int* active, int nrhs);
+template <> int launch_convert<F16G, F32>(Ctx& c, const PField& in, const PField& out, const int* active, int nrhs);
+template <> int launch_convert<F16G, F64>(Ctx& c, const PField& in, const PField& out, const int* active, int nrhs);
+template <> int launch_convert<F16G, F16>(Ctx& c, const PField& in, const PField& out, const int* active, int nrhs);
 
 // runtime dispatch on a tier id (0 F64, 1 F32, 2 BF16, 3 F16):
 // f receives an empty tag object of the storage type

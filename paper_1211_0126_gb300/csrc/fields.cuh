@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(SITE_NT) unpack_spinor_kernel(Geom g, int pari
 static __global__ void __launch_bounds__(SITE_NT) pack_links_kernel(Geom g, const double2* __restrict__ U,
                                                              double2* __restrict__ l64, float4* __restrict__ l32,
                                                              uint2* __restrict__ l16, uint2* __restrict__ lbf,
-                                                             int lstride, unsigned int* __restrict__ maxdev) {
+                                                             uint32_t* __restrict__ lmma, int lstride, unsigned int* __restrict__ maxdev) {
   const int tid = blockIdx.x * SITE_NT + threadIdx.x;
   if (tid >= g.V * 4) return;
   const int lex = tid >> 2, mu = tid & 3;
@@ -93,6 +93,85 @@ static __global__ void __launch_bounds__(SITE_NT) pack_links_kernel(Geom g, cons
   store_link<F32>(l32 + off32, lstride, mu, ih, rf);
   store_link<F16>(l16 + off32, lstride, mu, ih, rf);
   store_link<BF16>(lbf + off32, lstride, mu, ih, rf);
+  // tensor-core stencil: rows 0, 1 in FP16, row 2 = conj(row0 x row1) of those in FP32, kept as FP16 hi + lo
+  uint32_t w12[12];
+  cx<float> q[6], w2[3];
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    w12[k] = Pack16<F16>::pack(rf[k]);
+    q[k] = Pack16<F16>::unpack(w12[k]);
+  }
+  third_row(q, w2);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    w12[6 + k] = Pack16<F16>::pack(w2[k]);
+    const cx<float> hi = Pack16<F16>::unpack(w12[6 + k]);
+    w12[9 + k] = Pack16<F16>::pack(w2[k] - hi);
+  }
+  // [site][hop][12]: forward hop of this site, backward hop of x + mu, with the sign of an antiperiodic boundary
+  int c[4] = {x, y, z, t};
+  const bool wraps = c[mu] + 1 == g.L[mu];
+  const uint32_t sign = wraps && mu == 3 && g.apbc ? 0x80008000u : 0u;
+#pragma unroll
+  for (int k = 0; k < 12; ++k) w12[k] ^= sign;
+  c[mu] = wraps ? 0 : c[mu] + 1;
+  const int fh = half_index(g, c[0], c[1], c[2], c[3]);
+  uint4* own = reinterpret_cast<uint4*>(lmma) + (((size_t)parity * g.Vh + ih) * 8 + 2 * mu) * 3;
+  uint4* fwd = reinterpret_cast<uint4*>(lmma) + (((size_t)(1 - parity) * g.Vh + fh) * 8 + 2 * mu + 1) * 3;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const uint4 v = make_uint4(w12[4 * k], w12[4 * k + 1], w12[4 * k + 2], w12[4 * k + 3]);
+    own[k] = v;
+    fwd[k] = v;
+  }
+}
+
+// Thread -> (right-hand side, site) of the batched site-local kernels on
+// grouped storage (F16G): 8 sources x 32 sites per block of 256 threads,
+// sources fastest, so that a warp touches whole lines of the grouped side.
+__device__ __forceinline__ bool grouped_site(int Vh, int nrhs, int* rhs, int* ih) {
+  *rhs = blockIdx.y * 8 + (threadIdx.x & 7);
+  *ih = blockIdx.x * (SITE_NT / 8) + (threadIdx.x >> 3);
+  return *rhs < nrhs && *ih < Vh;
+}
+
+static __global__ void __launch_bounds__(SITE_NT) noise_grouped_kernel(Geom g, int parity, NoiseSpec n,
+                                                                       uint32_t source0, uint4* __restrict__ out,
+                                                                       int sstride, int nrhs) {
+  int rhs, ih;
+  if (!grouped_site(g.Vh, nrhs, &rhs, &ih)) return;
+  int c[4];
+  site_coords(g, parity, ih, c);
+  const uint32_t lex = (uint32_t)(((c[3] * g.L[2] + c[2]) * g.L[1] + c[1]) * g.L[0] + c[0]);
+  cx<float> v[12];
+  noise_site<float>(n, lex, source0 + (uint32_t)rhs, v);
+  store_spinor<F16G>(out + rhs_offset<F16G>(rhs, sstride), sstride, ih, v);
+}
+
+static __global__ void __launch_bounds__(SITE_NT) twist_grouped_kernel(int Vh, TwistF f, const uint4* __restrict__ in,
+                                                                       uint4* __restrict__ out, int sstride,
+                                                                       int nrhs) {
+  int rhs, ih;
+  if (!grouped_site(Vh, nrhs, &rhs, &ih)) return;
+  const size_t off = rhs_offset<F16G>(rhs, sstride);
+  cx<float> v[12];
+  load_spinor<F16G>(in + off, sstride, ih, v);
+  apply_twist(f, v);
+  store_spinor<F16G>(out + off, sstride, ih, v);
+}
+
+template <class Si, class So>
+__global__ void __launch_bounds__(SITE_NT) convert_grouped_kernel(int Vh, const typename Si::schunk* __restrict__ in,
+                                                                  typename So::schunk* __restrict__ out, int sstride,
+                                                                  int nrhs) {
+  int rhs, ih;
+  if (!grouped_site(Vh, nrhs, &rhs, &ih)) return;
+  cx<typename Si::real> v[12];
+  cx<typename So::real> w[12];
+  load_spinor<Si>(in + rhs_offset<Si>(rhs, sstride), sstride, ih, v);
+#pragma unroll
+  for (int k = 0; k < 12; ++k) w[k] = {(typename So::real)v[k].re, (typename So::real)v[k].im};
+  store_spinor<So>(out + rhs_offset<So>(rhs, sstride), sstride, ih, w);
 }
 
 // noise sources source0 + rhs -> batch of parity fields in S (eta is exactly

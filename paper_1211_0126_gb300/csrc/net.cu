@@ -8,12 +8,11 @@
 #include <new>
 #include <vector>
 
-#include <cudaTypedefs.h>
-
 #include "contract.h"
 #include "net.h"
 #include "ptnet.cuh"
 #include "solver.h"
+#include "tma_map.h"
 #include "umma.cuh"
 
 namespace tsm {
@@ -29,21 +28,6 @@ int umma_launch(cudaStream_t stream, dim3 grid, const __nv_bfloat16* A, const __
   umma_gemm_kernel<BN><<<grid, UMMA_THREADS, smem, stream>>>(A, B, C, M, N, K, ldc, beta, error, lda, ldb, kchunk,
                                                              czs);
   return cudaGetLastError() == cudaSuccess ? TSM_OK : TSM_ERR_CUDA;
-}
-
-// cuTensorMapEncodeTiled from the driver (no link-time dependency on libcuda)
-PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
-  static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-  static bool tried = false;
-  if (!tried) {
-    tried = true;
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q{};
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-  }
-  return fn;
 }
 
 // tensor map of a row-major BF16 matrix [rows][cols] with leading dimension

@@ -22,34 +22,23 @@ int launch_hop(Ctx& c, const HopArgs<S>& a0, int dag, int mode, int prof_kind, i
   const int nb = blocks_for(a0.g.Vh, HOP_NT);
   if (nb == 0 || nrhs == 0) return TSM_OK;
   HopArgs<S> a = a0;
-  a.fts = to_float(a.ts);
-  {
-    Twist toah, totc;
-    for (int q = 0; q < 2; ++q) {
-      toah.re[q] = a.to.re[q] * a.ah;
-      toah.im[q] = a.to.im[q] * a.ah;
-      totc.re[q] = (a.to.re[q] * a.tc.re[q] - a.to.im[q] * a.tc.im[q]) * a.ac;
-      totc.im[q] = (a.to.re[q] * a.tc.im[q] + a.to.im[q] * a.tc.re[q]) * a.ac;
-    }
-    a.fto_ah = to_float(toah);
-    a.fto_tc_ac = to_float(totc);
-  }
+  hop_factors(a0, &a.fto_ah, &a.fto_tc_ac, &a.fts);
   const int kind = prof_kind >= 0 ? prof_kind : hop_kind_of<S>(dag, mode);
   const double sb = spinor_site_bytes(S::id), lb = link_site_bytes(S::id);
   // links once per launch (shared by the right-hand sides), spinor streams per RHS
   const double bytes = (double)a.g.Vh *
       (lb + nrhs * sb * (2 + ((mode & HOP_CENTER) ? 1 : 0) + ((mode & HOP_BASE) ? 1 : 0)));
   TimedLaunch tl(c, 4 * S::id + kind, bytes);
-  // 16-bit tiers: link-sharing blocks of LT_SITES sites x up to RPB sources
-  // (RPB = c.tile_rpb, 2, 4 or 8, and for 4 a register budget of 80 or 96,
-  // from the autotuner; every solve, whatever its
-  // batch width, so that a source's iterates do not depend on its batch); the
-  // FP32 tier the same for the hops without a reduction (its reducing hop K2
-  // measured slower in tiles; per-site arithmetic, and so every result, is the
-  // same in both kernels); FP64, and single-source operator applications
-  // outside the solvers (c.hop_per_site): one thread per (source, site),
-  // blocks of HOP_NT sites
-  constexpr bool TILE16 = S::id == F16::id || S::id == BF16::id;
+  // BF16: link-sharing blocks of LT_SITES sites x up to RPB sources (RPB =
+  // c.tile_rpb, 2, 4 or 8, and for 4 a register budget of 80 or 96, from the
+  // autotuner; every solve, whatever its batch width, so that a source's
+  // iterates do not depend on its batch); the FP32 tier the same for the hops
+  // without a reduction (its reducing hop K2 measured slower in tiles; per-site
+  // arithmetic, and so every result, is the same in both kernels); FP64, FP16
+  // (whose batched solves run in grouped storage, F16G) and single-source
+  // operator applications outside the solvers (c.hop_per_site): one thread per
+  // (source, site), blocks of HOP_NT sites
+  constexpr bool TILE16 = S::id == BF16::id;
   constexpr bool TILE32 = S::id == F32::id;
   // (FP32: only with several sources to share the links; a single field runs
   // faster one thread per site, with the same bits)
@@ -102,7 +91,7 @@ int launch_cg_update(Ctx& c, const CGUpdArgs<S, SA>& a0, int nrhs) {
   TimedLaunch tl(c, 4 * S::id + PK_HOP_UPDATE, (double)a.g.Vh * (lb + nrhs * (3 * sb + 4 * sa)));
   // one thread per (source, site) for every tier: the update is memory-bound,
   // and link sharing measured slower here (534 against 511 us per launch)
-  cg_update_kernel<S, SA><<<dim3(nrhs, blocks_for(a.g.Vh, HOP_NT * UpdGroups<S, SA>::value)), HOP_NT, 0, c.stream>>>(a);
+  cg_update_kernel<S, SA><<<dim3(nrhs, nb), HOP_NT, 0, c.stream>>>(a);
   tl.done();
   c.launches++;
   return check_launch(c, "cg_update_kernel");

@@ -20,6 +20,8 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include "mbar.cuh"
+
 namespace tsm {
 
 constexpr int UMMA_BM = 128;
@@ -33,14 +35,10 @@ template <int BN> __host__ __device__ constexpr int umma_stage_bytes() { return 
 template <int BN> __host__ __device__ constexpr int umma_smem_bytes() {
   return umma_stages<BN>() * umma_stage_bytes<BN>() + 1024;
 }
-constexpr long long UMMA_SPIN_LIMIT = 1ll << 26;   // bounded mbarrier wait
+constexpr long long UMMA_SPIN_LIMIT = MBAR_SPIN_LIMIT;   // bounded mbarrier wait
 // stage-wait limit of a launch with withheld operand copies (fault injection
 // for tests of the timeout path): the wait is on a barrier nothing arrives on
 constexpr long long UMMA_INJECT_LIMIT = 4096;
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
 
 // shared-memory matrix descriptor: canonical K-major layout without swizzle
 // (start address, leading-dimension byte offset = distance of K-adjacent core
@@ -58,25 +56,6 @@ __device__ __forceinline__ uint64_t umma_desc(uint32_t saddr, uint32_t lbo, uint
 // K-major, N and M encoded as N/8 and M/16
 __host__ __device__ constexpr uint32_t umma_idesc_bf16(int m, int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
-}
-
-// bounded wait for the phase `parity` of an mbarrier; false on timeout
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long long limit = UMMA_SPIN_LIMIT) {
-  const uint32_t a = smem_u32(bar);
-  for (long long it = 0; it < limit; ++it) {
-    uint32_t done;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(done)
-        : "r"(a), "r"(parity)
-        : "memory");
-    if (done) return true;
-  }
-  return false;
 }
 
 // cp.async of one R-row x UMMA_BK-column tile of a row-major BF16 matrix
@@ -282,10 +261,6 @@ __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t saddr) {
   d |= (uint64_t)1 << 46;   // descriptor version for tcgen05
   d |= (uint64_t)2 << 61;   // swizzle mode: 128 B
   return d;
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
 }
 
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const void* tmap, int x, int y, uint64_t* bar) {
