@@ -61,20 +61,12 @@ int stage_out_finish(Ctx& c, double* user, const double* dev, size_t bytes, int 
 
 size_t spinor_bytes(const Ctx& c) { return (size_t)c.g.V * 24 * sizeof(double); }
 
-int pack_eo(Ctx& c, int prec, const double* canon, EOField f) {
-  return dispatch_prec(prec, [&](auto tag) {
-    using S = decltype(tag);
-    TSM_TRY(launch_pack<S>(c, 0, canon, f.e));
-    return launch_pack<S>(c, 1, canon, f.o);
-  });
+int pack_eo(Ctx& c, int prec, const double* canon, EOField f, int nrhs = 1) {
+  return dispatch_prec(prec, [&](auto tag) { return launch_pack<decltype(tag)>(c, canon, f.e, f.o, nrhs); });
 }
 
-int unpack_eo(Ctx& c, int prec, EOField f, double* canon) {
-  return dispatch_prec(prec, [&](auto tag) {
-    using S = decltype(tag);
-    TSM_TRY(launch_unpack<S>(c, 0, f.e, canon));
-    return launch_unpack<S>(c, 1, f.o, canon);
-  });
+int unpack_eo(Ctx& c, int prec, EOField f, double* canon, int nrhs = 1) {
+  return dispatch_prec(prec, [&](auto tag) { return launch_unpack<decltype(tag)>(c, f.e, f.o, canon, nrhs); });
 }
 
 int eo_fields(Ctx& c, const std::string& name, int prec, EOField* f, int nrhs = 1) {
@@ -95,28 +87,26 @@ template <class S>
 int apply_operator(Ctx& c, int op, int dagger, EOField in, EOField out) {
   const double k = c.lat.kappa, mu = c.lat.mu, k2 = k * k;
   const double m = dagger ? -mu : mu;
-  auto zero = [&](PField f) { return launch_convert<S, S>(c, PField{}, f); };
   switch (op) {
-    case TM_OP_FULL:
+    case TM_OP_FULL: {
+      HopArgs<S> h[2] = {hop_args<S>(c, 0), hop_args<S>(c, 1)};
       for (int par = 0; par < 2; ++par) {
-        HopArgs<S> h = hop_args<S>(c, par);
-        h.in = (par ? in.e : in.o).as<S>();
-        h.center = (par ? in.o : in.e).as<S>();
-        h.tc = twist_A(k, m);
-        h.ac = 1.0;
-        h.ah = -k;
-        h.out = (par ? out.o : out.e).as<S>();
-        TSM_TRY(launch_hop<S>(c, h, dagger, HOP_CENTER, -1));
+        h[par].in = (par ? in.e : in.o).as<S>();
+        h[par].center = (par ? in.o : in.e).as<S>();
+        h[par].tc = twist_A(k, m);
+        h[par].ac = 1.0;
+        h[par].ah = -k;
+        h[par].out = (par ? out.o : out.e).as<S>();
       }
-      return TSM_OK;
+      return launch_full<S>(c, h[0], h[1], dagger);
+    }
     case TM_OP_HOP_EO:
     case TM_OP_HOP_OE: {
       const int par = (op == TM_OP_HOP_EO) ? 0 : 1;
       HopArgs<S> h = hop_args<S>(c, par);
       h.in = (par ? in.e : in.o).as<S>();
       h.out = (par ? out.o : out.e).as<S>();
-      TSM_TRY(launch_hop<S>(c, h, dagger, 0, -1));
-      return zero(par ? out.e : out.o);
+      return launch_hop<S>(c, h, dagger, 0, -1);
     }
     case TM_OP_SCHUR:
     case TM_OP_NORMAL: {
@@ -161,7 +151,7 @@ int apply_operator(Ctx& c, int op, int dagger, EOField in, EOField out) {
         h.out = out.e.as<S>();
         TSM_TRY(launch_hop<S>(c, h, 1, HOP_CENTER, -1));
       }
-      return zero(out.o);
+      return TSM_OK;
     }
     default:
       return bad(TSM_ERR_ARG, "unknown operator");
@@ -405,15 +395,18 @@ int record_run(Ctx& c, const tsm_params* p, TsmRun& run, tsm_loop_stats* st) {
       }
       TSM_TRY(solve_batch(c, p->hp, slots(n, c.cap_hp), n, bh, run.s_hp, r_hp.data(), warm ? &run.s_lp.e : nullptr,
                           sp_lp));
-      for (int r = 0; r < n; ++r) {
-        if (!c.capturing) {
+      if (!c.capturing) {
+        for (int r = 0; r < n; ++r)
           if (r_lp[h0 + r].status != TSM_OK || r_hp[r].status != TSM_OK)
             return bad(TSM_ERR_NONFINITE, "NaN/Inf in a solve");
-          if (p->verify) {
-            double tr = 0.0;
-            TSM_TRY(true_residual(c, sp_hp, eo_at(bh, sp_hp, c.g.Vh, r), eo_at(run.s_hp, sp_hp, c.g.Vh, r), &tr));
-            st->hp_max_true_res = std::max(st->hp_max_true_res, tr);
-          }
+        if (p->verify) {
+          std::vector<double> tr(n);
+          TSM_TRY(true_residual(c, sp_hp, bh, run.s_hp, n, tr.data()));
+          for (double v : tr) st->hp_max_true_res = std::max(st->hp_max_true_res, v);
+        }
+      }
+      for (int r = 0; r < n; ++r) {
+        if (!c.capturing) {
           st->lp_iters += r_lp[h0 + r].iters;
           st->hp_iters += r_hp[r].iters;
           if (!r_hp[r].converged) st->hp_not_converged++;
@@ -557,23 +550,22 @@ int tsm_load_gauge(tsm_ctx* h, const tm_lattice* lat, const double* U, int on_de
   const double* dU = nullptr;
   TSM_TRY(stage_in(c, "gauge_canon", U, (size_t)V * 4 * 9 * 2 * sizeof(double), on_device, &dU));
   void* dev_max = nullptr;
-  TSM_TRY(c.buffer("gauge_maxdev", sizeof(unsigned int), &dev_max));
-  TSM_CUDA(cudaMemsetAsync(dev_max, 0, sizeof(unsigned int), c.stream));
-  const int nb = (int)((V * 4 + SITE_NT - 1) / SITE_NT);
+  TSM_TRY(c.buffer("gauge_maxdev", sizeof(double), &dev_max));
+  TSM_CUDA(cudaMemsetAsync(dev_max, 0, sizeof(double), c.stream));
+  const int nb = (int)((V + LINK_SITES - 1) / LINK_SITES);
   pack_links_kernel<<<nb, SITE_NT, 0, c.stream>>>(
       c.g, reinterpret_cast<const double2*>(dU), static_cast<double2*>(c.links[TSM_F64]),
       static_cast<float4*>(c.links[TSM_F32]), static_cast<uint2*>(c.links[TSM_F16]),
       static_cast<uint2*>(c.links[TSM_BF16]), static_cast<uint32_t*>(c.links[F16G::id]), c.lstride,
-      static_cast<unsigned int*>(dev_max));
+      static_cast<unsigned long long*>(dev_max));
   c.launches++;
   TSM_TRY(check_launch(c, "pack_links_kernel"));
-  unsigned int bits = 0;
-  TSM_CUDA(cudaMemcpyAsync(&bits, dev_max, sizeof(bits), cudaMemcpyDeviceToHost, c.stream));
+  double dev2 = 0.0;
+  TSM_CUDA(cudaMemcpyAsync(&dev2, dev_max, sizeof(dev2), cudaMemcpyDeviceToHost, c.stream));
   TSM_CUDA(cudaStreamSynchronize(c.stream));
-  float dev;
-  std::memcpy(&dev, &bits, sizeof(dev));
-  if (!(dev <= 1e-8f)) {
-    set_error("gauge links are not SU(3): max deviation %g", (double)dev);
+  const double dev = std::sqrt(dev2);   // NaN stays NaN
+  if (!(dev <= 1e-8)) {
+    set_error("gauge links are not SU(3): max deviation %g", dev);
     return TSM_ERR_NOT_UNITARY;
   }
   c.has_gauge = true;
@@ -594,7 +586,10 @@ int tm_dslash(tsm_ctx* h, int prec, int op, int dagger, const double* in, double
   EOField fi, fo;
   TSM_TRY(eo_fields(c, "ds_in", prec, &fi));
   TSM_TRY(eo_fields(c, "ds_out", prec, &fo));
-  TSM_TRY(pack_eo(c, prec, din, fi));
+  // parities the operator reads and writes (the other output parity is zero)
+  const bool in_e = op != TM_OP_HOP_EO, in_o = op == TM_OP_FULL || op == TM_OP_HOP_EO;
+  const bool out_e = op != TM_OP_HOP_OE, out_o = op == TM_OP_FULL || op == TM_OP_HOP_OE;
+  TSM_TRY(pack_eo(c, prec, din, EOField{in_e ? fi.e : PField{}, in_o ? fi.o : PField{}}));
   c.prof_this_launch = c.profile;
   c.hop_per_site = true;   // one field: the per-site stencil (no link sharing to exploit)
   int rc = dispatch_prec(prec, [&](auto tag) {
@@ -604,7 +599,7 @@ int tm_dslash(tsm_ctx* h, int prec, int op, int dagger, const double* in, double
   c.hop_per_site = false;
   c.prof_this_launch = false;
   TSM_TRY(rc);
-  TSM_TRY(unpack_eo(c, prec, fo, dout));
+  TSM_TRY(unpack_eo(c, prec, EOField{out_e ? fo.e : PField{}, out_o ? fo.o : PField{}}, dout));
   TSM_TRY(stage_out_finish(c, out, dout, bytes, on_device));
   TSM_CUDA(cudaStreamSynchronize(c.stream));
   return c.harvest_events();
@@ -627,27 +622,35 @@ int tm_solve_batch(tsm_ctx* h, int nrhs, const double* b, double* s, const tm_st
   TSM_TRY(eo_fields(c, "sv_s", sp, &fs, c.batch_cap));
   int worst = TSM_OK;
   std::vector<SolveResult> res(width);
+  std::vector<double> tres(width);
   for (int r0 = 0; r0 < nrhs; r0 += width) {
     const int n = std::min(width, nrhs - r0);
-    for (int r = 0; r < n; ++r) {
+    const size_t at = (size_t)r0 * c.g.V * 24;
+    // canonical sources and solutions of the batch at once; host callers' are
+    // staged a few at a time (256 MB, at least one source)
+    const int step = on_device ? n : std::max(1, std::min(n, (int)(((size_t)256 << 20) / bytes)));
+    for (int r = 0; r < n; r += step) {
+      const int m = std::min(step, n - r);
+      const size_t o = at + (size_t)r * c.g.V * 24;
       const double* db = nullptr;
-      TSM_TRY(stage_in(c, "io_in", b + (size_t)(r0 + r) * c.g.V * 24, bytes, on_device, &db));
-      TSM_TRY(pack_eo(c, sp, db, eo_at(fb, sp, c.g.Vh, r)));
+      TSM_TRY(stage_in(c, "io_in", b + o, m * bytes, on_device, &db));
+      TSM_TRY(pack_eo(c, sp, db, eo_at(fb, sp, c.g.Vh, r), m));
     }
     TSM_TRY(solve_batch(c, *stop, 0, n, fb, fs, res.data()));
+    for (int r = 0; r < n; r += step) {
+      const int m = std::min(step, n - r);
+      const size_t o = at + (size_t)r * c.g.V * 24;
+      double* ds = nullptr;
+      TSM_TRY(stage_out_ptr(c, "io_out", s + o, m * bytes, on_device, &ds));
+      TSM_TRY(unpack_eo(c, sp, eo_at(fs, sp, c.g.Vh, r), ds, m));
+      TSM_TRY(stage_out_finish(c, s + o, ds, m * bytes, on_device));
+    }
+    if (true_res) TSM_TRY(true_residual(c, sp, fb, fs, n, tres.data()));
+    else TSM_CUDA(cudaStreamSynchronize(c.stream));
     for (int r = 0; r < n; ++r) {
       const SolveResult& q = res[r];
       if (iters) iters[r0 + r] = q.iters;
-      if (true_res) {
-        double tr = 0.0;
-        TSM_TRY(true_residual(c, sp, eo_at(fb, sp, c.g.Vh, r), eo_at(fs, sp, c.g.Vh, r), &tr));
-        true_res[r0 + r] = tr;
-      }
-      double* ds = nullptr;
-      TSM_TRY(stage_out_ptr(c, "io_out", s + (size_t)(r0 + r) * c.g.V * 24, bytes, on_device, &ds));
-      TSM_TRY(unpack_eo(c, sp, eo_at(fs, sp, c.g.Vh, r), ds));
-      TSM_TRY(stage_out_finish(c, s + (size_t)(r0 + r) * c.g.V * 24, ds, bytes, on_device));
-      TSM_CUDA(cudaStreamSynchronize(c.stream));
+      if (true_res) true_res[r0 + r] = tres[r];
       if (q.status != TSM_OK) worst = q.status;
       else if (!q.converged && worst == TSM_OK) worst = TSM_ERR_NOT_CONVERGED;
     }

@@ -169,9 +169,10 @@ inline Twist twist_mul(const Twist& a, const Twist& b) {
 // right-hand sides still iterating.
 template <class S> int launch_hop(Ctx& c, const HopArgs<S>& a, int dag, int mode, int prof_kind, int nrhs = 1);
 
-// the FP32 kernels' epilogue factors of a hop, formed in FP64 and rounded once
+// the epilogue factors of a hop, formed in FP64 (rounded once for the FP32 kernels)
 template <class S>
-void hop_factors(const HopArgs<S>& a, TwistF* to_ah, TwistF* to_tc_ac, TwistF* ts) {
+void hop_factors(HopArgs<S>* h) {
+  const HopArgs<S>& a = *h;
   Twist toah, totc;
   for (int q = 0; q < 2; ++q) {
     toah.re[q] = a.to.re[q] * a.ah;
@@ -179,15 +180,21 @@ void hop_factors(const HopArgs<S>& a, TwistF* to_ah, TwistF* to_tc_ac, TwistF* t
     totc.re[q] = (a.to.re[q] * a.tc.re[q] - a.to.im[q] * a.tc.im[q]) * a.ac;
     totc.im[q] = (a.to.re[q] * a.tc.im[q] + a.to.im[q] * a.tc.re[q]) * a.ac;
   }
-  *to_ah = to_float(toah);
-  *to_tc_ac = to_float(totc);
-  *ts = to_float(a.ts);
+  h->fto_ah = to_float(toah);
+  h->fto_tc_ac = to_float(totc);
+  h->fts = to_float(a.ts);
+  h->to_ah = toah;
+  h->to_tc_ac = totc;
+  h->real_ah = toah.im[0] == 0.0 && toah.im[1] == 0.0 && toah.re[0] == toah.re[1];
+  h->one_ts = a.ts.re[0] == 1.0 && a.ts.re[1] == 1.0 && a.ts.im[0] == 0.0 && a.ts.im[1] == 0.0;
 }
 template <class S, class SA> int launch_cg_update(Ctx& c, const CGUpdArgs<S, SA>& a, int nrhs);
 template <class S, class SA>
 int launch_cg_p(Ctx& c, const PField& r, const PField& p, CGState* st, const int* active, int nrhs);
-template <class S> int launch_pack(Ctx& c, int parity, const double* canon, const PField& out);
-template <class S> int launch_unpack(Ctx& c, int parity, const PField& in, double* canon);
+template <class S> int launch_full(Ctx& c, const HopArgs<S>& e, const HopArgs<S>& o, int dag);
+// canonical spinors <-> even / odd fields; an empty field is left out (pack) or zero (unpack)
+template <class S> int launch_pack(Ctx& c, const double* canon, const PField& even, const PField& odd, int nrhs = 1);
+template <class S> int launch_unpack(Ctx& c, const PField& even, const PField& odd, double* canon, int nrhs = 1);
 template <class S>
 int launch_noise(Ctx& c, int parity, const NoiseSpec& n, uint32_t source0, const PField& out, int nrhs = 1);
 template <class S>

@@ -301,16 +301,13 @@ template int launch_contract<float, F16, F16>(Ctx&, const ContractPlan&, const N
                                               const EOField*, double2*, const EOField*, const EOField*);
 
 int apply_wilson(Ctx& c, int prec, EOField in, EOField out) {
-  // one field: the one-thread-per-site stencil (link tiles pay only when
-  // several sources share them)
-  const bool per_site = c.hop_per_site;
-  c.hop_per_site = true;
-  const int rc = dispatch_prec(prec, [&](auto tag) -> int {
+  return dispatch_prec(prec, [&](auto tag) -> int {
     using S = decltype(tag);
     // both parities: links, neighbour field, centre field, output
     TimedLaunch tl(c, PB_WILSON, (double)c.g.V * (link_site_bytes(S::id) + 3.0 * spinor_site_bytes(S::id)), true);
+    HopArgs<S> hs[2]{};
     for (int par = 0; par < 2; ++par) {
-      HopArgs<S> h{};
+      HopArgs<S>& h = hs[par];
       h.g = c.g;
       h.p_out = par;
       h.Uout = c.links_of<S>(par);
@@ -327,13 +324,11 @@ int apply_wilson(Ctx& c, int prec, EOField in, EOField out) {
       h.ts = twist_one();
       h.red = c.red;
       h.post = POST_NONE;
-      TSM_TRY(launch_hop<S>(c, h, 0, HOP_CENTER, -1));
     }
+    TSM_TRY(launch_full<S>(c, hs[0], hs[1], 0));
     tl.done();
     return (int)TSM_OK;
   });
-  c.hop_per_site = per_site;
-  return rc;
 }
 
 int reserve_contract(Ctx& c) {

@@ -152,6 +152,39 @@ __device__ __forceinline__ void su3_mul(const cx<R> r[9], const cx<R> h[6], cx<R
   }
 }
 
+// u = u0 + U h or u0 + U^dag h: the products' chains start from u0
+template <bool DAGU, class R>
+__device__ __forceinline__ void su3_mul_add(const cx<R> r[9], const cx<R> h[6], const cx<R> u0[6], cx<R> u[6]) {
+#pragma unroll
+  for (int s = 0; s < 2; ++s)
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      cx<R> v = u0[3 * s + i];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const cx<R> m = DAGU ? cconj(r[3 * k + i]) : r[3 * i + k], x = h[3 * s + k];
+        v.re = fma(m.re, x.re, v.re);
+        v.im = fma(m.re, x.im, v.im);
+        v.re = fma(-m.im, x.im, v.re);
+        v.im = fma(m.im, x.re, v.im);
+      }
+      u[3 * s + i] = v;
+    }
+}
+
+// the upper components of a direction's two hops, sum, and the lower ones, the
+// reconstruction (spin matrix of (1 + SG gamma_MU)) of diff
+template <int MU, int SG, bool FIRST, class R>
+__device__ __forceinline__ void accumulate_pair(cx<R> acc[12], const cx<R> sum[6], const cx<R> diff[6]) {
+  cx<R> low[12];
+  accumulate<MU, SG, true>(low, diff);
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    acc[k] = FIRST ? sum[k] : acc[k] + sum[k];
+    acc[6 + k] = FIRST ? low[6 + k] : acc[6 + k] + low[6 + k];
+  }
+}
+
 // One direction of the stencil at output site (c, ih) of parity p.
 // links(h, nb, r) fills r[0..8] with the three rows of the link of hop h
 // (2 MU forward at x, 2 MU + 1 backward at x - mu, neighbour index nb).
@@ -161,6 +194,11 @@ __device__ __forceinline__ void hop_dir(const Geom& g, const int c[4], const typ
   using R = typename S::real;
   constexpr int SF = DAG ? +1 : -1;   // forward hop: (1 + SF gamma_mu)
   constexpr int SB = -SF;             // backward hop
+  // FP64, bound by its pipe: the backward product's chains start from the
+  // forward product u_f, whose upper components then need one addition for both
+  // hops, and the lower ones (opposite projector signs) get u_f - u_b = 2 u_f -
+  // sum with one multiply-add: 204 instead of 216 FP64 instructions per direction
+  constexpr bool PAIR = sizeof(R) == 8;
   cx<R> h[6], u[6], r[9];
   // forward neighbour x + mu
   {
@@ -179,7 +217,7 @@ __device__ __forceinline__ void hop_dir(const Geom& g, const int c[4], const typ
     }
     links(2 * MU, -1, r);
     su3_mul<false>(r, h, u);
-    accumulate<MU, SF, MU == 0>(acc, u);   // the site's first hop assigns
+    if constexpr (!PAIR) accumulate<MU, SF, MU == 0>(acc, u);   // the site's first hop assigns
   }
   // backward neighbour x - mu
   {
@@ -197,8 +235,17 @@ __device__ __forceinline__ void hop_dir(const Geom& g, const int c[4], const typ
       }
     }
     links(2 * MU + 1, nb, r);
-    su3_mul<true>(r, h, u);
-    accumulate<MU, SB, false>(acc, u);
+    if constexpr (PAIR) {
+      cx<R> sum[6];
+      su3_mul_add<true>(r, h, u, sum);          // u_f + u_b
+#pragma unroll
+      for (int k = 0; k < 6; ++k)               // u_f - u_b
+        u[k] = {fma((R)2, u[k].re, -sum[k].re), fma((R)2, u[k].im, -sum[k].im)};
+      accumulate_pair<MU, SF, MU == 0>(acc, sum, u);
+    } else {
+      su3_mul<true>(r, h, u);
+      accumulate<MU, SB, false>(acc, u);
+    }
   }
 }
 
@@ -264,7 +311,9 @@ struct HopArgs {
   RedSlot red;                             // HOP_NORM
   int post;                                // PostOp for HOP_NORM
   TwistF fto_ah, fto_tc_ac, fts;           // FP32 kernels: to * ah, to * tc * ac and ts, formed in
-                                           // FP64 on the host and rounded once (set by launch_hop)
+                                           // FP64 on the host and rounded once (set by hop_factors)
+  Twist to_ah, to_tc_ac;                   // FP64 kernels: the products themselves
+  int real_ah, one_ts;                     // to_ah is one real number, ts is 1
 };
 
 constexpr int HOP_NT = 128;
@@ -295,18 +344,22 @@ __device__ __forceinline__ typename S::real hop_epilogue(const HopArgs<S>& a, si
       for (int k = 0; k < 12; ++k) acc[k] = acc[k] + v[k];
     }
   } else {
-    const R ah = (R)a.ah;
+    // FP64: the same combined factors; real ones cost half (a uniform branch)
+    if (a.real_ah) {
 #pragma unroll
-    for (int k = 0; k < 12; ++k) acc[k] = ah * acc[k];
+      for (int k = 0; k < 12; ++k) acc[k] = (R)a.to_ah.re[0] * acc[k];
+    } else {
+      apply_twist(a.to_ah, acc);
+    }
     if constexpr (MODE & HOP_CENTER) {
       cx<R> v[12];
       load_spinor<S>(a.center + off, a.sstride, ih, v);
-      apply_twist(a.tc, v);
-      const R ac = (R)a.ac;
 #pragma unroll
-      for (int k = 0; k < 12; ++k) acc[k] = acc[k] + ac * v[k];
+      for (int k = 0; k < 12; ++k) {
+        const R fr = (R)a.to_tc_ac.re[k / 6], fi = (R)a.to_tc_ac.im[k / 6];
+        acc[k] = {fma(-fi, v[k].im, fma(fr, v[k].re, acc[k].re)), fma(fi, v[k].re, fma(fr, v[k].im, acc[k].im))};
+      }
     }
-    apply_twist(a.to, acc);
   }
   if constexpr (MODE & HOP_BASE) {
     cx<R> v[12];
@@ -321,7 +374,7 @@ __device__ __forceinline__ typename S::real hop_epilogue(const HopArgs<S>& a, si
     part = s;
   }
   if constexpr (FP32) apply_twist(a.fts, acc);
-  else apply_twist(a.ts, acc);
+  else if (!a.one_ts) apply_twist(a.ts, acc);
   store_spinor<S>(a.out + off, a.sstride, ih, acc);
   return part;
 }
@@ -346,6 +399,154 @@ __global__ void __launch_bounds__(HOP_NT, HopMinBlocks<S>::value) hop_kernel(con
     if (grid_sum<HOP_NT>(part, a.red, rhs, &total) && threadIdx.x == 0 && a.st != nullptr)
       post_action(a.st + rhs, a.post, total);
   }
+}
+
+// both parities of the hop with a centre field (blockIdx.z = output parity), one field
+template <class S, int DAG>
+__global__ void __launch_bounds__(HOP_NT, HopMinBlocks<S>::value)
+    full_hop_kernel(const __grid_constant__ HopArgs<S> e, const __grid_constant__ HopArgs<S> o) {
+  const HopArgs<S>& a = blockIdx.z ? o : e;
+  const int ih = blockIdx.y * HOP_NT + threadIdx.x;
+  if (ih >= a.g.Vh) return;
+  int c[4];
+  site_coords(a.g, a.p_out, ih, c);
+  cx<typename S::real> acc[12];
+  hop_site<S, DAG>(a.g, ih, c, a.Uout, a.Uin, a.lstride, a.in, a.sstride, acc);
+  hop_epilogue<S, HOP_CENTER>(a, 0, ih, acc);
+}
+
+// The same in FP64 for a small lattice: four threads per site, one direction
+// each (a warp per direction, so that no warp diverges), then warp s joins the
+// four sums of spin s in shared memory.  A warp-wide FP64 instruction occupies
+// its scheduler for about 70 cycles on GB300, so below one warp per scheduler
+// (152 x 4 warps of 32 sites) a thread per site takes the time of its ~1000
+// FP64 instructions, 37 us, however small the lattice; a thread of four issues
+// about 240.
+constexpr int SPLIT_SITES = 152 * 4 * 32;
+
+template <int DAG>
+__global__ void __launch_bounds__(128)
+    split_hop_kernel(const __grid_constant__ HopArgs<F64> e, const __grid_constant__ HopArgs<F64> o) {
+  __shared__ double2 sh[4][12][32];
+  const HopArgs<F64>& a = blockIdx.z ? o : e;
+  const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int ih = blockIdx.x * 32 + lane;
+  if (ih < a.g.Vh) {
+    int c[4];
+    site_coords(a.g, a.p_out, ih, c);
+    cx<double> acc[12];
+#pragma unroll
+    for (int k = 0; k < 12; ++k) acc[k] = {0.0, 0.0};
+    const GlobalLinks<F64> links{a.Uout, a.Uin, a.lstride, ih};
+    if (q == 0) hop_dir<F64, DAG, 0>(a.g, c, a.in, a.sstride, links, acc);
+    else if (q == 1) hop_dir<F64, DAG, 1>(a.g, c, a.in, a.sstride, links, acc);
+    else if (q == 2) hop_dir<F64, DAG, 2>(a.g, c, a.in, a.sstride, links, acc);
+    else hop_dir<F64, DAG, 3>(a.g, c, a.in, a.sstride, links, acc);
+#pragma unroll
+    for (int k = 0; k < 12; ++k) sh[q][k][lane] = make_double2(acc[k].re, acc[k].im);
+  }
+  __syncthreads();
+  if (ih >= a.g.Vh) return;
+  const int half = q >> 1;   // chirality of spin q
+  const cx<double> ah = {a.to_ah.re[half], a.to_ah.im[half]}, cc = {a.to_tc_ac.re[half], a.to_tc_ac.im[half]};
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    cx<double> v = {0.0, 0.0};
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu) {
+      const double2 s = sh[mu][3 * q + k][lane];
+      v = mu == 0 ? cx<double>{s.x, s.y} : v + cx<double>{s.x, s.y};
+    }
+    const size_t at = (size_t)(3 * q + k) * a.sstride + ih;
+    const double2 ce = a.center[at];
+    const cx<double> w = ah * v + cc * cx<double>{ce.x, ce.y};
+    a.out[at] = make_double2(w.re, w.im);
+  }
+}
+
+// Squared norms of b - D_tm s and of b for a batch of sources, in FP64 from
+// fields of storage S (FP32 or FP64): one pass over both parities
+// (blockIdx.z), no widened copies, no stored residual.  Bound by the FP64 pipe:
+// 912 FP64 instructions per site (the hop kernel with its epilogue, the norm
+// kernel and the conversions took about 1150), the widening of FP32 components
+// is integer work beside them.  Partials: [2 parity + {residual, source}]
+// [source][block], added by residual_sum_kernel.
+struct ResidualArgs {
+  Geom g;
+  const double2* U[2];     // FP64 links of each parity
+  int lstride, sstride;
+  const void* b[2];
+  const void* s[2];
+  double kappa, two_km;    // D = 1 + i two_km gamma_5 - kappa H
+  double* partials;
+  int stride;              // blocks per parity and source
+  int nrhs;
+};
+
+// FP32 fields read as FP64
+struct F32as64 {
+  using real = double;
+  using schunk = float4;
+  static constexpr int SN = 6;
+  static constexpr int id = 5;   // internal
+};
+template <class S> struct Widened { using type = S; };
+template <> struct Widened<F32> { using type = F32as64; };
+
+template <class S>
+__global__ void __launch_bounds__(HOP_NT, 1) residual_kernel(const __grid_constant__ ResidualArgs a) {
+  using W = typename Widened<S>::type;
+  using C = typename W::schunk;
+  const int par = blockIdx.z, rhs = blockIdx.x;
+  const int ih = blockIdx.y * HOP_NT + threadIdx.x;
+  const size_t off = (size_t)rhs * W::SN * (size_t)a.sstride;
+  double nr = 0.0, nb = 0.0;
+  if (ih < a.g.Vh) {
+    int c[4];
+    site_coords(a.g, par, ih, c);
+    cx<double> acc[12], v[12];
+    hop_site_with<W, 0>(a.g, c, static_cast<const C*>(a.s[1 - par]) + off, a.sstride,
+                        GlobalLinks<F64>{a.U[par], a.U[1 - par], a.lstride, ih}, acc);
+    load_spinor<W>(static_cast<const C*>(a.s[par]) + off, a.sstride, ih, v);
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {   // kappa H s - (1 + i m gamma_5) s
+      const double m = k < 6 ? a.two_km : -a.two_km;
+      acc[k] = {fma(m, v[k].im, fma(a.kappa, acc[k].re, -v[k].re)), fma(-m, v[k].re, fma(a.kappa, acc[k].im, -v[k].im))};
+    }
+    load_spinor<W>(static_cast<const C*>(a.b[par]) + off, a.sstride, ih, v);
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+      const double re = acc[k].re + v[k].re, im = acc[k].im + v[k].im;
+      nr = fma(re, re, fma(im, im, nr));
+      nb = fma(v[k].re, v[k].re, fma(v[k].im, v[k].im, nb));
+    }
+  }
+  __shared__ double sh[HOP_NT / 32];
+  const double tr = block_sum<HOP_NT>(nr, sh);
+  const double tb = block_sum<HOP_NT>(nb, sh);
+  if (threadIdx.x == 0) {
+    double* p = a.partials + (size_t)rhs * a.stride + blockIdx.y;
+    const size_t plane = (size_t)a.nrhs * a.stride;
+    p[2 * par * plane] = tr;
+    p[(2 * par + 1) * plane] = tb;
+  }
+}
+
+// out[rhs] = {|b - D s|^2, |b|^2}: the partials of both parities in block order
+static __global__ void __launch_bounds__(256) residual_sum_kernel(const double* __restrict__ partials, int stride,
+                                                                  int nrhs, double2* __restrict__ out) {
+  __shared__ double sh[8];
+  const int rhs = blockIdx.x;
+  const size_t plane = (size_t)nrhs * stride;
+  double v[2];
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    double s = 0.0;
+    for (int par = 0; par < 2; ++par)
+      s += strided_sum_ordered(partials + (2 * par + q) * plane + (size_t)rhs * stride, threadIdx.x, stride, 256);
+    v[q] = block_sum<256>(s, sh);
+  }
+  if (threadIdx.x == 0) out[rhs] = make_double2(v[0], v[1]);
 }
 
 // ------------------------------------------------------------- fused CG update

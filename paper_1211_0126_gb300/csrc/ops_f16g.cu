@@ -81,14 +81,14 @@ int mma_launch(Ctx& c, const MmaHopArgs& m, const MmaMaps& maps, dim3 grid) {
   return check_launch(c, "mma_hop_kernel");
 }
 
-bool is_one(const Twist& t) { return t.re[0] == 1.0 && t.re[1] == 1.0 && t.im[0] == 0.0 && t.im[1] == 0.0; }
-
 }  // namespace
 
 template <>
-int launch_hop<F16G>(Ctx& c, const HopArgs<F16G>& a, int dag, int mode, int prof_kind, int nrhs) {
-  if (a.g.Vh == 0 || nrhs == 0) return TSM_OK;
-  if ((!(mode & HOP_NORM) && !is_one(a.ts)) || a.skip_rel || a.base != nullptr) {
+int launch_hop<F16G>(Ctx& c, const HopArgs<F16G>& a0, int dag, int mode, int prof_kind, int nrhs) {
+  if (a0.g.Vh == 0 || nrhs == 0) return TSM_OK;
+  HopArgs<F16G> a = a0;
+  hop_factors(&a);
+  if ((!(mode & HOP_NORM) && !a.one_ts) || a.skip_rel || a.base != nullptr) {
     set_error("grouped FP16 hop: epilogue not built (dag %d, mode %d)", dag, mode);
     return TSM_ERR_ARG;
   }
@@ -99,7 +99,9 @@ int launch_hop<F16G>(Ctx& c, const HopArgs<F16G>& a, int dag, int mode, int prof
   MmaMaps maps;
   TSM_TRY(in_maps(c, &maps, a.in));
   if (mode & HOP_CENTER) TSM_TRY(make_map(c, &maps.f[0], a.center, kMmaBox[MMA_BOX_TILE]));
-  hop_factors(a, &m.fto_ah, &m.fto_tc_ac, &m.fts);
+  m.fto_ah = a.fto_ah;
+  m.fto_tc_ac = a.fto_tc_ac;
+  m.fts = a.fts;
   m.active = a.active;
   m.nrhs = nrhs;
   m.skip = a.skip;

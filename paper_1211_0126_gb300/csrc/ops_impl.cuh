@@ -22,7 +22,7 @@ int launch_hop(Ctx& c, const HopArgs<S>& a0, int dag, int mode, int prof_kind, i
   const int nb = blocks_for(a0.g.Vh, HOP_NT);
   if (nb == 0 || nrhs == 0) return TSM_OK;
   HopArgs<S> a = a0;
-  hop_factors(a0, &a.fto_ah, &a.fto_tc_ac, &a.fts);
+  hop_factors(&a);
   const int kind = prof_kind >= 0 ? prof_kind : hop_kind_of<S>(dag, mode);
   const double sb = spinor_site_bytes(S::id), lb = link_site_bytes(S::id);
   // links once per launch (shared by the right-hand sides), spinor streams per RHS
@@ -80,6 +80,31 @@ int launch_hop(Ctx& c, const HopArgs<S>& a0, int dag, int mode, int prof_kind, i
   return check_launch(c, "hop_kernel");
 }
 
+// both parities of a hop with a centre field, one field (e.p_out = 0, o.p_out
+// = 1): one launch, so that a small lattice's two halves run side by side
+template <class S>
+int launch_full(Ctx& c, const HopArgs<S>& e0, const HopArgs<S>& o0, int dag) {
+  HopArgs<S> e = e0, o = o0;
+  hop_factors(&e);
+  hop_factors(&o);
+  const double sb = spinor_site_bytes(S::id), lb = link_site_bytes(S::id);
+  TimedLaunch tl(c, 4 * S::id + (dag ? PK_HOP_DAG : PK_HOP_XPAY), 2.0 * c.g.Vh * (lb + 3.0 * sb));
+  if (S::id == F64::id && 2 * c.g.Vh < SPLIT_SITES) {
+    const dim3 grid(blocks_for(c.g.Vh, 32), 1, 2);
+    if constexpr (S::id == F64::id) {
+      if (dag) split_hop_kernel<1><<<grid, 128, 0, c.stream>>>(e, o);
+      else split_hop_kernel<0><<<grid, 128, 0, c.stream>>>(e, o);
+    }
+  } else {
+    const dim3 grid(1, blocks_for(c.g.Vh, HOP_NT), 2);
+    if (dag) full_hop_kernel<S, 1><<<grid, HOP_NT, 0, c.stream>>>(e, o);
+    else full_hop_kernel<S, 0><<<grid, HOP_NT, 0, c.stream>>>(e, o);
+  }
+  tl.done();
+  c.launches++;
+  return check_launch(c, "full_hop_kernel");
+}
+
 template <class S, class SA>
 int launch_cg_update(Ctx& c, const CGUpdArgs<S, SA>& a0, int nrhs) {
   const int nb = blocks_for(a0.g.Vh, HOP_NT);
@@ -107,19 +132,19 @@ int launch_cg_p(Ctx& c, const PField& r, const PField& p, CGState* st, const int
 }
 
 template <class S>
-int launch_pack(Ctx& c, int parity, const double* canon, const PField& out) {
-  const int nb = blocks_for(c.g.Vh, SITE_NT);
-  pack_spinor_kernel<S><<<nb, SITE_NT, 0, c.stream>>>(c.g, parity, reinterpret_cast<const double2*>(canon),
-                                                      out.as<S>(), c.sstride);
+int launch_pack(Ctx& c, const double* canon, const PField& even, const PField& odd, int nrhs) {
+  if (nrhs == 0) return TSM_OK;
+  pack_spinor_kernel<S><<<dim3(blocks_for(c.g.V, CANON_SITES), nrhs), SITE_NT, 0, c.stream>>>(
+      c.g, reinterpret_cast<const double2*>(canon), even.as<S>(), odd.as<S>(), c.sstride);
   c.launches++;
   return check_launch(c, "pack_spinor_kernel");
 }
 
 template <class S>
-int launch_unpack(Ctx& c, int parity, const PField& in, double* canon) {
-  const int nb = blocks_for(c.g.Vh, SITE_NT);
-  unpack_spinor_kernel<S><<<nb, SITE_NT, 0, c.stream>>>(c.g, parity, in.as<S>(), c.sstride,
-                                                        reinterpret_cast<double2*>(canon));
+int launch_unpack(Ctx& c, const PField& even, const PField& odd, double* canon, int nrhs) {
+  if (nrhs == 0) return TSM_OK;
+  unpack_spinor_kernel<S><<<dim3(blocks_for(c.g.V, CANON_SITES), nrhs), SITE_NT, 0, c.stream>>>(
+      c.g, even.as<S>(), odd.as<S>(), c.sstride, reinterpret_cast<double2*>(canon));
   c.launches++;
   return check_launch(c, "unpack_spinor_kernel");
 }
@@ -166,8 +191,9 @@ int launch_convert(Ctx& c, const PField& in, const PField& out, const int* activ
 
 #define TSM_INSTANTIATE_STORAGE(S)                                                                    \
   template int tsm::launch_hop<S>(Ctx&, const HopArgs<S>&, int, int, int, int);                      \
-  template int tsm::launch_pack<S>(Ctx&, int, const double*, const PField&);                         \
-  template int tsm::launch_unpack<S>(Ctx&, int, const PField&, double*);                             \
+  template int tsm::launch_pack<S>(Ctx&, const double*, const PField&, const PField&, int);          \
+  template int tsm::launch_unpack<S>(Ctx&, const PField&, const PField&, double*, int);              \
+  template int tsm::launch_full<S>(Ctx&, const HopArgs<S>&, const HopArgs<S>&, int);                 \
   template int tsm::launch_noise<S>(Ctx&, int, const NoiseSpec&, uint32_t, const PField&, int);      \
   template int tsm::launch_twist<S>(Ctx&, const Twist&, const PField&, const PField&, const CGState*, \
                                     const int*, int);                                                \

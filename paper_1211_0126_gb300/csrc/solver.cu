@@ -532,44 +532,42 @@ int solve_batch(Ctx& c, const tm_stop& stop, int s0, int nrhs, EOField b, EOFiel
   }
 }
 
-int true_residual(Ctx& c, int prec, EOField b, EOField s, double* out) {
-  const double k = c.lat.kappa, mu = c.lat.mu;
-  EOField b64 = b, s64 = s;
-  if (prec != TSM_F64) {
-    TSM_TRY(c.field("tr_be", TSM_F64, &b64.e));
-    TSM_TRY(c.field("tr_bo", TSM_F64, &b64.o));
-    TSM_TRY(c.field("tr_se", TSM_F64, &s64.e));
-    TSM_TRY(c.field("tr_so", TSM_F64, &s64.o));
-    TSM_TRY((launch_convert<F32, F64>(c, b.e, b64.e)));
-    TSM_TRY((launch_convert<F32, F64>(c, b.o, b64.o)));
-    TSM_TRY((launch_convert<F32, F64>(c, s.e, s64.e)));
-    TSM_TRY((launch_convert<F32, F64>(c, s.o, s64.o)));
+int true_residual(Ctx& c, int prec, EOField b, EOField s, int nrhs, double* out) {
+  if (prec != TSM_F64 && prec != TSM_F32) {
+    set_error("true residual of fields of tier %d (FP64 or FP32 expected)", prec);
+    return TSM_ERR_ARG;
   }
-  PField tmp;
-  TSM_TRY(c.field("tr_tmp", TSM_F64, &tmp));
-  CGState* aux = c.states + (Ctx::kMaxStates - 4);
+  if (nrhs < 1) return TSM_OK;
+  const int blocks = (c.g.Vh + HOP_NT - 1) / HOP_NT;
+  void *part = nullptr, *sums = nullptr;
+  TSM_TRY(c.buffer("tr_partial", (size_t)4 * nrhs * blocks * sizeof(double), &part));
+  TSM_TRY(c.buffer("tr_sums", (size_t)nrhs * sizeof(double2), &sums));
+  ResidualArgs a{};
+  a.g = c.g;
+  a.lstride = c.lstride;
+  a.sstride = c.sstride;
   for (int par = 0; par < 2; ++par) {
-    // r_p = b_p - (A s_p - kappa H s_{1-p})
-    HopArgs<F64> h = hop_args<F64>(c, par);
-    h.in = (par ? s64.e : s64.o).as<F64>();
-    h.center = (par ? s64.o : s64.e).as<F64>();
-    h.tc = twist_A(k, mu);
-    h.ac = 1.0;
-    h.ah = -k;
-    h.to = twist_scale(-1.0);
-    h.base = (par ? b64.o : b64.e).as<F64>();
-    h.out = tmp.as<F64>();
-    h.st = aux + par;
-    h.post = POST_NONE;
-    TSM_TRY(launch_hop<F64>(c, h, 0, HOP_CENTER | HOP_NORM | HOP_BASE, -1));
-    TSM_TRY(launch_norm<F64>(c, par ? b64.o : b64.e, aux + 2 + par, POST_NONE));
+    a.U[par] = c.links_of<F64>(par);
+    a.b[par] = (par ? b.o : b.e).p;
+    a.s[par] = (par ? s.o : s.e).p;
   }
-  TSM_CUDA(cudaMemcpyAsync(c.h_states + (Ctx::kMaxStates - 4), aux, 4 * sizeof(CGState), cudaMemcpyDeviceToHost,
-                           c.stream));
+  a.kappa = c.lat.kappa;
+  a.two_km = 2.0 * c.lat.kappa * c.lat.mu;
+  a.partials = static_cast<double*>(part);
+  a.stride = blocks;
+  a.nrhs = nrhs;
+  const dim3 grid(nrhs, blocks, 2);
+  if (prec == TSM_F64) residual_kernel<F64><<<grid, HOP_NT, 0, c.stream>>>(a);
+  else residual_kernel<F32><<<grid, HOP_NT, 0, c.stream>>>(a);
+  c.launches++;
+  TSM_TRY(check_launch(c, "residual_kernel"));
+  residual_sum_kernel<<<nrhs, 256, 0, c.stream>>>(a.partials, blocks, nrhs, static_cast<double2*>(sums));
+  c.launches++;
+  TSM_TRY(check_launch(c, "residual_sum_kernel"));
+  std::vector<double2> h(nrhs);
+  TSM_CUDA(cudaMemcpyAsync(h.data(), sums, (size_t)nrhs * sizeof(double2), cudaMemcpyDeviceToHost, c.stream));
   TSM_CUDA(cudaStreamSynchronize(c.stream));
-  const CGState* hs = c.h_states + (Ctx::kMaxStates - 4);
-  const double nr = hs[0].aux + hs[1].aux, nb = hs[2].aux + hs[3].aux;
-  *out = nb > 0 ? std::sqrt(nr / nb) : std::sqrt(nr);
+  for (int r = 0; r < nrhs; ++r) out[r] = h[r].y > 0 ? std::sqrt(h[r].x / h[r].y) : std::sqrt(h[r].x);
   return TSM_OK;
 }
 

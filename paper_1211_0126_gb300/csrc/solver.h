@@ -42,8 +42,9 @@ int solve_batch(Ctx& c, const tm_stop& stop, int s0, int nrhs, EOField b, EOFiel
 // (source / solution storage sol_prec as in solve_batch).
 int reserve_solver(Ctx& c, const tm_stop& stop, int sol_prec = -1);
 
-// ||b - D_tm s|| / ||b|| in FP64 (fields of tier prec).
-int true_residual(Ctx& c, int prec, EOField b, EOField s, double* out);
+// ||b - D_tm s|| / ||b|| in FP64 of nrhs sources (batches of fields of tier
+// prec, FP32 or FP64).  Waits for the stream.
+int true_residual(Ctx& c, int prec, EOField b, EOField s, int nrhs, double* out);
 
 // hop arguments pre-filled for this context (links of storage S, unit twists)
 template <class S>
