@@ -32,6 +32,14 @@ template <class R> __device__ __forceinline__ cx<R> cconj(cx<R> a) { return {a.r
 template <class R> __device__ __forceinline__ cx<R> cjmul(cx<R> a, cx<R> b) {
   return {a.re * b.re + a.im * b.im, a.re * b.im - a.im * b.re};
 }
+// acc + a b and acc + conj(a) b as chains of four multiply-adds (acc + a * b
+// compiles to six instructions: the sum of the two products comes first)
+template <class R> __device__ __forceinline__ cx<R> cmac(cx<R> acc, cx<R> a, cx<R> b) {
+  return {fma(-a.im, b.im, fma(a.re, b.re, acc.re)), fma(a.im, b.re, fma(a.re, b.im, acc.im))};
+}
+template <class R> __device__ __forceinline__ cx<R> cjmac(cx<R> acc, cx<R> a, cx<R> b) {
+  return {fma(a.im, b.im, fma(a.re, b.re, acc.re)), fma(-a.im, b.re, fma(a.re, b.im, acc.im))};
+}
 template <class R> __device__ __forceinline__ cx<R> times_i(cx<R> a) { return {-a.im, a.re}; }
 template <class R> __device__ __forceinline__ R norm2(cx<R> a) { return a.re * a.re + a.im * a.im; }
 
@@ -426,6 +434,10 @@ struct CGState {
   int need_rel;     // 1: a reliable update is due before the next iteration
   int final_check;  // 1: the iterated residual met the rule; the update decides
 };
+
+// a source the CG kernels leave alone: it met its rule, or it waits for its
+// reliable update
+__device__ __forceinline__ bool cg_idle(const CGState& s) { return s.done | s.need_rel; }
 
 enum PostOp {
   POST_NONE = 0,    // write the sum to st->aux

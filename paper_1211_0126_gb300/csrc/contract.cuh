@@ -315,7 +315,7 @@ __global__ void __launch_bounds__(ContractNT<R>::value) contract_kernel(const Co
           cx<R> acc = {0, 0};
 #pragma unroll
           for (int cc = 0; cc < 3; ++cc)
-            acc = acc + cjmul(cx<R>{(R)va[3 * x + cc].re, (R)va[3 * x + cc].im},
+            acc = cjmac(acc, cx<R>{(R)va[3 * x + cc].re, (R)va[3 * x + cc].im},
                               cx<R>{(R)wa[3 * y + cc].re, (R)wa[3 * y + cc].im});
           S[x][y] = acc;
         }
@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(ContractNT<R>::value) contract_kernel(const Co
             cx<R> acc = {0, 0};
 #pragma unroll
             for (int cc = 0; cc < 3; ++cc)
-              acc = acc + cjmul(cx<R>{(R)vb[3 * x + cc].re, (R)vb[3 * x + cc].im},
+              acc = cjmac(acc, cx<R>{(R)vb[3 * x + cc].re, (R)vb[3 * x + cc].im},
                                 cx<R>{(R)wb[3 * y + cc].re, (R)wb[3 * y + cc].im});
             S[x][y] = S[x][y] - acc;
           }
@@ -367,8 +367,8 @@ __global__ void __launch_bounds__(ContractNT<R>::value) contract_kernel(const Co
 #pragma unroll
         for (int y = 0; y < 4; ++y) {
           cx<R> acc = cjmul(eta[3 * x], s[3 * y]);
-          acc = acc + cjmul(eta[3 * x + 1], s[3 * y + 1]);
-          acc = acc + cjmul(eta[3 * x + 2], s[3 * y + 2]);
+          acc = cjmac(acc, eta[3 * x + 1], s[3 * y + 1]);
+          acc = cjmac(acc, eta[3 * x + 2], s[3 * y + 2]);
           S[x][y] = acc;
         }
     } else {
@@ -396,7 +396,7 @@ __global__ void __launch_bounds__(ContractNT<R>::value) contract_kernel(const Co
             cx<R> acc = {0, 0};
 #pragma unroll
             for (int cc = 0; cc < 3; ++cc)
-              acc = acc + cjmul(d[3 * x + cc], sa[3 * y + cc]) + cjmul(sb[3 * x + cc], d[3 * y + cc]);
+              acc = cjmac(cjmac(acc, d[3 * x + cc], sa[3 * y + cc]), sb[3 * x + cc], d[3 * y + cc]);
             S[x][y] = acc;
           }
       } else {
@@ -405,8 +405,8 @@ __global__ void __launch_bounds__(ContractNT<R>::value) contract_kernel(const Co
 #pragma unroll
           for (int y = 0; y < 4; ++y) {
             cx<R> acc = cjmul(sa[3 * x], sa[3 * y]);
-            acc = acc + cjmul(sa[3 * x + 1], sa[3 * y + 1]);
-            acc = acc + cjmul(sa[3 * x + 2], sa[3 * y + 2]);
+            acc = cjmac(acc, sa[3 * x + 1], sa[3 * y + 1]);
+            acc = cjmac(acc, sa[3 * x + 2], sa[3 * y + 2]);
             S[x][y] = acc;
           }
       }
@@ -466,7 +466,7 @@ __device__ __forceinline__ void colour_mul(const cx<R> u[9], const cx<R> f[12], 
     for (int a = 0; a < 3; ++a) {
       cx<R> acc = {0, 0};
 #pragma unroll
-      for (int b = 0; b < 3; ++b) acc = acc + (DAGU ? cjmul(u[3 * b + a], f[3 * sp + b]) : u[3 * a + b] * f[3 * sp + b]);
+      for (int b = 0; b < 3; ++b) acc = DAGU ? cjmac(acc, u[3 * b + a], f[3 * sp + b]) : cmac(acc, u[3 * a + b], f[3 * sp + b]);
       out[3 * sp + a] = sign * acc;
     }
 }
@@ -536,7 +536,7 @@ __global__ void __launch_bounds__(ContractNT<R>::value) deriv_contract_kernel(co
         cx<R> acc = {0, 0};
 #pragma unroll
         for (int cc = 0; cc < 3; ++cc)
-          acc = acc + cjmul(eta[3 * x + cc], ds[3 * y + cc]) - cjmul(de[3 * x + cc], s[3 * y + cc]);
+          acc = cjmac(cjmac(acc, eta[3 * x + cc], ds[3 * y + cc]), cx<R>{-de[3 * x + cc].re, -de[3 * x + cc].im}, s[3 * y + cc]);
         S[x][y] = (R)0.25 * acc;
       }
   }

@@ -136,18 +136,13 @@ __device__ __forceinline__ void accumulate(cx<R> acc[12], const cx<R> u[6]) {
 // r holds the three rows of U (r[6..8] = row 2)
 template <bool DAGU, class R>
 __device__ __forceinline__ void su3_mul(const cx<R> r[9], const cx<R> h[6], cx<R> u[6]) {
-  const cx<R>* w = r + 6;
 #pragma unroll
   for (int s = 0; s < 2; ++s) {
     const cx<R> a = h[3 * s], b = h[3 * s + 1], c = h[3 * s + 2];
-    if constexpr (!DAGU) {
-      u[3 * s + 0] = r[0] * a + r[1] * b + r[2] * c;
-      u[3 * s + 1] = r[3] * a + r[4] * b + r[5] * c;
-      u[3 * s + 2] = w[0] * a + w[1] * b + w[2] * c;
-    } else {
-      u[3 * s + 0] = cjmul(r[0], a) + cjmul(r[3], b) + cjmul(w[0], c);
-      u[3 * s + 1] = cjmul(r[1], a) + cjmul(r[4], b) + cjmul(w[1], c);
-      u[3 * s + 2] = cjmul(r[2], a) + cjmul(r[5], b) + cjmul(w[2], c);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      if constexpr (!DAGU) u[3 * s + i] = cmac(cmac(r[3 * i] * a, r[3 * i + 1], b), r[3 * i + 2], c);
+      else u[3 * s + i] = cjmac(cjmac(cjmul(r[i], a), r[3 + i], b), r[6 + i], c);
     }
   }
 }
@@ -161,13 +156,8 @@ __device__ __forceinline__ void su3_mul_add(const cx<R> r[9], const cx<R> h[6], 
     for (int i = 0; i < 3; ++i) {
       cx<R> v = u0[3 * s + i];
 #pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        const cx<R> m = DAGU ? cconj(r[3 * k + i]) : r[3 * i + k], x = h[3 * s + k];
-        v.re = fma(m.re, x.re, v.re);
-        v.im = fma(m.re, x.im, v.im);
-        v.re = fma(-m.im, x.im, v.re);
-        v.im = fma(m.im, x.re, v.im);
-      }
+      for (int k = 0; k < 3; ++k)
+        v = DAGU ? cjmac(v, r[3 * k + i], h[3 * s + k]) : cmac(v, r[3 * i + k], h[3 * s + k]);
       u[3 * s + i] = v;
     }
 }
@@ -305,7 +295,7 @@ struct HopArgs {
   double ac, ah;
   Twist tc, to, ts;
   const int* active;                       // optional list of right-hand sides
-  const CGState* skip;                     // optional: a RHS returns at once when skip[rhs].done
+  const CGState* skip;                     // optional: a RHS returns at once when cg_idle(skip[rhs])
   int skip_rel;                            // 1: instead, return unless skip[rhs].need_rel
   CGState* st;                             // states receiving the HOP_NORM post action
   RedSlot red;                             // HOP_NORM
@@ -383,7 +373,7 @@ template <class S, int DAG, int MODE>
 __global__ void __launch_bounds__(HOP_NT, HopMinBlocks<S>::value) hop_kernel(const HopArgs<S> a) {
   using R = typename S::real;
   const int rhs = rhs_slot(a.active);
-  if (a.skip != nullptr && (a.skip_rel ? !a.skip[rhs].need_rel : a.skip[rhs].done)) return;
+  if (a.skip != nullptr && (a.skip_rel ? !a.skip[rhs].need_rel : cg_idle(a.skip[rhs]))) return;
   const size_t off = rhs_offset<S>(rhs, a.sstride);
   const int ih = blockIdx.y * HOP_NT + threadIdx.x;
   R part = 0;   // FP32 kernels: FP32 up to the warp sums
@@ -611,7 +601,7 @@ __global__ void __launch_bounds__(HOP_NT, HopMinBlocks<S>::value) cg_update_kern
   using R = typename S::real;
   const int rhs = rhs_slot(a.active);
   CGState* st = a.st + rhs;
-  if (st->done) return;
+  if (cg_idle(*st)) return;
   const size_t off = rhs_offset<S>(rhs, a.sstride), offa = rhs_offset<SA>(rhs, a.sstride);
   typename SA::real part = 0;
   const int ih = blockIdx.y * HOP_NT + threadIdx.x;
@@ -766,7 +756,7 @@ __global__ void __launch_bounds__(LT_SITES * RPB, (TileMinBlocks<RPB, REGS>::val
   __shared__ LinkTile tile;
   using R = typename S::real;
   int rhs = tile_rhs(a.active, nrhs);
-  if (rhs >= 0 && a.skip != nullptr && (a.skip_rel ? !a.skip[rhs].need_rel : a.skip[rhs].done)) rhs = -1;
+  if (rhs >= 0 && a.skip != nullptr && (a.skip_rel ? !a.skip[rhs].need_rel : cg_idle(a.skip[rhs]))) rhs = -1;
   if (!__syncthreads_or(rhs >= 0)) return;   // every right-hand side of the block is idle
   // a reducing block walks LT_GROUPS<MODE> consecutive groups of 32 sites, so
   // that its grid-sum step (fence, ticket, barrier) is paid once per group run
@@ -795,7 +785,7 @@ __global__ void __launch_bounds__(256) cg_p_kernel(const typename SA::schunk* __
                                                    typename S::schunk* __restrict__ p, int sstride, int Vh,
                                                    const int* active, const CGState* st) {
   const int rhs = rhs_slot(active);
-  if (st[rhs].done) return;
+  if (cg_idle(st[rhs])) return;
   const int ih = blockIdx.y * blockDim.x + threadIdx.x;
   if (ih >= Vh) return;
   using R = typename S::real;
