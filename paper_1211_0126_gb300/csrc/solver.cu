@@ -317,8 +317,7 @@ static int cg_solve(Ctx& c, const tm_stop& stop, int s0, int nrhs, EOField b, EO
       TSM_TRY(check_launch(c, "rel_finish_kernel"));
     }
   }
-  // one CG iteration over the listed right-hand sides (n of them), followed,
-  // with reliable updates, by the FP64 update of those that asked for one
+  // one CG iteration over the listed right-hand sides (n of them)
   auto iteration = [&](const int* dact, int n, bool timed) -> int {
     c.prof_this_launch = c.profile && timed;
     HopArgs<S> h = hop_args<S>(c, 1);   // K1
@@ -368,13 +367,16 @@ static int cg_solve(Ctx& c, const tm_stop& stop, int s0, int nrhs, EOField b, EO
     TSM_TRY((launch_cg_update<S, SA>(c, u, n)));
     c.prof_this_launch = false;
     TSM_TRY((launch_cg_p<S, SA>(c, r, p, st, dact, n)));   // K5
+    return TSM_OK;
+  };
+  // reliable update (Sleijpen & van der Vorst; Clark et al. for lattice QCD):
+  // for every listed right-hand side whose residual fell by delta since the last
+  // update, or that met its stopping rule, fold the FP32 increment into the
+  // FP64 solution, replace the iterated residual by the normal residual of the
+  // true (FP64) Schur residual and restart the search direction from it; the
+  // others return at once from these kernels
+  auto reliable_update = [&](const int* dact, int n) -> int {
     if constexpr (REL) {
-      // reliable update (Sleijpen & van der Vorst; Clark et al. for lattice QCD):
-      // for every right-hand side whose residual fell by delta since the last
-      // update, or that met its stopping rule, fold the FP32 increment into the
-      // FP64 solution, replace the iterated residual by the normal residual of
-      // the true (FP64) Schur residual and restart the search direction from
-      // it; the others return at once from these kernels
       const int blocks = (c.g.Vh + SITE_NT - 1) / SITE_NT;
       accumulate_solution_kernel<<<dim3(n, blocks), SITE_NT, 0, c.stream>>>(c.g.Vh, x.as<F32>(), x64.as<F64>(),
                                                                            c.sstride, dact, st);
@@ -395,14 +397,34 @@ static int cg_solve(Ctx& c, const tm_stop& stop, int s0, int nrhs, EOField b, EO
   if (c.capturing) {
     // graph mode: the iterations become a graph while-loop whose condition a
     // device kernel clears once every source has met its stopping rule
-    TSM_TRY(capture_while(c, st, nrhs, stop.max_iter, [&]() { return iteration(nullptr, nrhs, false); }));
+    TSM_TRY(capture_while(c, st, nrhs, stop.max_iter, [&]() {
+      TSM_TRY(iteration(nullptr, nrhs, false));
+      return reliable_update(nullptr, nrhs);
+    }));
   } else {
     TSM_TRY(read_states(c, s0, nrhs, hs));
   }
   auto iterating = [&](int i) { return !c.capturing && !hs[i].done && hs[i].status == 0; };
-  const int chunk = 8;
+  const int chunk = 8, longest = REL ? 24 : 8;
   long long launched = 0;   // guards the host loop against states that stop advancing
   for (;;) {
+    if constexpr (REL) {
+      // A source that asked for a reliable update (or met its rule, which the
+      // update's FP64 residual has to confirm) waits, its iterates frozen, until
+      // the host sees it here: the eight kernels of the update are launched for
+      // those sources alone, two to four times per solve, instead of after every
+      // iteration (12^3x24, 8 sources, to 1e-12: about 40 of the 150 us of an
+      // iteration were launches that returned at once)
+      std::vector<int> rel;
+      for (int i = 0; i < nrhs; ++i)
+        if (iterating(i) && hs[i].need_rel) rel.push_back(i);
+      if (!rel.empty()) {
+        const int* drel = nullptr;
+        TSM_TRY(upload_list(c, 1, rel, &drel));
+        TSM_TRY(reliable_update(drel, (int)rel.size()));
+        TSM_TRY(read_states(c, s0, nrhs, hs));
+      }
+    }
     std::vector<int> act;
     int min_left = stop.max_iter;
     for (int i = 0; i < nrhs; ++i)
@@ -411,7 +433,7 @@ static int cg_solve(Ctx& c, const tm_stop& stop, int s0, int nrhs, EOField b, EO
         min_left = std::min(min_left, stop.max_iter - hs[i].iter);
       }
     if (act.empty()) break;
-    if (launched > 2 * (long long)stop.max_iter + 64) {
+    if (launched > 8 * (long long)stop.max_iter + 64) {
       set_error("solver state stopped advancing after %lld iterations", launched);
       return TSM_ERR_CUDA;
     }
@@ -420,11 +442,11 @@ static int cg_solve(Ctx& c, const tm_stop& stop, int s0, int nrhs, EOField b, EO
     TSM_TRY(upload_list(c, 0, act, &dact));
     int m = chunk;
     // after the first chunk: about as many iterations as the slowest listed
-    // source still needs at its convergence rate so far (rr falls by rr / rr0
-    // in iter iterations), so that a straggler or two do not drag a chunk of
-    // empty iterations behind them; the device still decides every stop
+    // source still needs, at its convergence rate so far (rr falls by rr / rr0
+    // in iter iterations), to its stopping rule or its next reliable update, so
+    // that a straggler or two do not drag a chunk of empty iterations behind
+    // them; the device still decides every stop
     if (launched > 0 && stop.rel_tol > 0.0) {
-      const double goal = stop.rel_tol * stop.rel_tol;   // rr / rr0 at the stopping rule
       int need = 1;
       for (int i : act) {
         const CGState& q = hs[i];
@@ -433,8 +455,10 @@ static int cg_solve(Ctx& c, const tm_stop& stop, int s0, int nrhs, EOField b, EO
           need = chunk;
           break;
         }
+        double goal = stop.rel_tol * stop.rel_tol;   // rr / rr0 at the next event
+        if (REL) goal = std::max(goal, q.delta2 * q.rr_ref / q.rr0);
         const double est = q.iter * std::log(goal / drop) / std::log(drop);
-        if (est > need) need = est < chunk ? (int)std::ceil(est) : chunk;
+        if (est > need) need = est < longest ? (int)std::ceil(est) : longest;
       }
       m = need;
     }
