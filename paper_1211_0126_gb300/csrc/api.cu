@@ -287,7 +287,8 @@ int record_run(Ctx& c, const tsm_params* p, TsmRun& run, tsm_loop_stats* st) {
       return launch_noise<S>(c, 1, ns, j0, f.o, n);
     });
   };
-  auto contract_to = [&](uint32_t j, EOField a, int pa, const EOField* b, int pb, double2* out) {
+  // the values of n consecutive sources, fields in batches
+  auto contract_to = [&](uint32_t j, EOField a, int pa, const EOField* b, int pb, double2* out, int n) {
     const ContractPlan& plan = run.plan;
     EOField wa{}, wb{};
     const EOField *pwa = nullptr, *pwb = nullptr;
@@ -302,20 +303,20 @@ int record_run(Ctx& c, const tsm_params* p, TsmRun& run, tsm_loop_stats* st) {
         pwb = &wb;
       }
     }
-    if (run.fp64_path) return launch_contract<double, F64, F64>(c, plan, ns, j, a, b, out, pwa, pwb);
+    if (run.fp64_path) return launch_contract<double, F64, F64>(c, plan, ns, j, a, b, out, pwa, pwb, n);
     if (b == nullptr) pb = pa;
-    if (pa == TSM_F64 && pb == TSM_F64) return launch_contract<float, F64, F64>(c, plan, ns, j, a, b, out, pwa, pwb);
-    if (pa == TSM_F64 && pb == TSM_F32) return launch_contract<float, F64, F32>(c, plan, ns, j, a, b, out, pwa, pwb);
-    if (pa == TSM_F64 && pb == TSM_F16) return launch_contract<float, F64, F16>(c, plan, ns, j, a, b, out, pwa, pwb);
-    if (pa == TSM_F32 && pb == TSM_F32) return launch_contract<float, F32, F32>(c, plan, ns, j, a, b, out, pwa, pwb);
-    if (pa == TSM_F32 && pb == TSM_F64) return launch_contract<float, F32, F64>(c, plan, ns, j, a, b, out, pwa, pwb);
-    if (pa == TSM_F32 && pb == TSM_F16) return launch_contract<float, F32, F16>(c, plan, ns, j, a, b, out, pwa, pwb);
-    if (pa == TSM_F16 && pb == TSM_F16) return launch_contract<float, F16, F16>(c, plan, ns, j, a, b, out, pwa, pwb);
+    if (pa == TSM_F64 && pb == TSM_F64) return launch_contract<float, F64, F64>(c, plan, ns, j, a, b, out, pwa, pwb, n);
+    if (pa == TSM_F64 && pb == TSM_F32) return launch_contract<float, F64, F32>(c, plan, ns, j, a, b, out, pwa, pwb, n);
+    if (pa == TSM_F64 && pb == TSM_F16) return launch_contract<float, F64, F16>(c, plan, ns, j, a, b, out, pwa, pwb, n);
+    if (pa == TSM_F32 && pb == TSM_F32) return launch_contract<float, F32, F32>(c, plan, ns, j, a, b, out, pwa, pwb, n);
+    if (pa == TSM_F32 && pb == TSM_F64) return launch_contract<float, F32, F64>(c, plan, ns, j, a, b, out, pwa, pwb, n);
+    if (pa == TSM_F32 && pb == TSM_F16) return launch_contract<float, F32, F16>(c, plan, ns, j, a, b, out, pwa, pwb, n);
+    if (pa == TSM_F16 && pb == TSM_F16) return launch_contract<float, F16, F16>(c, plan, ns, j, a, b, out, pwa, pwb, n);
     return bad(TSM_ERR_ARG, "no contraction for these field tiers");
   };
-  // value of source j for set 0 (HP-set corrections) or 1 (LP set), idx-th of its set
-  auto contract = [&](uint32_t j, EOField a, int pa, const EOField* b, int pb, int set, int idx) -> int {
-    if (!run.fft) return contract_to(j, a, pa, b, pb, (set ? run.d_lp : run.d_corr) + (size_t)idx * E);
+  // value of one source
+  auto contract_one = [&](uint32_t j, EOField a, int pa, const EOField* b, int pb, int set, int idx) -> int {
+    if (!run.fft) return contract_to(j, a, pa, b, pb, (set ? run.d_lp : run.d_corr) + (size_t)idx * E, 1);
     FftProjector& f = run.fftp;
     const GammaTab& gam = run.plan.gam;
     if (run.fp64_path) return f.accumulate<double, F64, F64>(c, gam, ns, j, a, b, set, idx + 1);
@@ -328,6 +329,21 @@ int record_run(Ctx& c, const tsm_params* p, TsmRun& run, tsm_loop_stats* st) {
     if (pa == TSM_F32 && pb == TSM_F16) return f.accumulate<float, F32, F16>(c, gam, ns, j, a, b, set, idx + 1);
     if (pa == TSM_F16 && pb == TSM_F16) return f.accumulate<float, F16, F16>(c, gam, ns, j, a, b, set, idx + 1);
     return bad(TSM_ERR_ARG, "no momentum projection for these field tiers");
+  };
+  // values of sources j .. j + n - 1 for set 0 (HP-set corrections) or 1 (LP
+  // set), idx-th of its set on: the local and derivative contractions take the
+  // batch at once, D_W and the momentum transform one source after the other
+  auto contract = [&](uint32_t j, EOField a, int pa, const EOField* b, int pb, int set, int idx, int n) -> int {
+    const bool single = run.fft || run.plan.one_end == CT_GEN_ONE_END;
+    for (int r = 0; single && n > 1 && r < n; ++r) {
+      const EOField ar = eo_at(a, pa, c.g.Vh, r);
+      EOField br{};
+      if (b != nullptr) br = eo_at(*b, pb, c.g.Vh, r);
+      TSM_TRY(contract_one(j + r, ar, pa, b ? &br : nullptr, pb, set, idx + r));
+    }
+    if (single && n > 1) return TSM_OK;
+    if (run.fft) return contract_one(j, a, pa, b, pb, set, idx);
+    return contract_to(j, a, pa, b, pb, (set ? run.d_lp : run.d_corr) + (size_t)idx * E, n);
   };
   // the LP solutions of a batch in the layout the contractions read
   auto unpack_lp = [&](EOField sol, EOField dst, int n) -> int {
@@ -364,9 +380,7 @@ int record_run(Ctx& c, const tsm_params* p, TsmRun& run, tsm_loop_stats* st) {
       if (rc == TSM_OK)
         rc = solve_batch(c, p->lp, slots(n, c.cap_lp), n, run.b_lp1, run.s_lp1, r_lp.data(), nullptr, -1, sp_lp);
       if (rc == TSM_OK) rc = unpack_lp(run.s_lp1, run.c_lp1, n);
-      for (int r = 0; r < n && rc == TSM_OK; ++r)
-        rc = contract(j0 + r, eo_at(run.c_lp1, cp_lp, c.g.Vh, r), cp_lp, nullptr, cp_lp, 1,
-                      (int)(j0 + r - p->lp_begin));
+      if (rc == TSM_OK) rc = contract(j0, run.c_lp1, cp_lp, nullptr, cp_lp, 1, (int)(j0 - p->lp_begin), n);
     }
     std::swap(r_lp, r_lp1);
     if (rc == TSM_OK && cudaEventRecord(c.join_ev, c.stream) != cudaSuccess) rc = TSM_ERR_CUDA;
@@ -411,10 +425,9 @@ int record_run(Ctx& c, const tsm_params* p, TsmRun& run, tsm_loop_stats* st) {
           st->hp_iters += r_hp[r].iters;
           if (!r_hp[r].converged) st->hp_not_converged++;
         }
-        const EOField sl = eo_at(run.c_lp, cp_lp, c.g.Vh, h0 + r);
-        TSM_TRY(contract(j0 + r, eo_at(run.s_hp, sp_hp, c.g.Vh, r), sp_hp, &sl, cp_lp, 0,
-                         (int)(j0 + r - p->hp_begin)));
       }
+      const EOField sl = eo_at(run.c_lp, cp_lp, c.g.Vh, h0);
+      TSM_TRY(contract(j0, run.s_hp, sp_hp, &sl, cp_lp, 0, (int)(j0 - p->hp_begin), n));
     }
   }
   // LP set: the same LP map, L(s_LP)
@@ -429,9 +442,8 @@ int record_run(Ctx& c, const tsm_params* p, TsmRun& run, tsm_loop_stats* st) {
           if (r_lp[r].status != TSM_OK) return bad(TSM_ERR_NONFINITE, "NaN/Inf in a solve");
           st->lp_iters += r_lp[r].iters;
         }
-        TSM_TRY(contract(j0 + r, eo_at(cl, cp_lp, c.g.Vh, r), cp_lp, nullptr, cp_lp, 1,
-                         (int)(j0 + r - p->lp_begin)));
       }
+      TSM_TRY(contract(j0, cl, cp_lp, nullptr, cp_lp, 1, (int)(j0 - p->lp_begin), n));
     }
     return TSM_OK;
   };
@@ -696,14 +708,17 @@ static int contract_entry(tsm_ctx* h, int one_end, int prec, uint64_t seed, int 
     plan.deriv_mask = deriv_mask;
   }
   const size_t bytes = spinor_bytes(c);
+  // the FP32 contraction of one solution rounds it to FP32 first, so that it is
+  // packed as FP32; differences and D_W are formed in FP64
+  const int pf = prec == TSM_F32 && s_b == nullptr && one_end != CT_GEN_ONE_END ? TSM_F32 : TSM_F64;
   EOField fa, fb;
-  TSM_TRY(eo_fields(c, "ct_a", TSM_F64, &fa));
-  TSM_TRY(eo_fields(c, "ct_b", TSM_F64, &fb));
+  TSM_TRY(eo_fields(c, "ct_a", pf, &fa));
   const double* da = nullptr;
   TSM_TRY(stage_in(c, "io_in", s_a, bytes, on_device, &da));
-  TSM_TRY(pack_eo(c, TSM_F64, da, fa));
+  TSM_TRY(pack_eo(c, pf, da, fa));
   if (s_b) {
     const double* db = nullptr;
+    TSM_TRY(eo_fields(c, "ct_b", TSM_F64, &fb));
     TSM_TRY(stage_in(c, "io_in2", s_b, bytes, on_device, &db));
     TSM_TRY(pack_eo(c, TSM_F64, db, fb));
   }
@@ -725,6 +740,9 @@ static int contract_entry(tsm_ctx* h, int one_end, int prec, uint64_t seed, int 
   if (prec == TSM_F64)
     TSM_TRY((launch_contract<double, F64, F64>(c, plan, ns, source, fa, s_b ? &fb : nullptr,
                                                reinterpret_cast<double2*>(dout), pwa, pwb)));
+  else if (pf == TSM_F32)
+    TSM_TRY((launch_contract<float, F32, F32>(c, plan, ns, source, fa, nullptr, reinterpret_cast<double2*>(dout), pwa,
+                                              pwb)));
   else
     TSM_TRY((launch_contract<float, F64, F64>(c, plan, ns, source, fa, s_b ? &fb : nullptr,
                                               reinterpret_cast<double2*>(dout), pwa, pwb)));
@@ -762,12 +780,12 @@ int tsm_contract_fft(tsm_ctx* h, int prec, uint64_t seed, int kind, uint32_t sou
   const size_t bytes = spinor_bytes(c);
   EOField fa, fb;
   TSM_TRY(eo_fields(c, "ct_a", TSM_F64, &fa));
-  TSM_TRY(eo_fields(c, "ct_b", TSM_F64, &fb));
   const double* da = nullptr;
   TSM_TRY(stage_in(c, "io_in", s_a, bytes, on_device, &da));
   TSM_TRY(pack_eo(c, TSM_F64, da, fa));
   if (s_b) {
     const double* db = nullptr;
+    TSM_TRY(eo_fields(c, "ct_b", TSM_F64, &fb));
     TSM_TRY(stage_in(c, "io_in2", s_b, bytes, on_device, &db));
     TSM_TRY(pack_eo(c, TSM_F64, db, fb));
   }

@@ -204,6 +204,14 @@ __device__ __forceinline__ double widen_f64(float v) {
   return (double)v;
 }
 
+// (R)x with the 64-bit narrowing and widening off the FP64 pipe
+template <class R, class T>
+__device__ __forceinline__ R real_cast(T x) {
+  if constexpr (sizeof(R) == 4 && sizeof(T) == 8) return narrow_f32(x);
+  else if constexpr (sizeof(R) == 8 && sizeof(T) == 4) return widen_f64(x);
+  else return x;
+}
+
 // load / store of the 12 complex components v[3*spin + colour]
 template <class S>
 __device__ __forceinline__ void load_spinor(const typename S::schunk* __restrict__ b, int stride, int i,
@@ -597,7 +605,7 @@ __device__ __forceinline__ int rhs_slot(const int* active) {
 
 // offset of right-hand side `rhs` in a batch of contiguous fields of storage S
 template <class S>
-__device__ __forceinline__ size_t rhs_offset(int rhs, int sstride) {
+__host__ __device__ __forceinline__ size_t rhs_offset(int rhs, int sstride) {
   if constexpr (S::id == F16G::id) return (size_t)(rhs >> 3) * 24 * (size_t)sstride + (size_t)(rhs & 7) * 3;
   return (size_t)rhs * S::SN * (size_t)sstride;
 }

@@ -187,9 +187,26 @@ int ContractPlan::prepare(Ctx& c, const int* gammas, int n_gamma, const int* mom
   return TSM_OK;
 }
 
+// block partials of one source at the most outputs a pass has
+static size_t contract_bytes(const Ctx& c) {
+  constexpr int NT = ContractNT<double>::value;   // the smaller block: the most partials
+  const int vs2 = c.lat.L[0] * c.lat.L[1] * c.lat.L[2] / 2;
+  return (size_t)c.lat.L[3] * 2 * ((vs2 + NT - 1) / NT) * CT_MAXG * CT_MAXQ * sizeof(double2);
+}
+
+// Partials of one launch: with several sources a launch fills the GPU on small
+// lattices (8^3x16, 64 sources: 64 x (5.8 + 3.8) us of single launches) and the
+// launches' tails overlap on large ones.
+constexpr size_t CT_PART_BYTES = (size_t)64 << 20;
+
 template <class R, class SA, class SB>
 int launch_contract(Ctx& c, const ContractPlan& plan, const NoiseSpec& ns, uint32_t source, EOField a,
-                    const EOField* b, double2* out, const EOField* wa, const EOField* wb) {
+                    const EOField* b, double2* out, const EOField* wa, const EOField* wb, int n) {
+  if (n < 1) return TSM_OK;
+  if (n > 1 && wa != nullptr) {
+    set_error("generalised one-end contractions take one source at a time");
+    return TSM_ERR_ARG;
+  }
   if (plan.one_end == CT_GEN_ONE_END && (wa == nullptr || (b != nullptr && wb == nullptr))) {
     set_error("generalised one-end contraction needs D_W of its fields");
     return TSM_ERR_ARG;
@@ -199,57 +216,65 @@ int launch_contract(Ctx& c, const ContractPlan& plan, const NoiseSpec& ns, uint3
   const int T = c.lat.L[3];
   const int nbx = (vs2 + NT - 1) / NT;
   const size_t block = (size_t)plan.ng * plan.n_q * T;   // one [n_gamma][n_q][T] output block
+  const size_t entries = (size_t)plan.entries(T);        // outputs per source
+  // sources per launch: as many as keep the block partials within CT_PART_BYTES
+  // (they go out and come back through L2), at least one
+  const size_t per = (size_t)T * 2 * nbx * plan.ng * std::min(CT_MAXQ, plan.n_q);
+  const int step = (int)std::max<size_t>(1, std::min<size_t>((size_t)n, CT_PART_BYTES / (per * sizeof(double2))));
   // one kernel + fixed-order reduction per chunk of at most CT_MAXQ momenta
   // algorithmic bytes per site of a pass: the fields it reads (noise is regenerated)
   const double sa = spinor_site_bytes(SA::id), sbb = spinor_site_bytes(SB::id);
   const double fields = sa + (b ? sbb : 0.0) + (wa ? sa : 0.0) + (wb ? sbb : 0.0);
   auto passes = [&](double2* dst, int kind, double site_bytes, auto&& launch) -> int {
-    for (int q0 = 0; q0 < plan.n_q; q0 += CT_MAXQ) {
-      const int nq = std::min(CT_MAXQ, plan.n_q - q0);
-      const int nout = plan.ng * nq;
-      // + block partials written and read back, + the output block
-      TimedLaunch tl(c, kind,
-                     (double)c.g.V * site_bytes + (double)T * 2 * nbx * nout * 32.0 + (double)nout * T * 16.0, true);
-      void* part = nullptr;
-      TSM_TRY(c.buffer("contract_partial", (size_t)T * 2 * nbx * CT_MAXG * CT_MAXQ * sizeof(double2), &part));
-      ContractArgs<SA, SB> args{};
-      args.g = c.g;
-      args.noise = ns;
-      args.source = source;
-      args.a[0] = a.e.as<SA>();
-      args.a[1] = a.o.as<SA>();
-      args.b[0] = b ? b->e.as<SB>() : nullptr;
-      args.b[1] = b ? b->o.as<SB>() : nullptr;
-      args.sstride = c.sstride;
-      args.gam = plan.gam;
-      args.mom = plan.passes[q0 / CT_MAXQ];
-      args.nq = nq;
-      args.phx = plan.phx + (size_t)q0 * c.lat.L[0];
-      args.phy = plan.phy + (size_t)q0 * c.lat.L[1];
-      args.phz = plan.phz + (size_t)q0 * c.lat.L[2];
-      args.fphx = plan.fphx + (size_t)q0 * c.lat.L[0];
-      args.fphy = plan.fphy + (size_t)q0 * c.lat.L[1];
-      args.fphz = plan.fphz + (size_t)q0 * c.lat.L[2];
-      args.partial = static_cast<double2*>(part);
-      args.nbx = nbx;
-      args.wa[0] = wa ? wa->e.as<SA>() : nullptr;
-      args.wa[1] = wa ? wa->o.as<SA>() : nullptr;
-      args.wb[0] = wb ? wb->e.as<SB>() : nullptr;
-      args.wb[1] = wb ? wb->o.as<SB>() : nullptr;
-      args.fre = plan.one_end == CT_GEN_ONE_END ? 2.0 : 0.0;
-      args.fim = plan.one_end == CT_ONE_END ? -4.0 * c.lat.kappa * c.lat.mu : 0.0;
-      args.ffre = (float)args.fre;
-      args.ffim = (float)args.fim;
-      launch(args, dim3(nbx, T, 2));
-      c.launches++;
-      TSM_TRY(check_launch(c, "contract_kernel"));
-      const dim3 rgrid((unsigned)((nout + 31) / 32), (unsigned)T), rblock(32, CT_RED_WARPS);
-      contract_reduce_kernel<<<rgrid, rblock, 0, c.stream>>>(static_cast<double2*>(part), T, nbx, plan.ng, nq,
-                                                             plan.n_q, q0, dst);
-      c.launches++;
-      TSM_TRY(check_launch(c, "contract_reduce_kernel"));
-      tl.done();
-    }
+    for (int k0 = 0; k0 < n; k0 += step)
+      for (int q0 = 0; q0 < plan.n_q; q0 += CT_MAXQ) {
+        const int m = std::min(step, n - k0);
+        const int nq = std::min(CT_MAXQ, plan.n_q - q0);
+        const int nout = plan.ng * nq;
+        const size_t pstride = (size_t)T * 2 * nbx * nout;
+        // + block partials written and read back, + the output block
+        TimedLaunch tl(c, kind, m * ((double)c.g.V * site_bytes + (double)pstride * 32.0 + (double)nout * T * 16.0), true);
+        void* part = nullptr;
+        TSM_TRY(c.buffer("contract_partial", std::max((size_t)m * pstride * sizeof(double2), contract_bytes(c)), &part));
+        ContractArgs<SA, SB> args{};
+        args.g = c.g;
+        args.noise = ns;
+        args.source = source + (uint32_t)k0;
+        args.a[0] = a.e.as<SA>() + rhs_offset<SA>(k0, c.sstride);
+        args.a[1] = a.o.as<SA>() + rhs_offset<SA>(k0, c.sstride);
+        args.b[0] = b ? b->e.as<SB>() + rhs_offset<SB>(k0, c.sstride) : nullptr;
+        args.b[1] = b ? b->o.as<SB>() + rhs_offset<SB>(k0, c.sstride) : nullptr;
+        args.sstride = c.sstride;
+        args.gam = plan.gam;
+        args.mom = plan.passes[q0 / CT_MAXQ];
+        args.nq = nq;
+        args.phx = plan.phx + (size_t)q0 * c.lat.L[0];
+        args.phy = plan.phy + (size_t)q0 * c.lat.L[1];
+        args.phz = plan.phz + (size_t)q0 * c.lat.L[2];
+        args.fphx = plan.fphx + (size_t)q0 * c.lat.L[0];
+        args.fphy = plan.fphy + (size_t)q0 * c.lat.L[1];
+        args.fphz = plan.fphz + (size_t)q0 * c.lat.L[2];
+        args.partial = static_cast<double2*>(part);
+        args.nbx = nbx;
+        args.pstride = pstride;
+        args.wa[0] = wa ? wa->e.as<SA>() : nullptr;
+        args.wa[1] = wa ? wa->o.as<SA>() : nullptr;
+        args.wb[0] = wb ? wb->e.as<SB>() : nullptr;
+        args.wb[1] = wb ? wb->o.as<SB>() : nullptr;
+        args.fre = plan.one_end == CT_GEN_ONE_END ? 2.0 : 0.0;
+        args.fim = plan.one_end == CT_ONE_END ? -4.0 * c.lat.kappa * c.lat.mu : 0.0;
+        args.ffre = (float)args.fre;
+        args.ffim = (float)args.fim;
+        launch(args, dim3(nbx, T, 2 * m));
+        c.launches++;
+        TSM_TRY(check_launch(c, "contract_kernel"));
+        const dim3 rgrid((unsigned)((nout + 31) / 32), (unsigned)T, (unsigned)m), rblock(32, CT_RED_WARPS);
+        contract_reduce_kernel<<<rgrid, rblock, 0, c.stream>>>(static_cast<double2*>(part), pstride, T, nbx, plan.ng, nq,
+                                                               plan.n_q, q0, dst + k0 * entries, entries);
+        c.launches++;
+        TSM_TRY(check_launch(c, "contract_reduce_kernel"));
+        tl.done();
+      }
     return TSM_OK;
   };
   double2* dst = out;
@@ -282,23 +307,23 @@ int launch_contract(Ctx& c, const ContractPlan& plan, const NoiseSpec& ns, uint3
 }
 
 template int launch_contract<double, F64, F64>(Ctx&, const ContractPlan&, const NoiseSpec&, uint32_t, EOField,
-                                               const EOField*, double2*, const EOField*, const EOField*);
+                                               const EOField*, double2*, const EOField*, const EOField*, int);
 template int launch_contract<float, F64, F64>(Ctx&, const ContractPlan&, const NoiseSpec&, uint32_t, EOField,
-                                              const EOField*, double2*, const EOField*, const EOField*);
+                                              const EOField*, double2*, const EOField*, const EOField*, int);
 template int launch_contract<float, F32, F32>(Ctx&, const ContractPlan&, const NoiseSpec&, uint32_t, EOField,
-                                              const EOField*, double2*, const EOField*, const EOField*);
+                                              const EOField*, double2*, const EOField*, const EOField*, int);
 template int launch_contract<float, F64, F32>(Ctx&, const ContractPlan&, const NoiseSpec&, uint32_t, EOField,
-                                              const EOField*, double2*, const EOField*, const EOField*);
+                                              const EOField*, double2*, const EOField*, const EOField*, int);
 template int launch_contract<double, F64, F32>(Ctx&, const ContractPlan&, const NoiseSpec&, uint32_t, EOField,
-                                               const EOField*, double2*, const EOField*, const EOField*);
+                                               const EOField*, double2*, const EOField*, const EOField*, int);
 template int launch_contract<float, F32, F64>(Ctx&, const ContractPlan&, const NoiseSpec&, uint32_t, EOField,
-                                              const EOField*, double2*, const EOField*, const EOField*);
+                                              const EOField*, double2*, const EOField*, const EOField*, int);
 template int launch_contract<float, F64, F16>(Ctx&, const ContractPlan&, const NoiseSpec&, uint32_t, EOField,
-                                              const EOField*, double2*, const EOField*, const EOField*);
+                                              const EOField*, double2*, const EOField*, const EOField*, int);
 template int launch_contract<float, F32, F16>(Ctx&, const ContractPlan&, const NoiseSpec&, uint32_t, EOField,
-                                              const EOField*, double2*, const EOField*, const EOField*);
+                                              const EOField*, double2*, const EOField*, const EOField*, int);
 template int launch_contract<float, F16, F16>(Ctx&, const ContractPlan&, const NoiseSpec&, uint32_t, EOField,
-                                              const EOField*, double2*, const EOField*, const EOField*);
+                                              const EOField*, double2*, const EOField*, const EOField*, int);
 
 int apply_wilson(Ctx& c, int prec, EOField in, EOField out) {
   return dispatch_prec(prec, [&](auto tag) -> int {
@@ -332,11 +357,8 @@ int apply_wilson(Ctx& c, int prec, EOField in, EOField out) {
 }
 
 int reserve_contract(Ctx& c) {
-  constexpr int NT = ContractNT<double>::value;   // the smaller block: the most partials
-  const int vs2 = c.lat.L[0] * c.lat.L[1] * c.lat.L[2] / 2;
-  const int nbx = (vs2 + NT - 1) / NT;
   void* part = nullptr;
-  return c.buffer("contract_partial", (size_t)c.lat.L[3] * 2 * nbx * CT_MAXG * CT_MAXQ * sizeof(double2), &part);
+  return c.buffer("contract_partial", std::max(CT_PART_BYTES, contract_bytes(c)), &part);
 }
 
 int launch_combine(Ctx& c, const double2* corr, int n_hp, const double2* lp, int n_lp, int E, double2* est,

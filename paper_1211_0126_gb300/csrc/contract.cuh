@@ -71,8 +71,8 @@ template <class SA, class SB>
 struct ContractArgs {
   Geom g;
   NoiseSpec noise;
-  uint32_t source;
-  const typename SA::schunk* a[2];   // even, odd
+  uint32_t source;                   // of batch entry 0; entry k: source + k
+  const typename SA::schunk* a[2];   // even, odd: batches of fields, one per source
   const typename SB::schunk* b[2];   // may be null
   const typename SA::schunk* wa[2];  // MODE 2: D_W a
   const typename SB::schunk* wb[2];  // MODE 2: D_W b (when b is given)
@@ -83,8 +83,9 @@ struct ContractArgs {
   const double2* phx;   // [nq][Lx]
   const double2* phy;   // [nq][Ly]
   const double2* phz;   // [nq][Lz]
-  double2* partial;     // [T][2][nbx][ng*nq]
+  double2* partial;     // [source][T][2][nbx][ng*nq]
   int nbx;
+  size_t pstride;       // partials of one source
   double fre, fim;      // one-end factor -4 i kappa mu (OE only)
   const float2* fphx;   // phase tables and factor rounded once to FP32 on the host
   const float2* fphy;
@@ -215,7 +216,7 @@ template <> struct Vec2<double> {
 // memory, and each output is formed from its class's cosine and sine sums
 // (times f when MODE applies a factor).  A fixed order throughout.
 template <class R, int NT, bool FACTOR, class SA, class SB>
-__device__ __forceinline__ void ct_reduce(const ContractArgs<SA, SB>& a, unsigned char* smem, int t, int parity) {
+__device__ __forceinline__ void ct_reduce(const ContractArgs<SA, SB>& a, unsigned char* smem, int src, int t, int parity) {
   const int tid = threadIdx.x;
   const int ng = a.gam.n, ncp = a.mom.ncp;
   const int gt_n = (ng + 3) >> 2, ct_n = ncp >> 2, types = gt_n * ct_n;
@@ -275,7 +276,7 @@ __device__ __forceinline__ void ct_reduce(const ContractArgs<SA, SB>& a, unsigne
   }
   __syncthreads();
   const int nout = ng * a.nq;
-  double2* dst = a.partial + ((size_t)(t * 2 + parity) * a.nbx + blockIdx.x) * nout;
+  double2* dst = a.partial + src * a.pstride + ((size_t)(t * 2 + parity) * a.nbx + blockIdx.x) * nout;
   for (int k = tid; k < nout; k += NT) {
     const int gi = k % ng, q = k / ng;
     const R* cs = chan + (gi * CT_CHS + a.mom.qch[q]) * 2;
@@ -295,7 +296,8 @@ __global__ void __launch_bounds__(ContractNT<R>::value) contract_kernel(const Co
   constexpr bool OE = MODE == CT_ONE_END;
   constexpr int NT = ContractNT<R>::value;
   __shared__ __align__(16) unsigned char smem[CtSmem<R, NT>::bytes];
-  const int t = blockIdx.y, parity = blockIdx.z;
+  // blockIdx.z: source of the batch, parity
+  const int t = blockIdx.y, parity = blockIdx.z & 1, src = blockIdx.z >> 1;
   const int vs2 = a.g.L[0] * a.g.L[1] * a.g.L[2] / 2;
   const int local = blockIdx.x * NT + threadIdx.x;
   const bool valid = local < vs2;
@@ -306,8 +308,8 @@ __global__ void __launch_bounds__(ContractNT<R>::value) contract_kernel(const Co
     site_coords(a.g, parity, ih, c);
     if constexpr (MODE == CT_GEN_ONE_END) {
       cx<typename SA::real> va[12], wa[12];
-      load_spinor<SA>(a.a[parity], a.sstride, ih, va);
-      load_spinor<SA>(a.wa[parity], a.sstride, ih, wa);
+      load_spinor<SA>(a.a[parity] + rhs_offset<SA>(src, a.sstride), a.sstride, ih, va);
+      load_spinor<SA>(a.wa[parity] + rhs_offset<SA>(src, a.sstride), a.sstride, ih, wa);
 #pragma unroll
       for (int x = 0; x < 4; ++x)
 #pragma unroll
@@ -315,14 +317,14 @@ __global__ void __launch_bounds__(ContractNT<R>::value) contract_kernel(const Co
           cx<R> acc = {0, 0};
 #pragma unroll
           for (int cc = 0; cc < 3; ++cc)
-            acc = cjmac(acc, cx<R>{(R)va[3 * x + cc].re, (R)va[3 * x + cc].im},
-                              cx<R>{(R)wa[3 * y + cc].re, (R)wa[3 * y + cc].im});
+            acc = cjmac(acc, cx<R>{real_cast<R>(va[3 * x + cc].re), real_cast<R>(va[3 * x + cc].im)},
+                              cx<R>{real_cast<R>(wa[3 * y + cc].re), real_cast<R>(wa[3 * y + cc].im)});
           S[x][y] = acc;
         }
       if (a.b[0] != nullptr) {
         cx<typename SB::real> vb[12], wb[12];
-        load_spinor<SB>(a.b[parity], a.sstride, ih, vb);
-        load_spinor<SB>(a.wb[parity], a.sstride, ih, wb);
+        load_spinor<SB>(a.b[parity] + rhs_offset<SB>(src, a.sstride), a.sstride, ih, vb);
+        load_spinor<SB>(a.wb[parity] + rhs_offset<SB>(src, a.sstride), a.sstride, ih, wb);
 #pragma unroll
         for (int x = 0; x < 4; ++x)
 #pragma unroll
@@ -330,8 +332,8 @@ __global__ void __launch_bounds__(ContractNT<R>::value) contract_kernel(const Co
             cx<R> acc = {0, 0};
 #pragma unroll
             for (int cc = 0; cc < 3; ++cc)
-              acc = cjmac(acc, cx<R>{(R)vb[3 * x + cc].re, (R)vb[3 * x + cc].im},
-                                cx<R>{(R)wb[3 * y + cc].re, (R)wb[3 * y + cc].im});
+              acc = cjmac(acc, cx<R>{real_cast<R>(vb[3 * x + cc].re), real_cast<R>(vb[3 * x + cc].im)},
+                                cx<R>{real_cast<R>(wb[3 * y + cc].re), real_cast<R>(wb[3 * y + cc].im)});
             S[x][y] = S[x][y] - acc;
           }
       }
@@ -344,22 +346,22 @@ __global__ void __launch_bounds__(ContractNT<R>::value) contract_kernel(const Co
     } else if constexpr (!OE) {
       const uint32_t lex = (uint32_t)(((c[3] * a.g.L[2] + c[2]) * a.g.L[1] + c[1]) * a.g.L[0] + c[0]);
       cx<R> eta[12], s[12];
-      noise_site<R>(a.noise, lex, a.source, eta);
+      noise_site<R>(a.noise, lex, a.source + (uint32_t)src, eta);
       {
         cx<typename SA::real> va[12];
-        load_spinor<SA>(a.a[parity], a.sstride, ih, va);
+        load_spinor<SA>(a.a[parity] + rhs_offset<SA>(src, a.sstride), a.sstride, ih, va);
         if (a.b[0] != nullptr) {
           cx<typename SB::real> vb[12];
-          load_spinor<SB>(a.b[parity], a.sstride, ih, vb);
+          load_spinor<SB>(a.b[parity] + rhs_offset<SB>(src, a.sstride), a.sstride, ih, vb);
           using W = typename SA::real;  // subtract in the solution's own precision
 #pragma unroll
           for (int k = 0; k < 12; ++k) {
-            const W re = va[k].re - (W)vb[k].re, im = va[k].im - (W)vb[k].im;
-            s[k] = {(R)re, (R)im};
+            const W re = va[k].re - real_cast<W>(vb[k].re), im = va[k].im - real_cast<W>(vb[k].im);
+            s[k] = {real_cast<R>(re), real_cast<R>(im)};
           }
         } else {
 #pragma unroll
-          for (int k = 0; k < 12; ++k) s[k] = {(R)va[k].re, (R)va[k].im};
+          for (int k = 0; k < 12; ++k) s[k] = {real_cast<R>(va[k].re), real_cast<R>(va[k].im)};
         }
       }
 #pragma unroll
@@ -374,19 +376,19 @@ __global__ void __launch_bounds__(ContractNT<R>::value) contract_kernel(const Co
     } else {
       cx<R> sa[12];
       cx<typename SA::real> va[12];
-      load_spinor<SA>(a.a[parity], a.sstride, ih, va);
+      load_spinor<SA>(a.a[parity] + rhs_offset<SA>(src, a.sstride), a.sstride, ih, va);
 #pragma unroll
-      for (int k = 0; k < 12; ++k) sa[k] = {(R)va[k].re, (R)va[k].im};
+      for (int k = 0; k < 12; ++k) sa[k] = {real_cast<R>(va[k].re), real_cast<R>(va[k].im)};
       if (a.b[0] != nullptr) {
         cx<typename SB::real> vb[12];
-        load_spinor<SB>(a.b[parity], a.sstride, ih, vb);
+        load_spinor<SB>(a.b[parity] + rhs_offset<SB>(src, a.sstride), a.sstride, ih, vb);
         using W = typename SA::real;
         cx<R> d[12], sb[12];
 #pragma unroll
         for (int k = 0; k < 12; ++k) {
-          const W re = va[k].re - (W)vb[k].re, im = va[k].im - (W)vb[k].im;
-          d[k] = {(R)re, (R)im};
-          sb[k] = {(R)vb[k].re, (R)vb[k].im};
+          const W re = va[k].re - real_cast<W>(vb[k].re), im = va[k].im - real_cast<W>(vb[k].im);
+          d[k] = {real_cast<R>(re), real_cast<R>(im)};
+          sb[k] = {real_cast<R>(vb[k].re), real_cast<R>(vb[k].im)};
         }
         // a^dag X a - b^dag X b = d^dag X a + b^dag X d
 #pragma unroll
@@ -420,7 +422,7 @@ __global__ void __launch_bounds__(ContractNT<R>::value) contract_kernel(const Co
   }
   ct_stage<R, NT>(a, smem, valid, S, c);
   __syncthreads();
-  ct_reduce<R, NT, MODE != CT_STANDARD>(a, smem, t, parity);
+  ct_reduce<R, NT, MODE != CT_STANDARD>(a, smem, src, t, parity);
 }
 
 // ---------------------------------------------------------------- one-derivative insertions
@@ -442,18 +444,18 @@ struct DerivArgs {
 };
 
 template <class R, class SA, class SB>
-__device__ __forceinline__ void deriv_field(const ContractArgs<SA, SB>& a, int parity, int ih, cx<R> s[12]) {
+__device__ __forceinline__ void deriv_field(const ContractArgs<SA, SB>& a, int src, int parity, int ih, cx<R> s[12]) {
   cx<typename SA::real> va[12];
-  load_spinor<SA>(a.a[parity], a.sstride, ih, va);
+  load_spinor<SA>(a.a[parity] + rhs_offset<SA>(src, a.sstride), a.sstride, ih, va);
   if (a.b[0] != nullptr) {
     cx<typename SB::real> vb[12];
-    load_spinor<SB>(a.b[parity], a.sstride, ih, vb);
+    load_spinor<SB>(a.b[parity] + rhs_offset<SB>(src, a.sstride), a.sstride, ih, vb);
     using W = typename SA::real;
 #pragma unroll
-    for (int k = 0; k < 12; ++k) s[k] = {(R)(va[k].re - (W)vb[k].re), (R)(va[k].im - (W)vb[k].im)};
+    for (int k = 0; k < 12; ++k) s[k] = {real_cast<R>(va[k].re - real_cast<W>(vb[k].re)), real_cast<R>(va[k].im - real_cast<W>(vb[k].im))};
   } else {
 #pragma unroll
-    for (int k = 0; k < 12; ++k) s[k] = {(R)va[k].re, (R)va[k].im};
+    for (int k = 0; k < 12; ++k) s[k] = {real_cast<R>(va[k].re), real_cast<R>(va[k].im)};
   }
 }
 
@@ -476,7 +478,8 @@ __global__ void __launch_bounds__(ContractNT<R>::value) deriv_contract_kernel(co
   constexpr int NT = ContractNT<R>::value;
   const ContractArgs<SA, SB>& a = d.base;
   __shared__ __align__(16) unsigned char smem[CtSmem<R, NT>::bytes];
-  const int t = blockIdx.y, parity = blockIdx.z;
+  // blockIdx.z: source of the batch, parity
+  const int t = blockIdx.y, parity = blockIdx.z & 1, src = blockIdx.z >> 1;
   const int vs2 = a.g.L[0] * a.g.L[1] * a.g.L[2] / 2;
   const int local = blockIdx.x * NT + threadIdx.x;
   const bool valid = local < vs2;
@@ -513,19 +516,19 @@ __global__ void __launch_bounds__(ContractNT<R>::value) deriv_contract_kernel(co
       for (int k = 0; k < 9; ++k) ub[k] = {(R)r[k].re, (R)r[k].im};
     }
     cx<R> eta[12], s[12], ds[12], de[12], tmp[12], f[12];
-    noise_site<R>(a.noise, lex, a.source, eta);
-    deriv_field<R>(a, parity, ih, s);
+    noise_site<R>(a.noise, lex, a.source + (uint32_t)src, eta);
+    deriv_field<R>(a, src, parity, ih, s);
     // D s = T+ s - T- s
-    deriv_field<R>(a, 1 - parity, hf, f);
+    deriv_field<R>(a, src, 1 - parity, hf, f);
     colour_mul<false>(uf, f, sf, ds);
-    deriv_field<R>(a, 1 - parity, hb, f);
+    deriv_field<R>(a, src, 1 - parity, hb, f);
     colour_mul<true>(ub, f, sb, tmp);
 #pragma unroll
     for (int k = 0; k < 12; ++k) ds[k] = ds[k] - tmp[k];
     // D eta = T+ eta - T- eta
-    noise_site<R>(a.noise, lexf, a.source, f);
+    noise_site<R>(a.noise, lexf, a.source + (uint32_t)src, f);
     colour_mul<false>(uf, f, sf, de);
-    noise_site<R>(a.noise, lexb, a.source, f);
+    noise_site<R>(a.noise, lexb, a.source + (uint32_t)src, f);
     colour_mul<true>(ub, f, sb, tmp);
 #pragma unroll
     for (int k = 0; k < 12; ++k) de[k] = de[k] - tmp[k];
@@ -542,7 +545,7 @@ __global__ void __launch_bounds__(ContractNT<R>::value) deriv_contract_kernel(co
   }
   ct_stage<R, NT>(a, smem, valid, S, c);
   __syncthreads();
-  ct_reduce<R, NT, false>(a, smem, t, parity);
+  ct_reduce<R, NT, false>(a, smem, src, t, parity);
 }
 
 // sum the block partials of one timeslice in fixed order into the output
@@ -553,8 +556,10 @@ __global__ void __launch_bounds__(ContractNT<R>::value) deriv_contract_kernel(co
 // flight, then warp 0 adds the eight warp sums in warp order.
 constexpr int CT_RED_WARPS = 8;
 static __global__ void __launch_bounds__(32 * CT_RED_WARPS)
-contract_reduce_kernel(const double2* __restrict__ partial, int T, int nbx, int ng, int nq, int nq_total, int q0,
-                       double2* __restrict__ out) {
+contract_reduce_kernel(const double2* __restrict__ partial, size_t pstride, int T, int nbx, int ng, int nq,
+                       int nq_total, int q0, double2* __restrict__ out, size_t ostride) {
+  partial += blockIdx.z * pstride;   // blockIdx.z: source of the batch
+  out += blockIdx.z * ostride;
   __shared__ double2 sh[CT_RED_WARPS][32];
   const int nout = ng * nq, t = blockIdx.y, rows = 2 * nbx;
   const int gq = blockIdx.x * 32 + threadIdx.x, w = threadIdx.y;

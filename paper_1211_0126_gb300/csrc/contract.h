@@ -38,10 +38,12 @@ NoiseSpec make_noise(uint64_t seed, int kind);
 
 // out[g][q][t] (device, complex) = sum_t-slice e^{iqx} eta^dag Gamma_g (a - b), or
 // with plan.one_end the one-end values f(a) - f(b), f(s) = -4 i kappa mu s^dag g5 Gamma_g s
-// (plan.one_end == 2 needs wa = D_W a and, with b, wb = D_W b)
+// (plan.one_end == 2 needs wa = D_W a and, with b, wb = D_W b).  n sources
+// (source, source + 1, ...; not with plan.one_end == 2): a and b are batches of
+// fields, out receives plan.entries() values per source
 template <class R, class SA, class SB>
 int launch_contract(Ctx& c, const ContractPlan& plan, const NoiseSpec& ns, uint32_t source, EOField a,
-                    const EOField* b, double2* out, const EOField* wa = nullptr, const EOField* wb = nullptr);
+                    const EOField* b, double2* out, const EOField* wa = nullptr, const EOField* wb = nullptr, int n = 1);
 
 // out = D_W in = in - kappa H in on both parities (fields of tier prec)
 int apply_wilson(Ctx& c, int prec, EOField in, EOField out);

@@ -238,10 +238,10 @@ __global__ void __launch_bounds__(FFT_XY_NT, XYMinBlocks<R>::value) fft_xy_kerne
       load_spinor<SB>(parity ? b1 : b0, sstride, ih, vb);
       using W = typename SA::real;
 #pragma unroll
-      for (int k = 0; k < 12; ++k) s[k] = {(R)(va[k].re - (W)vb[k].re), (R)(va[k].im - (W)vb[k].im)};
+      for (int k = 0; k < 12; ++k) s[k] = {real_cast<R>(va[k].re - real_cast<W>(vb[k].re)), real_cast<R>(va[k].im - real_cast<W>(vb[k].im))};
     } else {
 #pragma unroll
-      for (int k = 0; k < 12; ++k) s[k] = {(R)va[k].re, (R)va[k].im};
+      for (int k = 0; k < 12; ++k) s[k] = {real_cast<R>(va[k].re), real_cast<R>(va[k].im)};
     }
     cx<R> S[4][4];
 #pragma unroll
