@@ -490,11 +490,13 @@ int tsm_create(int device, void* cuda_stream, tsm_ctx** out) {
   int rc = select_device(c);
   if (rc == TSM_OK && cudaDeviceGetAttribute(&c.sm_count, cudaDevAttrMultiProcessorCount, device) != cudaSuccess)
     rc = TSM_ERR_CUDA;
-  if (rc == TSM_OK && cudaMallocHost(&c.h_err, sizeof(int)) != cudaSuccess) rc = TSM_ERR_CUDA;
-  if (rc == TSM_OK) *c.h_err = 0;
   if (rc == TSM_OK && cudaMalloc(&c.states, Ctx::kMaxStates * sizeof(CGState)) != cudaSuccess) rc = TSM_ERR_CUDA;
-  if (rc == TSM_OK && cudaMallocHost(&c.h_states, Ctx::kMaxStates * sizeof(CGState)) != cudaSuccess)
+  if (rc == TSM_OK && cudaMallocHost(&c.h_states, Ctx::kMaxStates * sizeof(CGState) + sizeof(int)) != cudaSuccess)
     rc = TSM_ERR_CUDA;
+  if (rc == TSM_OK) {
+    c.h_err = reinterpret_cast<int*>(c.h_states + Ctx::kMaxStates);
+    *c.h_err = 0;
+  }
   if (rc == TSM_OK && cudaMalloc(&c.red.counter, Ctx::kMaxBatch * sizeof(unsigned int)) != cudaSuccess)
     rc = TSM_ERR_CUDA;
   if (rc == TSM_OK && cudaMemset(c.red.counter, 0, Ctx::kMaxBatch * sizeof(unsigned int)) != cudaSuccess)
@@ -543,16 +545,20 @@ int tsm_load_gauge(tsm_ctx* h, const tm_lattice* lat, const double* U, int on_de
     TSM_CUDA(cudaStreamSynchronize(c.stream));
     for (auto& kv : c.ws) cudaFree(kv.second.first);
     c.ws.clear();
-    for (void*& l : c.links) {
-      if (l) cudaFree(l);
-      l = nullptr;
-    }
+    if (c.links_base) cudaFree(c.links_base);
+    c.links_base = nullptr;
     const size_t vh = (size_t)c.g.Vh;
-    TSM_CUDA(cudaMalloc(&c.links[TSM_F64], 2 * 4 * F64::LN * vh * sizeof(double2)));
-    TSM_CUDA(cudaMalloc(&c.links[TSM_F32], 2 * 4 * F32::LN * vh * sizeof(float4)));
-    TSM_CUDA(cudaMalloc(&c.links[TSM_BF16], 2 * 4 * BF16::LN * vh * sizeof(uint2)));
-    TSM_CUDA(cudaMalloc(&c.links[TSM_F16], 2 * 4 * F16::LN * vh * sizeof(uint2)));
-    TSM_CUDA(cudaMalloc(&c.links[F16G::id], 2 * 4 * F16G::LN * vh * sizeof(uint32_t)));
+    // the links of every storage in one allocation
+    const size_t per_site[5] = {4 * F64::LN * sizeof(double2), 4 * F32::LN * sizeof(float4),
+                                4 * BF16::LN * sizeof(uint2), 4 * F16::LN * sizeof(uint2),
+                                4 * F16G::LN * sizeof(uint32_t)};
+    size_t off[5], total = 0;
+    for (int k = 0; k < 5; ++k) {
+      off[k] = total;
+      total += (2 * vh * per_site[k] + 255) & ~(size_t)255;
+    }
+    TSM_CUDA(cudaMalloc(&c.links_base, total));
+    for (int k = 0; k < 5; ++k) c.links[k] = static_cast<char*>(c.links_base) + off[k];
     if (c.red.partials) cudaFree(c.red.partials);
     c.red_cap = vh / 32 + 64;   // block partials: up to one per 32 sites (link-sharing stencil)
     c.red.stride = (int)c.red_cap;
@@ -1006,7 +1012,7 @@ int tsm_loops_graph(tsm_ctx** ctxs, const tsm_params* params, int n, double** lo
           st[i].hp_iters += q.iter;
           if (q.status != 0) rc = TSM_ERR_NONFINITE;
           const bool met = q.rr0 == 0.0 || (q.tol <= 0.0 ? q.iter >= q.max_iter
-                                                         : !(std::sqrt(q.rr) >= q.tol * std::sqrt(q.rr0)));
+                                                         : rule_met(&q, q.rr));
           if (!met) st[i].hp_not_converged++;
         }
       if (stats) stats[i] = st[i];

@@ -123,12 +123,10 @@ void Ctx::free_all() {
   cudaStreamSynchronize(stream);
   for (auto& kv : ws) cudaFree(kv.second.first);
   ws.clear();
-  for (void*& l : links) {
-    if (l) cudaFree(l);
-    l = nullptr;
-  }
-  if (h_err) cudaFreeHost(h_err);
-  h_err = nullptr;
+  if (links_base) cudaFree(links_base);
+  links_base = nullptr;
+  for (void*& l : links) l = nullptr;
+  h_err = nullptr;   // lives behind h_states
   if (red.partials) cudaFree(red.partials);
   if (red.counter) cudaFree(red.counter);
   if (red_branch.partials) cudaFree(red_branch.partials);

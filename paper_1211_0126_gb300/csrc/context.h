@@ -65,6 +65,7 @@ struct Ctx {
   int lstride = 0;       // chunk stride of link fields (= Vh)
   // F64, F32, BF16, F16: [2][4][LN][lstride]; F16G: [2][lstride][8][12] words
   void* links[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
+  void* links_base = nullptr;   // their allocation
   int sm_count = 1;
   int* h_err = nullptr;                 // pinned, device-visible: set by a kernel whose bounded wait ran out
   std::map<std::string, std::pair<void*, size_t>> ws;      // named device workspace
@@ -161,6 +162,23 @@ inline Twist twist_mul(const Twist& a, const Twist& b) {
     t.im[q] = a.re[q] * b.im[q] + a.im[q] * b.re[q];
   }
   return t;
+}
+
+// launch with programmatic dependence on the stream's previous kernel (see
+// pdl_wait); under stream capture an ordinary launch
+template <class... P, class... A>
+cudaError_t launch_pdl(const Ctx& c, void (*k)(P...), dim3 grid, dim3 block, size_t smem, A&&... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = c.stream;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = c.capturing ? 0 : 1;
+  return cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
 }
 
 // ---- launch helpers (instantiated per storage type in ops_*.cu).  Batched

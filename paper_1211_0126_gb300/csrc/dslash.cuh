@@ -372,6 +372,7 @@ __device__ __forceinline__ typename S::real hop_epilogue(const HopArgs<S>& a, si
 template <class S, int DAG, int MODE>
 __global__ void __launch_bounds__(HOP_NT, HopMinBlocks<S>::value) hop_kernel(const HopArgs<S> a) {
   using R = typename S::real;
+  pdl_wait();
   const int rhs = rhs_slot(a.active);
   if (a.skip != nullptr && (a.skip_rel ? !a.skip[rhs].need_rel : cg_idle(a.skip[rhs]))) return;
   const size_t off = rhs_offset<S>(rhs, a.sstride);
@@ -384,6 +385,7 @@ __global__ void __launch_bounds__(HOP_NT, HopMinBlocks<S>::value) hop_kernel(con
     hop_site<S, DAG>(a.g, ih, c, a.Uout, a.Uin, a.lstride, a.in + off, a.sstride, acc);
     part = hop_epilogue<S, MODE>(a, off, ih, acc);
   }
+  pdl_trigger();
   if constexpr (MODE & HOP_NORM) {
     double total;
     if (grid_sum<HOP_NT>(part, a.red, rhs, &total) && threadIdx.x == 0 && a.st != nullptr)
@@ -599,6 +601,7 @@ __device__ __forceinline__ typename SA::real cg_update_epilogue(const CGUpdArgs<
 template <class S, class SA>
 __global__ void __launch_bounds__(HOP_NT, HopMinBlocks<S>::value) cg_update_kernel(const CGUpdArgs<S, SA> a) {
   using R = typename S::real;
+  pdl_wait();
   const int rhs = rhs_slot(a.active);
   CGState* st = a.st + rhs;
   if (cg_idle(*st)) return;
@@ -612,6 +615,7 @@ __global__ void __launch_bounds__(HOP_NT, HopMinBlocks<S>::value) cg_update_kern
     hop_site<S, 1>(a.g, ih, c, a.Ue, a.Uo, a.lstride, a.t + off, a.sstride, acc);
     part = cg_update_epilogue<S, SA>(a, st, off, offa, ih, acc);
   }
+  pdl_trigger();
   double total;
   if (grid_sum<HOP_NT>(part, a.red, rhs, &total) && threadIdx.x == 0) post_action(st, POST_RR, total);
 }
@@ -755,6 +759,13 @@ __global__ void __launch_bounds__(LT_SITES * RPB, (TileMinBlocks<RPB, REGS>::val
     hop_tile_kernel(const HopArgs<S> a, int nrhs) {
   __shared__ LinkTile tile;
   using R = typename S::real;
+  {   // the first group's links do not depend on the previous kernel
+    const int ih = blockIdx.y * LtGroups<MODE>::value * LT_SITES + threadIdx.x;
+    int c[4] = {0, 0, 0, 0};
+    if (ih < a.g.Vh) site_coords(a.g, a.p_out, ih, c);
+    stage_tile<S>(a.g, ih, c, a.Uout, a.Uin, a.lstride, tile);
+  }
+  pdl_wait();
   int rhs = tile_rhs(a.active, nrhs);
   if (rhs >= 0 && a.skip != nullptr && (a.skip_rel ? !a.skip[rhs].need_rel : cg_idle(a.skip[rhs]))) rhs = -1;
   if (!__syncthreads_or(rhs >= 0)) return;   // every right-hand side of the block is idle
@@ -766,9 +777,11 @@ __global__ void __launch_bounds__(LT_SITES * RPB, (TileMinBlocks<RPB, REGS>::val
     const int ih = (blockIdx.y * LtGroups<MODE>::value + grp) * LT_SITES + threadIdx.x;
     int c[4] = {0, 0, 0, 0};
     if (ih < a.g.Vh) site_coords(a.g, a.p_out, ih, c);
-    if (grp > 0) __syncthreads();   // the previous group's links are consumed
-    stage_tile<S>(a.g, ih, c, a.Uout, a.Uin, a.lstride, tile);
-    __syncthreads();
+    if (grp > 0) {
+      __syncthreads();   // the previous group's links are consumed
+      stage_tile<S>(a.g, ih, c, a.Uout, a.Uin, a.lstride, tile);
+      __syncthreads();
+    }
     if (rhs >= 0 && ih < a.g.Vh) {
       const size_t off = rhs_offset<S>(rhs, a.sstride);
       cx<R> acc[12];
@@ -776,6 +789,7 @@ __global__ void __launch_bounds__(LT_SITES * RPB, (TileMinBlocks<RPB, REGS>::val
       part += hop_epilogue<S, MODE>(a, off, ih, acc);
     }
   }
+  pdl_trigger();
   if constexpr (MODE & HOP_NORM) tile_grid_sum<RPB>(part, rhs, a.red, a.st, a.post);
 }
 
@@ -784,6 +798,7 @@ template <class S, class SA>
 __global__ void __launch_bounds__(256) cg_p_kernel(const typename SA::schunk* __restrict__ r,
                                                    typename S::schunk* __restrict__ p, int sstride, int Vh,
                                                    const int* active, const CGState* st) {
+  pdl_wait();
   const int rhs = rhs_slot(active);
   if (cg_idle(st[rhs])) return;
   const int ih = blockIdx.y * blockDim.x + threadIdx.x;

@@ -347,6 +347,7 @@ __global__ void __launch_bounds__(MMA_NT, 1) mma_hop_kernel(const MmaHopArgs a, 
         if (lane < 8) s_sum[warp][j][lane] = 0.0;
       }
   }
+  pdl_wait();
   __syncthreads();
   // the launch's live sources as a bit mask over the batch
   if (threadIdx.x < a.nrhs) {
@@ -575,6 +576,7 @@ __global__ void __launch_bounds__(MMA_NT, 1) mma_hop_kernel(const MmaHopArgs a, 
     }
     __syncthreads();
   }
+  pdl_trigger();
   if constexpr (NORM) {
     __shared__ bool s_last;
     if (threadIdx.x < 64 && ((mask >> threadIdx.x) & 1ull)) {
@@ -604,6 +606,7 @@ __global__ void __launch_bounds__(MMA_NT, 1) mma_hop_kernel(const MmaHopArgs a, 
 // (24 chunks); memory-bound
 static __global__ void __launch_bounds__(256) mma_p_kernel(const uint4* __restrict__ r, uint4* __restrict__ p, int Vh,
                                                            const int* active, int nrhs, const CGState* st) {
+  pdl_wait();
   const int lane = threadIdx.x & 31, q = lane % 3, row = lane / 3;
   const int k = blockIdx.x * 8 + row;
   if (lane >= 24 || k >= nrhs) return;

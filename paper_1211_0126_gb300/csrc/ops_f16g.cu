@@ -76,7 +76,7 @@ template <int DAG, int MODE>
 int mma_launch(Ctx& c, const MmaHopArgs& m, const MmaMaps& maps, dim3 grid) {
   constexpr int smem = MmaStage<MODE>::BYTES * MmaStage<MODE>::COUNT;
   TSM_CUDA(cudaFuncSetAttribute(mma_hop_kernel<DAG, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  mma_hop_kernel<DAG, MODE><<<grid, MMA_NT, smem, c.stream>>>(m, maps);
+  (void)launch_pdl(c, mma_hop_kernel<DAG, MODE>, grid, dim3(MMA_NT), smem, m, maps);
   c.launches++;
   return check_launch(c, "mma_hop_kernel");
 }
@@ -156,7 +156,7 @@ template <>
 int launch_cg_p<F16G, F16G>(Ctx& c, const PField& r, const PField& p, CGState* st, const int* active, int nrhs) {
   if (c.g.Vh == 0 || nrhs == 0) return TSM_OK;
   const dim3 grid(groups_of(nrhs), std::min(blocks_for(c.g.Vh, 32), 8 * c.sm_count));
-  mma_p_kernel<<<grid, 256, 0, c.stream>>>(r.as<F16G>(), p.as<F16G>(), c.g.Vh, active, nrhs, st);
+  (void)launch_pdl(c, mma_p_kernel, grid, dim3(256), 0, r.as<F16G>(), p.as<F16G>(), c.g.Vh, active, nrhs, st);
   c.launches++;
   return check_launch(c, "mma_p_kernel");
 }

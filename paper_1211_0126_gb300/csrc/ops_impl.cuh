@@ -49,19 +49,20 @@ int launch_hop(Ctx& c, const HopArgs<S>& a0, int dag, int mode, int prof_kind, i
   const int tile_sites = LT_SITES * ((mode & HOP_NORM) ? LtGroups<HOP_NORM>::value : LtGroups<0>::value);
   const dim3 grid = tile ? dim3((nrhs + rpb - 1) / rpb, blocks_for(a.g.Vh, tile_sites)) : dim3(nrhs, nb);
   const dim3 block = tile ? dim3(LT_SITES, rpb) : dim3(HOP_NT);
-#define TSM_HOP_CASE(D, M)                                                                        \
-  if (dag == (D) && mode == (M)) {                                                                \
-    if (tile) {                                                                                   \
-      if constexpr (TILE16 || (TILE32 && !((M) & HOP_NORM))) {                                    \
-        if (RPB == 2) hop_tile_kernel<S, (D), (M), 2, 80><<<grid, block, 0, c.stream>>>(a, nrhs); \
-        else if (RPB == 8) hop_tile_kernel<S, (D), (M), 8, 80><<<grid, block, 0, c.stream>>>(a, nrhs); \
-        else if (wide) hop_tile_kernel<S, (D), (M), 4, 96><<<grid, block, 0, c.stream>>>(a, nrhs); \
-        else hop_tile_kernel<S, (D), (M), 4, 80><<<grid, block, 0, c.stream>>>(a, nrhs);          \
-      }                                                                                           \
-    } else {                                                                                      \
-      hop_kernel<S, (D), (M)><<<grid, block, 0, c.stream>>>(a);                                   \
-    }                                                                                             \
+#define TSM_HOP_CASE(D, M)                                                                  \
+  if (dag == (D) && mode == (M)) {                                                          \
+    if (tile) {                                                                             \
+      if constexpr (TILE16 || (TILE32 && !((M) & HOP_NORM))) {                              \
+        if (RPB == 2) le = launch_pdl(c, hop_tile_kernel<S, (D), (M), 2, 80>, grid, block, 0, a, nrhs); \
+        else if (RPB == 8) le = launch_pdl(c, hop_tile_kernel<S, (D), (M), 8, 80>, grid, block, 0, a, nrhs); \
+        else if (wide) le = launch_pdl(c, hop_tile_kernel<S, (D), (M), 4, 96>, grid, block, 0, a, nrhs); \
+        else le = launch_pdl(c, hop_tile_kernel<S, (D), (M), 4, 80>, grid, block, 0, a, nrhs); \
+      }                                                                                     \
+    } else {                                                                                \
+      le = launch_pdl(c, hop_kernel<S, (D), (M)>, grid, block, 0, a);                       \
+    }                                                                                       \
   }
+  cudaError_t le = cudaSuccess;
   TSM_HOP_CASE(0, 0)
   else TSM_HOP_CASE(0, HOP_CENTER)
   else TSM_HOP_CASE(0, HOP_CENTER | HOP_NORM)
@@ -75,6 +76,7 @@ int launch_hop(Ctx& c, const HopArgs<S>& a0, int dag, int mode, int prof_kind, i
     return TSM_ERR_ARG;
   }
 #undef TSM_HOP_CASE
+  (void)le;   // check_launch reports it
   tl.done();
   c.launches++;
   return check_launch(c, "hop_kernel");
@@ -116,7 +118,7 @@ int launch_cg_update(Ctx& c, const CGUpdArgs<S, SA>& a0, int nrhs) {
   TimedLaunch tl(c, 4 * S::id + PK_HOP_UPDATE, (double)a.g.Vh * (lb + nrhs * (3 * sb + 4 * sa)));
   // one thread per (source, site) for every tier: the update is memory-bound,
   // and link sharing measured slower here (534 against 511 us per launch)
-  cg_update_kernel<S, SA><<<dim3(nrhs, nb), HOP_NT, 0, c.stream>>>(a);
+  (void)launch_pdl(c, cg_update_kernel<S, SA>, dim3(nrhs, nb), dim3(HOP_NT), 0, a);
   tl.done();
   c.launches++;
   return check_launch(c, "cg_update_kernel");
@@ -126,7 +128,8 @@ template <class S, class SA>
 int launch_cg_p(Ctx& c, const PField& r, const PField& p, CGState* st, const int* active, int nrhs) {
   const int nb = blocks_for(c.g.Vh, SITE_NT);
   if (nb == 0 || nrhs == 0) return TSM_OK;
-  cg_p_kernel<S, SA><<<dim3(nrhs, nb), SITE_NT, 0, c.stream>>>(r.as<SA>(), p.as<S>(), c.sstride, c.g.Vh, active, st);
+  (void)launch_pdl(c, cg_p_kernel<S, SA>, dim3(nrhs, nb), dim3(SITE_NT), 0, r.as<SA>(), p.as<S>(), c.sstride, c.g.Vh,
+                   active, st);
   c.launches++;
   return check_launch(c, "cg_p_kernel");
 }

@@ -493,7 +493,7 @@ static int cg_solve(Ctx& c, const tm_stop& stop, int s0, int nrhs, EOField b, EO
     o.rel_res = q.rr0 > 0 ? std::sqrt(q.rr / q.rr0) : 0.0;
     if (q.rr0 == 0.0) o.converged = 1;
     else if (stop.rel_tol <= 0.0) o.converged = q.iter >= stop.max_iter;
-    else o.converged = !(std::sqrt(q.rr) >= stop.rel_tol * std::sqrt(q.rr0));
+    else o.converged = rule_met(&q, q.rr);
   }
   return TSM_OK;
 }
