@@ -10,6 +10,7 @@
 
 #include "contract.h"
 #include "net.h"
+#include "ptlayer.cuh"
 #include "ptnet.cuh"
 #include "solver.h"
 #include "tma_map.h"
@@ -197,10 +198,41 @@ int Net::pack(cudaStream_t s) {
     const int n = l.n4() * l.k36();
     pt_pack_weights_kernel<<<grid1(n, 256), 256, 0, s>>>(l.wr, l.wi, l.n4(), l.k36(), l.B, l.Bt);
     TSM_CUDA(cudaGetLastError());
+    if (l.Bs != nullptr) {
+      const int bn = pt_tile(l.cout), gj = pt_groups(l.cin), st = pt_steps(l.cin);
+      pt_pack_stages_kernel<<<grid1((long long)st * (bn / 8) * gj * (PT_CORE / 16), 256), 256, 0, s>>>(
+          l.B, 2 * l.n4(), PT_PATHS * l.cin, bn, gj, st, reinterpret_cast<uint4*>(l.Bs));
+      TSM_CUDA(cudaGetLastError());
+    }
   }
   packed = true;
   return TSM_OK;
 }
+
+namespace {
+
+// one layer, transports and channel mixing fused (up to 32 output channels)
+template <int BN>
+int layer_launch(Ctx& c, const NetGeom& ng, const NetLayer& l, const float* X, int nb, float* Y, int* err) {
+  const int gj = pt_groups(l.cin), steps = pt_steps(l.cin), smem = pt_layer_smem<BN>(gj);
+  TSM_CUDA(cudaFuncSetAttribute(pt_layer_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  pt_layer_kernel<BN><<<dim3(grid1(c.g.V, PT_SITES), nb), 256, smem, c.stream>>>(ng, X, l.cin, l.Bs, 8 * l.cout, Y, gj,
+                                                                                 steps, err);
+  return check_net_launch(c, "pt_layer_kernel");
+}
+
+int launch_layer(Ctx& c, const NetGeom& ng, const NetLayer& l, const float* X, int nb, float* Y, int* err) {
+  switch (pt_tile(l.cout)) {
+    case 16: return layer_launch<16>(c, ng, l, X, nb, Y, err);
+    case 64: return layer_launch<64>(c, ng, l, X, nb, Y, err);
+    case 96: return layer_launch<96>(c, ng, l, X, nb, Y, err);
+    case 128: return layer_launch<128>(c, ng, l, X, nb, Y, err);
+    case 192: return layer_launch<192>(c, ng, l, X, nb, Y, err);
+    default: return layer_launch<256>(c, ng, l, X, nb, Y, err);
+  }
+}
+
+}  // namespace
 
 int Net::forward(Ctx& c, const float* X0, int nb, float** out) {
   TSM_TRY(reserve(c.g.V, nb));
@@ -211,11 +243,17 @@ int Net::forward(Ctx& c, const float* X0, int nb, float** out) {
   for (size_t li = 0; li < layers.size(); ++li) {
     const NetLayer& l = layers[li];
     const int K2 = 72 * l.cin, N2 = 8 * l.cout;
-    pt_gather_kernel<<<dim3(grid1((long long)V * PT_PATHS * l.cin, NET_NT), nb), NET_NT, 0, c.stream>>>(ng, X, l.cin,
-                                                                                                        Z);
-    TSM_TRY(check_net_launch(c, "pt_gather_kernel"));
-    TSM_TRY(launch_umma_gemm_ex(c.stream, Z, K2, l.B, K2, acts[li + 1], N2, M, N2, K2, 0, 1, d_err, nullptr));
-    TSM_TRY(check_net_launch(c, "umma_gemm_kernel"));
+    // fused up to one tile of 256 columns (figures at pt_layer_kernel); wider
+    // layers gather Z once and multiply it tile by tile
+    if (l.Bs != nullptr) {
+      TSM_TRY(launch_layer(c, ng, l, X, nb, acts[li + 1], d_err));
+    } else {
+      pt_gather_kernel<<<dim3(grid1((long long)V * PT_PATHS * l.cin, NET_NT), nb), NET_NT, 0, c.stream>>>(
+          ng, X, l.cin, Z);
+      TSM_TRY(check_net_launch(c, "pt_gather_kernel"));
+      TSM_TRY(launch_umma_gemm_ex(c.stream, Z, K2, l.B, K2, acts[li + 1], N2, M, N2, K2, 0, 1, d_err, nullptr));
+      TSM_TRY(check_net_launch(c, "umma_gemm_kernel"));
+    }
     X = acts[li + 1];
   }
   *out = acts[layers.size()];
@@ -283,6 +321,7 @@ void Net::free_all() {
     dfree(l.vi);
     dfree(l.B);
     dfree(l.Bt);
+    dfree(l.Bs);
   }
   for (PairGroup& g : groups) {
     dfree(g.R);
@@ -435,6 +474,8 @@ extern "C" int tsm_net_create(int device, int n_layers, const int* channels, uin
       if (rc == TSM_OK) rc = dalloc(a, cnt);
     if (rc == TSM_OK) rc = dalloc(&l.B, 4 * cnt);
     if (rc == TSM_OK) rc = dalloc(&l.Bt, 4 * cnt);
+    if (rc == TSM_OK && pt_tile(l.cout) > 0)
+      rc = dalloc(&l.Bs, (size_t)pt_steps(l.cin) * (pt_tile(l.cout) / 8) * pt_groups(l.cin) * PT_CORE);
     if (rc != TSM_OK) break;
     for (float** a : arrs)
       if (*a != l.wr && *a != l.wi && cudaMemset(*a, 0, cnt * sizeof(float)) != cudaSuccess) rc = TSM_ERR_CUDA;

@@ -24,6 +24,7 @@ struct NetLayer {
   float *gr = nullptr, *gi = nullptr;      // gradient accumulators
   float *mr = nullptr, *vr = nullptr, *mi = nullptr, *vi = nullptr;   // Adam moments
   __nv_bfloat16 *B = nullptr, *Bt = nullptr;   // packed block weights [8 cout][72 cin] and transpose
+  uint8_t* Bs = nullptr;   // the same, stage by stage for pt_layer_kernel (null: more than 256 columns)
   int n4() const { return 4 * cout; }
   int k36() const { return 36 * cin; }
 };
