@@ -114,9 +114,11 @@ __global__ void __launch_bounds__(SITE_NT) unpack_spinor_kernel(Geom g, const ty
 // records the largest squared deviation from SU(3).  A block moves the links of
 // 64 consecutive sites through shared memory, so that the reads and the stores
 // of a direction run over consecutive sites.  Bound by the FP64 pipe: the check
-// takes 66 FP64 instructions per link (2.7 million links at 24^3x48); squares,
-// compared as integers, need no square root or FP64 comparison, and the
-// narrowing runs on the integer pipe.
+// takes 64 FP64 instructions per link, products as chains of multiply-adds (2.7
+// million links at 24^3x48: 290 us at two results per SM and clock; load_gauge
+// 732 -> 648 us against sums of separate products); squares, compared as
+// integers, need no square root or FP64 comparison, and the narrowing runs on
+// the integer pipe.
 constexpr int LINK_SITES = 64;
 
 static __global__ void __launch_bounds__(SITE_NT) pack_links_kernel(Geom g, const double2* __restrict__ U,
@@ -145,17 +147,23 @@ static __global__ void __launch_bounds__(SITE_NT) pack_links_kernel(Geom g, cons
     cx<double> r[9], w[3];
 #pragma unroll
     for (int k = 0; k < 9; ++k) r[k] = {m[k].x, m[k].y};
-    third_row(r, w);
+    // the reconstructed row 2, conj(row0 x row1), as chains of multiply-adds
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const cx<double> x = r[(k + 1) % 3], y = r[3 + (k + 2) % 3], u = r[(k + 2) % 3], v = r[3 + (k + 1) % 3];
+      w[k] = cconj(cmac(x * y, cx<double>{-u.re, -u.im}, v));
+    }
+    auto norm2_add = [](double acc, cx<double> a) { return fma(a.im, a.im, fma(a.re, a.re, acc)); };
     // SU(3) check: unit rows, orthogonal rows, stored row 2 equals the reconstruction
     auto worse = [&](double sq) {   // squares are non-negative: their bits order like the values, NaN on top
       const unsigned long long b = (unsigned long long)__double_as_longlong(sq) & 0x7fffffffffffffffull;
       dev2 = b > dev2 ? b : dev2;
     };
-    const double n0 = norm2(r[0]) + norm2(r[1]) + norm2(r[2]) - 1.0;
-    const double n1 = norm2(r[3]) + norm2(r[4]) + norm2(r[5]) - 1.0;
+    const double n0 = norm2_add(norm2_add(norm2_add(-1.0, r[0]), r[1]), r[2]);
+    const double n1 = norm2_add(norm2_add(norm2_add(-1.0, r[3]), r[4]), r[5]);
     worse(n0 * n0);
     worse(n1 * n1);
-    worse(norm2(cjmul(r[0], r[3]) + cjmul(r[1], r[4]) + cjmul(r[2], r[5])));
+    worse(norm2(cjmac(cjmac(cjmul(r[0], r[3]), r[1], r[4]), r[2], r[5])));
 #pragma unroll
     for (int k = 0; k < 3; ++k) worse(norm2(r[6 + k] - w[k]));
     const size_t off64 = (size_t)parity * 4 * F64::LN * lstride;
