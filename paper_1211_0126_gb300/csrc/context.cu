@@ -111,6 +111,20 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
   return fn;
 }
 
+int Ctx::staging(size_t bytes, void** out) {
+  TSM_CUDA(cudaStreamSynchronize(stream));
+  if (bytes > h_stage_bytes) {
+    if (h_stage) cudaFreeHost(h_stage);
+    h_stage = nullptr;
+    h_stage_bytes = 0;
+    const size_t want = bytes < (64u << 10) ? (64u << 10) : bytes;
+    TSM_CUDA(cudaMallocHost(&h_stage, want));
+    h_stage_bytes = want;
+  }
+  *out = h_stage;
+  return TSM_OK;
+}
+
 int Ctx::check_waits() {
   volatile int* e = h_err;
   if (e == nullptr || *e == 0) return TSM_OK;
@@ -127,6 +141,9 @@ void Ctx::free_all() {
   links_base = nullptr;
   for (void*& l : links) l = nullptr;
   h_err = nullptr;   // lives behind h_states
+  if (h_stage) cudaFreeHost(h_stage);
+  h_stage = nullptr;
+  h_stage_bytes = 0;
   if (red.partials) cudaFree(red.partials);
   if (red.counter) cudaFree(red.counter);
   if (red_branch.partials) cudaFree(red_branch.partials);

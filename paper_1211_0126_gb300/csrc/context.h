@@ -67,6 +67,8 @@ struct Ctx {
   void* links[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
   void* links_base = nullptr;   // their allocation
   int sm_count = 1;
+  void* h_stage = nullptr;              // see staging()
+  size_t h_stage_bytes = 0;
   int* h_err = nullptr;                 // pinned, device-visible: set by a kernel whose bounded wait ran out
   std::map<std::string, std::pair<void*, size_t>> ws;      // named device workspace
   RedSlot red{};
@@ -128,6 +130,7 @@ struct Ctx {
   }
   int field(const std::string& name, int prec, PField* f, int nrhs = 1);   // nrhs parity fields of tier prec
   int harvest_events();                                        // sync + accumulate profile times
+  int staging(size_t bytes, void** out);   // pinned host buffer, kept and grown; waits for the copies out of it
   int check_waits();   // after a stream sync: TSM_ERR_TIMEOUT if a kernel's bounded wait ran out since the last check
   void free_all();
 };

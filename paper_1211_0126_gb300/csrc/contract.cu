@@ -155,33 +155,34 @@ int ContractPlan::prepare(Ctx& c, const int* gammas, int n_gamma, const int* mom
     TSM_TRY(group_momenta(L, moms + 3 * q0, std::min(CT_MAXQ, n_q - q0), &m));
     passes.push_back(m);
   }
-  std::vector<double2> tab((size_t)n_q * (L[0] + L[1] + L[2]));
+  // tables in FP64 and rounded once to FP32, written into the context's pinned
+  // staging buffer: one asynchronous copy, in order with the launches
+  const size_t n_tab = (size_t)n_q * (L[0] + L[1] + L[2]);
+  const size_t bytes = n_tab * (sizeof(double2) + sizeof(float2));
+  void *host = nullptr, *dev = nullptr;
+  TSM_TRY(c.staging(bytes, &host));
+  double2* tab = static_cast<double2*>(host);
+  float2* ftab = reinterpret_cast<float2*>(tab + n_tab);
   const double twopi = 2.0 * std::acos(-1.0);
   size_t off = 0;
   for (int ax = 0; ax < 3; ++ax)
-    for (int q = 0; q < n_q; ++q)
-      for (int x = 0; x < L[ax]; ++x) {
+    for (int q = 0; q < n_q; ++q) {
+      const long long n = moms[3 * q + ax];
+      for (int x = 0; x < L[ax]; ++x, ++off) {
         // reduce n*x mod L exactly in integers before the angle is formed
-        long long nx = (long long)moms[3 * q + ax] * x;
-        nx %= L[ax];
+        long long nx = (n * x) % L[ax];
         if (nx < 0) nx += L[ax];
         const double ang = twopi * (double)nx / (double)L[ax];
-        tab[off++] = make_double2(std::cos(ang), std::sin(ang));
+        tab[off] = nx == 0 ? make_double2(1.0, 0.0) : make_double2(std::cos(ang), std::sin(ang));
+        ftab[off] = make_float2((float)tab[off].x, (float)tab[off].y);
       }
-  void* dev = nullptr;
-  TSM_TRY(c.buffer("phase_tab", tab.size() * sizeof(double2), &dev));
-  TSM_CUDA(cudaMemcpyAsync(dev, tab.data(), tab.size() * sizeof(double2), cudaMemcpyHostToDevice, c.stream));
-  TSM_CUDA(cudaStreamSynchronize(c.stream));
+    }
+  TSM_TRY(c.buffer("phase_tab", bytes, &dev));
+  TSM_CUDA(cudaMemcpyAsync(dev, host, bytes, cudaMemcpyHostToDevice, c.stream));
   phx = static_cast<double2*>(dev);
   phy = phx + (size_t)n_q * L[0];
   phz = phy + (size_t)n_q * L[1];
-  std::vector<float2> ftab(tab.size());
-  for (size_t k = 0; k < tab.size(); ++k) ftab[k] = make_float2((float)tab[k].x, (float)tab[k].y);
-  void* fdev = nullptr;
-  TSM_TRY(c.buffer("phase_tab_f32", ftab.size() * sizeof(float2), &fdev));
-  TSM_CUDA(cudaMemcpyAsync(fdev, ftab.data(), ftab.size() * sizeof(float2), cudaMemcpyHostToDevice, c.stream));
-  TSM_CUDA(cudaStreamSynchronize(c.stream));
-  fphx = static_cast<float2*>(fdev);
+  fphx = reinterpret_cast<const float2*>(phx + n_tab);
   fphy = fphx + (size_t)n_q * L[0];
   fphz = fphy + (size_t)n_q * L[1];
   return TSM_OK;
@@ -364,7 +365,7 @@ int reserve_contract(Ctx& c) {
 int launch_combine(Ctx& c, const double2* corr, int n_hp, const double2* lp, int n_lp, int E, double2* est,
                    double* err, double2* lp_mean, double2* corr_mean) {
   if (E <= 0) return TSM_OK;
-  combine_kernel<<<(E + 127) / 128, 128, 0, c.stream>>>(corr, n_hp, lp, n_lp, E, est, err, lp_mean, corr_mean);
+  combine_kernel<<<(E + 31) / 32, 32, 0, c.stream>>>(corr, n_hp, lp, n_lp, E, est, err, lp_mean, corr_mean);
   c.launches++;
   return check_launch(c, "combine_kernel");
 }

@@ -596,6 +596,46 @@ contract_reduce_kernel(const double2* __restrict__ partial, size_t pstride, int 
   }
 }
 
+// sum over the sources of one entry's values, and of their squared distances
+// from m, in source order with eight loads in flight (the plain loop's bits)
+__device__ __forceinline__ void entry_sum(const double2* __restrict__ v, int n, int E, double& re, double& im) {
+  int j = 0;
+  for (; j + 8 <= n; j += 8) {
+    double2 b[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) b[u] = v[(size_t)(j + u) * E];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      re += b[u].x;
+      im += b[u].y;
+    }
+  }
+  for (; j < n; ++j) {
+    re += v[(size_t)j * E].x;
+    im += v[(size_t)j * E].y;
+  }
+}
+__device__ __forceinline__ double entry_spread(const double2* __restrict__ v, int n, int E, double mr, double mi) {
+  double s = 0.0;
+  int j = 0;
+  for (; j + 8 <= n; j += 8) {
+    double2 b[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) b[u] = v[(size_t)(j + u) * E];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const double dr = b[u].x - mr, di = b[u].y - mi;
+      s += dr * dr + di * di;
+    }
+  }
+  for (; j < n; ++j) {
+    const double2 b = v[(size_t)j * E];
+    const double dr = b.x - mr, di = b.y - mi;
+    s += dr * dr + di * di;
+  }
+  return s;
+}
+
 // Eq. 2.4 per entry: mean of the corrections + mean of the LP set; error from
 // the unbiased complex sample variances, two passes in source order.
 static __global__ void combine_kernel(const double2* __restrict__ corr, int n_hp, const double2* __restrict__ lp, int n_lp,
@@ -605,40 +645,16 @@ static __global__ void combine_kernel(const double2* __restrict__ corr, int n_hp
   if (e >= E) return;
   double mcr = 0.0, mci = 0.0, mlr = 0.0, mli = 0.0, var = 0.0;
   if (n_hp > 0) {
-    for (int j = 0; j < n_hp; ++j) {
-      const double2 v = corr[(size_t)j * E + e];
-      mcr += v.x;
-      mci += v.y;
-    }
+    entry_sum(corr + e, n_hp, E, mcr, mci);
     mcr /= n_hp;
     mci /= n_hp;
-    if (n_hp > 1) {
-      double s = 0.0;
-      for (int j = 0; j < n_hp; ++j) {
-        const double2 v = corr[(size_t)j * E + e];
-        const double dr = v.x - mcr, di = v.y - mci;
-        s += dr * dr + di * di;
-      }
-      var += s / (n_hp - 1) / n_hp;
-    }
+    if (n_hp > 1) var += entry_spread(corr + e, n_hp, E, mcr, mci) / (n_hp - 1) / n_hp;
   }
   if (n_lp > 0) {
-    for (int j = 0; j < n_lp; ++j) {
-      const double2 v = lp[(size_t)j * E + e];
-      mlr += v.x;
-      mli += v.y;
-    }
+    entry_sum(lp + e, n_lp, E, mlr, mli);
     mlr /= n_lp;
     mli /= n_lp;
-    if (n_lp > 1) {
-      double s = 0.0;
-      for (int j = 0; j < n_lp; ++j) {
-        const double2 v = lp[(size_t)j * E + e];
-        const double dr = v.x - mlr, di = v.y - mli;
-        s += dr * dr + di * di;
-      }
-      var += s / (n_lp - 1) / n_lp;
-    }
+    if (n_lp > 1) var += entry_spread(lp + e, n_lp, E, mlr, mli) / (n_lp - 1) / n_lp;
   }
   if (est) est[e] = make_double2(mcr + mlr, mci + mli);
   if (err) err[e] = sqrt(var);
