@@ -58,7 +58,7 @@ def parse():
     ap.add_argument("--no-extras", action="store_true", help="skip e2e / equal-error / cpu-baseline legs")
     ap.add_argument("--batch", type=int, default=None,
                     help="sources solved together (multi-RHS kernels); default: the autotuner's choice (tsm_tune: "
-                         "batch width and sources per link-sharing block of the FP16 stencil)")
+                         "batch width)")
     ap.add_argument("--reliable-delta", type=float, default=None, help="override the HP reliable-update delta")
     ap.add_argument("--hp-warm-start", action="store_true",
                     help="HP solves start from their source's LP solution instead of zero")
@@ -515,7 +515,7 @@ def tune_table(tsm, times):
 
 def kernel_source_hash():
     h = hashlib.sha256()
-    for f in ("dslash.cuh", "common.cuh"):
+    for f in ("mma_hop.cuh", "common.cuh"):
         with open(os.path.join(ROOT, "paper_1211_0126_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]

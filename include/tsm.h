@@ -81,7 +81,10 @@ typedef enum {
  *   TSM_BF16, TSM_F16  16-bit storage of links and Krylov/operator vectors,
  *            FP32 arithmetic.  TSM_F16 keeps the CG residual and iterate in
  *            FP16 as well (relative precision 2^-11, below the truncation of
- *            an LP solve); TSM_BF16 keeps them in FP32.  Sources and solutions
+ *            an LP solve) and solves in groups of 8 sources on the tensor
+ *            cores (FP16 products, FP32 sums): a group costs the same however
+ *            few of its sources are used, so batches of a multiple of 8 pay
+ *            most; TSM_BF16 keeps them in FP32.  Sources and solutions
  *            are exchanged in FP32 for both through tm_solve_batch; inside
  *            tsm_loops / tsm_loops_graph the TSM_F16 tier also keeps its noise
  *            source, Schur source and solution in FP16 (the solution is FP16
@@ -253,7 +256,7 @@ typedef struct {
   uint32_t lp_begin, lp_end;
   tm_stop hp;               /* stopping rule / tier of the HP solves */
   tm_stop lp;               /* stopping rule / tier of the LP solves (same map for both sets) */
-  int batch;                /* sources solved together (>= 1; 1 = single-RHS kernels) */
+  int batch;                /* sources solved together (>= 1; FP16 LP solves round it up to a multiple of 8) */
   const int* gammas; int n_gamma;
   const int* moms; int n_q; /* host pointers */
   int verify;               /* 1: recompute every HP solution's true residual in FP64
@@ -321,7 +324,7 @@ int tsm_loops_graph(tsm_ctx** ctxs, const tsm_params* params, int n, double** lo
 int tsm_tune_batch(tsm_ctx* ctx, const tm_stop* stop, int* best, double* times_ms);
 
 /* Autotuner of the whole multi-RHS launch shape: the batch width as above
- * and, for the 16-bit tiers and FP32, the block shape of their link-sharing
+ * and, for BF16 and FP32, the block shape of their link-sharing
  * stencil (blocks of 32 sites x 2, 4 or 8 sources, one warp per source; the
  * block's links are widened once and shared; FP32 uses it for its hops
  * without a reduction), the 4-source blocks compiled for either 80 or 96
@@ -335,14 +338,16 @@ int tsm_tune_batch(tsm_ctx* ctx, const tm_stop* stop, int* best, double* times_m
  * per context, lattice and stopping rule.  times_ms (may be NULL): 16 entries,
  * [width k][shape q] = ms per source for widths {8, 16, 32, 64} and shapes
  * {2 sources / 80 registers, 4 / 80, 8 / 80, 4 / 96} (0 where a shape does not
- * apply).  tsm_tune_batch runs the same search and reports, per width, the best
+ * apply; TSM_F16, whose blocks are fixed, is timed once per width and reports
+ * that time for every shape).  tsm_tune_batch runs the same search and reports, per width, the best
  * time over the shapes. */
 int tsm_tune(tsm_ctx* ctx, const tm_stop* stop, int* best_batch, int* best_tile, int* best_regs, double* times_ms);
 
 /* Set the block shape of the link-sharing stencil of tier prec (TSM_F16,
  * TSM_BF16 or TSM_F32) for this context's later solves, as tsm_tune does:
  * tile_sources 2, 4 or 8 sources per block, max_regs 80 (or 96 with 4
- * sources); 4 and 80 by default.  TSM_ERR_ARG for other tiers or values. */
+ * sources); 4 and 80 by default.  TSM_F16 accepts the call and is unaffected
+ * by it.  TSM_ERR_ARG for other tiers or values. */
 int tsm_set_tile(tsm_ctx* ctx, int prec, int tile_sources, int max_regs);
 
 

@@ -415,7 +415,7 @@ def tsm_tune(h, stp):
     """Autotuned launch shape for the loaded lattice and tier: returns (best
     batch width, best sources per link-sharing block, its register budget,
     per-source ms [4][4] for widths 8, 16, 32, 64 x the block shapes of
-    TILE_SHAPES)."""
+    TILE_SHAPES; the FP16 tier's blocks are fixed, one time stands for all)."""
     best = ctypes.c_int(0)
     tile = ctypes.c_int(0)
     regs = ctypes.c_int(0)
