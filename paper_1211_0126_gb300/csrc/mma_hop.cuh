@@ -32,10 +32,10 @@
 // share an accumulator each.
 //
 // Neighbours reach the warps through shared memory: a block works on tiles of
-// 2 x 2 rows (y, z) of up to 4 half-sites in x, one site per warp, and four
-// more warps copy the tile's distinct neighbour sites (92 instead of 8 x 16) for one
-// group of 8 sources per ring stage with TMA: the own rows as one box of
-// (4 + 2) x 2 x 2 sites, the y, z and t edges as two boxes each, and the sites
+// 2 x 2 rows (y, z) of up to W = 4 or 6 half-sites in x, one site per warp, and four
+// more warps copy the tile's distinct neighbour sites (92 instead of 8 x 16 at W = 4) for
+// one group of 8 sources per ring stage with TMA: the own rows as one box of
+// (W + 2) x 2 x 2 sites, the y, z and t edges as two boxes each, and the sites
 // that wrap around in x (at most 4, where a box has zeros) as plain bulk copies.
 // The centre fields of the epilogues arrive in the same stage.
 #pragma once
@@ -47,32 +47,40 @@
 
 namespace tsm {
 
-constexpr int MMA_WARPS = 16;                        // consumer warps = sites of a tile
 constexpr int MMA_COPIERS = 4;                       // copy warps (one thread each)
-constexpr int MMA_NT = 32 * (MMA_WARPS + MMA_COPIERS);
-constexpr int MMA_W = 4;                             // half-sites in x of a tile at most
 constexpr int MMA_GROUPS = 8;                        // groups of 8 sources of a batch at most
 constexpr int MMA_FLUSH = 8;                         // tiles whose norms add up in FP32 before they join the FP64 sum
 constexpr int MMA_CHUNKS = 24;                       // 16-byte chunks per site of a group
 constexpr long long MMA_SPIN_LIMIT = 1ll << 22;      // polls of a ring wait
 
-// slots (sites) of a ring stage: the own rows [zz][yy][6] from x0 - 1 on (the
-// sites x +- 1 of the other parity; they are also the y and z neighbours inside
-// the tile), the wrapped site of each row, the edges [e][row][4] in y, z and t,
-// then the rows [zz][yy][4] of the centre fields
-constexpr int MMA_SLOT_WRAP = 24, MMA_SLOT_Y = 28, MMA_SLOT_Z = 44, MMA_SLOT_T = 60, MMA_SLOT_F = 92;
+// A tile of 2 x 2 rows of W half-sites: a warp per site and the copy warps (one
+// thread each).  Slots (sites) of a ring stage: the own rows [zz][yy][W + 2] from
+// x0 - 1 on (the sites x +- 1 of the other parity; they are also the y and z
+// neighbours inside the tile), the wrapped site of each row, the edges
+// [e][row][W] in y, z and t, then the rows [zz][yy][W] of the centre fields.
+template <int TW> struct MmaShape {
+  static constexpr int W = TW, WARPS = 4 * W, NT = 32 * (WARPS + MMA_COPIERS);
+  static constexpr int WRAP = 4 * (W + 2), Y = WRAP + 4, Z = Y + 4 * W, T = Z + 4 * W, F = T + 8 * W;
+  static constexpr bool LINKS_SMEM = W > 4;   // the next tile's link words wait in shared memory instead of registers
+  static constexpr int LINK_BYTES = LINKS_SMEM ? WARPS * 96 * 4 : 0;
+};
 
-// box shapes (x, y, z sites) of the tensor maps
+// box shapes (x, y, z sites) of the tensor maps of a shape
 enum MmaBox { MMA_BOX_OWN = 0, MMA_BOX_Y = 1, MMA_BOX_Z = 2, MMA_BOX_TILE = 3, MMA_BOXES = 4 };
-constexpr int kMmaBox[MMA_BOXES][3] = {{6, 2, 2}, {4, 1, 2}, {4, 2, 1}, {4, 2, 2}};
+inline void mma_box(int k, int w, int box[3]) {
+  box[0] = k == MMA_BOX_OWN ? w + 2 : w;
+  box[1] = k == MMA_BOX_Y ? 1 : 2;
+  box[2] = k == MMA_BOX_Z ? 1 : 2;
+}
 
 enum { MMA_HOP = 0, MMA_HOP_CENTER = 1, MMA_HOP_CENTER_NORM = 3, MMA_UPDATE = 8 };
 
-template <int MODE> struct MmaStage {
+template <int MODE, class SH> struct MmaStage {
   static constexpr int FIELDS = MODE == MMA_HOP ? 0 : MODE == MMA_UPDATE ? 4 : 1;
-  static constexpr int SLOTS = MMA_SLOT_F + 16 * FIELDS;
+  static constexpr int SLOTS = SH::F + 4 * SH::W * FIELDS;
   static constexpr int BYTES = SLOTS * MMA_CHUNKS * 16;
-  static constexpr int COUNT = MODE == MMA_HOP ? 5 : MODE == MMA_UPDATE ? 3 : 4;
+  static constexpr int COUNT = (MODE == MMA_HOP ? 5 : MODE == MMA_UPDATE ? 3 : 4) - (SH::W > 4);
+  static constexpr int SMEM = BYTES * COUNT + SH::LINK_BYTES;
 };
 
 // tiles of a lattice: ntx x nyp x nzp x T, x fastest; gx .. gt: the grid's
@@ -219,7 +227,7 @@ struct MmaSlots {
 // H psi (or H^dag psi) of one site for 8 sources: nb points at the lane's chunk
 // of the stage.
 // acc: four spins of colour q (lanes q = 3: the lo part of colour 2)
-template <int DAG>
+template <int DAG, int W>
 __device__ __forceinline__ void mma_site(const uint4* nb, const MmaSlots& sl, const uint32_t (&B)[4][2],
                                          const uint32_t (&BL)[4][2], float (&acc)[8]) {
   constexpr int SF = DAG ? +1 : -1;
@@ -241,7 +249,7 @@ __device__ __forceinline__ void mma_site(const uint4* nb, const MmaSlots& sl, co
   mma_f16(yb, a, BL[2][0], BL[2][1]);      // rows: spin 2 | -spin 3
   yb[2] = -yb[2];
   yb[3] = -yb[3];
-  project_word<3, SF>((nb + sl.t)[16 * MMA_CHUNKS], a[0], a[1]);
+  project_word<3, SF>((nb + sl.t)[4 * W * MMA_CHUNKS], a[0], a[1]);
   project_word<3, -SF>(nb[sl.t], a[2], a[3]);
   mma_f16(up, a, B[3][0], B[3][1]);
   mma_f16(yb, a, BL[3][0], BL[3][1]);      // rows: spin 2 | spin 3
@@ -293,18 +301,25 @@ __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap* map
       : "memory");
 }
 
-// Bound by instruction issue (about 200 warp instructions per site and group of
-// 8 sources, issue slots 67 % busy with 16 + 4 warps of 96 registers; HMMA 17 %)
-// for K1 and K3, by HBM for K4.  Measured at 24^3x48 with 32 sources against the
-// FP32 FMA stencil it replaced (1727 thread instructions per source-site): K1
-// 575 -> 370 us, K2 690 -> 477, K3 574 -> 368, K4 849 -> 614 (5.9 TB/s); with
-// one group of 8: K1 152 -> 139, K2 199 -> 174, K4 233 -> 196.  A group costs the
-// same however few of its 8 rows are used (4 sources: K1 83 -> 139 us), but a
-// source's bits must not depend on its batch, so every FP16 solve runs here and
-// the loop estimators fill whole groups.  Tried on the way: neighbours loaded
+// K4 is bound by HBM.  K1-K3 are bound within the SM, by no single unit: copies
+// and stores alone take 192 us where K1 takes 290, arithmetic on resident data
+// alone 291 (24^3x48, 24 sources, W = 4); issue slots 67 % busy, shared-memory
+// wavefronts 55 % and the copies' writes beside them, HMMA 19 %, in chains of 1350
+// cycles a site and group that four warps per scheduler overlap.  W = 6 has six
+// (24 + 4 warps at 72 registers: the next link words wait in shared memory, the lane
+// constants are formed per tile) and fewer neighbour sites per output site (5.5
+// against 5.75).  24^3x48, 32 sources: K1 370 -> 349 us, K2 473 -> 463; 12^3x24 (3
+// half-sites of a W = 4 tile used): K1 42.8 -> 35.0, K2 56.6 -> 48.6.  Against
+// the FP32 FMA stencil that these kernels replaced (1727 thread instructions per
+// source-site), 24^3x48, 32 sources: K1 575, K2 690, K3 574, K4 849 -> 614 (5.9
+// TB/s); with one group of 8: K1 152 -> 139, K2 199 -> 171, K4 233 -> 194.  A group
+// costs the same however few of its 8 rows are used (4 sources: K1 83 -> 139 us),
+// but a source's bits must not depend on its batch, so every FP16 solve runs here
+// and the loop estimators fill whole groups.  Tried on the way: neighbours loaded
 // from L2 by each warp one item ahead (K1 560 us, latency-bound at 39 % issue),
 // bulk copies of rows issued by one warp (676 us, the copy warp set the pace) and
-// by four (375 us), all boxes issued by one thread (485 us).
+// by four (375 us), all boxes issued by one thread (485 us), W = 6 with two copy
+// warps (356).
 //
 // K1-K4 of the FP16 tier: persistent blocks, block b takes the tiles b, b +
 // gridDim.y, ... and walks the live groups of 8 sources of each with the site's
@@ -313,20 +328,21 @@ __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap* map
 // batch.
 //   MODE MMA_HOP*:   out = ts q, q = to_ah H in + to_tc_ac center; <q, q> with NORM
 //   MODE MMA_UPDATE: v = A(-mu) w - kappa^2 H in, r -= alpha v, x += alpha p; <r, r>
-template <int DAG, int MODE>
-__global__ void __launch_bounds__(MMA_NT, 1) mma_hop_kernel(const MmaHopArgs a, const __grid_constant__ MmaMaps maps) {
+template <int DAG, int MODE, int W>
+__global__ void __launch_bounds__(MmaShape<W>::NT, 1) mma_hop_kernel(const MmaHopArgs a, const __grid_constant__ MmaMaps maps) {
   constexpr bool NORM = MODE == MMA_HOP_CENTER_NORM || MODE == MMA_UPDATE;
   constexpr bool CENTER = MODE != MMA_HOP;
   constexpr bool UPD = MODE == MMA_UPDATE;
-  using ST = MmaStage<MODE>;
+  using SH = MmaShape<W>;
+  using ST = MmaStage<MODE, SH>;
   extern __shared__ __align__(128) uint4 mma_ring[];
   __shared__ __align__(8) uint64_t s_full[ST::COUNT], s_empty[ST::COUNT];
   __shared__ unsigned long long s_mask;
   __shared__ int s_grp[MMA_GROUPS], s_timeout, s_issued;
   __shared__ size_t s_goff[MMA_GROUPS];   // chunk offset of each live group
   __shared__ float s_alpha[UPD ? MMA_GROUPS * 8 : 1];
-  __shared__ float s_part[NORM ? MMA_WARPS : 1][MMA_GROUPS][32];
-  __shared__ double s_sum[NORM ? MMA_WARPS : 1][MMA_GROUPS][8];
+  __shared__ float s_part[NORM ? SH::WARPS : 1][MMA_GROUPS][32];
+  __shared__ double s_sum[NORM ? SH::WARPS : 1][MMA_GROUPS][8];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = lane & 3, row = lane >> 2;
   const int qc = q < 3 ? q : 2;
   if (threadIdx.x == 0) {
@@ -336,12 +352,12 @@ __global__ void __launch_bounds__(MMA_NT, 1) mma_hop_kernel(const MmaHopArgs a, 
 #pragma unroll
     for (int i = 0; i < ST::COUNT; ++i) {
       mbar_init(&s_full[i], 1);
-      mbar_init(&s_empty[i], MMA_WARPS);
+      mbar_init(&s_empty[i], SH::WARPS);
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if constexpr (NORM) {
-    if (warp < MMA_WARPS)
+    if (warp < SH::WARPS)
       for (int j = 0; j < MMA_GROUPS; ++j) {
         s_part[warp][j][lane] = 0.f;
         if (lane < 8) s_sum[warp][j][lane] = 0.0;
@@ -370,10 +386,10 @@ __global__ void __launch_bounds__(MMA_NT, 1) mma_hop_kernel(const MmaHopArgs a, 
     }
   __syncthreads();
   const int ntile = a.tl.ntiles;
-  if (warp >= MMA_WARPS) {
+  if (warp >= SH::WARPS) {
     // ---- copy warps: one thread of each issues every fourth box of a stage (a
     // box costs its thread about 150 cycles; one thread alone set the pace)
-    const int copier = warp - MMA_WARPS;
+    const int copier = warp - SH::WARPS;
     if (lane == 0) {
       const MmaTiles& g = a.tl;
       MmaTile tl(g, blockIdx.y);
@@ -395,27 +411,28 @@ __global__ void __launch_bounds__(MMA_NT, 1) mma_hop_kernel(const MmaHopArgs a, 
           const int tg = g.T * s_grp[j];
           // rows whose output sites start even (s = 0) wrap on the left, the others on the right
           const int wraps = (left ? 2 : 0) + (right ? 2 : 0);
-          if (copier == 0) mbar_expect_tx(bar, (uint32_t)((88 + wraps + 16 * ST::FIELDS) * MMA_CHUNKS * 16));
+          if (copier == 0)
+            mbar_expect_tx(bar, (uint32_t)((SH::F - 4 + wraps + 4 * W * ST::FIELDS) * MMA_CHUNKS * 16));
           auto at = [&](int slot) { return dst + (uint32_t)(slot * MMA_CHUNKS * 16); };
           if (copier == 0) {
             tma_load_5d(at(0), &maps.in[MMA_BOX_OWN], x0 - 1, y0, z0, tg + t, bar);
-            tma_load_5d(at(MMA_SLOT_Y), &maps.in[MMA_BOX_Y], x0, ym, z0, tg + t, bar);
+            tma_load_5d(at(SH::Y), &maps.in[MMA_BOX_Y], x0, ym, z0, tg + t, bar);
           } else if (copier == 1) {
-            tma_load_5d(at(MMA_SLOT_Y + 8), &maps.in[MMA_BOX_Y], x0, yp, z0, tg + t, bar);
-            tma_load_5d(at(MMA_SLOT_Z), &maps.in[MMA_BOX_Z], x0, y0, zm, tg + t, bar);
+            tma_load_5d(at(SH::Y + 2 * W), &maps.in[MMA_BOX_Y], x0, yp, z0, tg + t, bar);
+            tma_load_5d(at(SH::Z), &maps.in[MMA_BOX_Z], x0, y0, zm, tg + t, bar);
           } else if (copier == 2) {
-            tma_load_5d(at(MMA_SLOT_Z + 8), &maps.in[MMA_BOX_Z], x0, y0, zp, tg + t, bar);
-            tma_load_5d(at(MMA_SLOT_T), &maps.in[MMA_BOX_TILE], x0, y0, z0, tg + tm, bar);
+            tma_load_5d(at(SH::Z + 2 * W), &maps.in[MMA_BOX_Z], x0, y0, zp, tg + t, bar);
+            tma_load_5d(at(SH::T), &maps.in[MMA_BOX_TILE], x0, y0, z0, tg + tm, bar);
           } else {
-            tma_load_5d(at(MMA_SLOT_T + 16), &maps.in[MMA_BOX_TILE], x0, y0, z0, tg + tp, bar);
-            if (ST::FIELDS == 1) tma_load_5d(at(MMA_SLOT_F), &maps.f[0], x0, y0, z0, tg + t, bar);
+            tma_load_5d(at(SH::T + 4 * W), &maps.in[MMA_BOX_TILE], x0, y0, z0, tg + tp, bar);
+            if (ST::FIELDS == 1) tma_load_5d(at(SH::F), &maps.f[0], x0, y0, z0, tg + t, bar);
           }
-          if (ST::FIELDS == 4) tma_load_5d(at(MMA_SLOT_F + 16 * copier), &maps.f[copier], x0, y0, z0, tg + t, bar);
+          if (ST::FIELDS == 4) tma_load_5d(at(SH::F + 4 * W * copier), &maps.f[copier], x0, y0, z0, tg + t, bar);
           if (wraps) {
             const int r = copier, s = (a.parity + r + (r >> 1) + t) & 1;
             if (s ? right : left) {
               const int rb = ((t * g.Lz + z0 + (r >> 1)) * g.Ly + y0 + (r & 1)) * g.Lxh;
-              bulk_load(at(MMA_SLOT_WRAP + r), a.in + s_goff[j] + (size_t)(rb + (s ? 0 : g.Lxh - 1)) * MMA_CHUNKS,
+              bulk_load(at(SH::WRAP + r), a.in + s_goff[j] + (size_t)(rb + (s ? 0 : g.Lxh - 1)) * MMA_CHUNKS,
                         MMA_CHUNKS * 16, bar);
             }
           }
@@ -430,19 +447,28 @@ __global__ void __launch_bounds__(MMA_NT, 1) mma_hop_kernel(const MmaHopArgs a, 
     }
   } else {
     // ---- one site of the tile per warp
-    const int r = warp >> 2, dx = warp & 3, yy = r & 1, zz = r >> 1;
-    const MmaLane L(lane);
-    uint32_t wr[8];   // the site's link words of this lane, fetched one tile ahead
+    const int r = warp / W, dx = warp % W, yy = r & 1, zz = r >> 1;
+    // the site's link words, fetched one tile ahead
+    uint32_t wr[8];
+    uint32_t* link_words = reinterpret_cast<uint32_t*>(reinterpret_cast<unsigned char*>(mma_ring) + ST::BYTES * ST::COUNT) + warp * 96;
+    const MmaLane L0(lane);
     auto site_of = [&](const MmaTile& tl) {
       return ((tl.t * a.tl.Lz + 2 * tl.zp + zz) * a.tl.Ly + 2 * tl.yp + yy) * a.tl.Lxh + tl.tx * a.tl.W + dx;
     };
     auto width = [&](const MmaTile& tl) { return min(a.tl.W, a.tl.Lxh - tl.tx * a.tl.W); };
     auto fetch_links = [&](int site) {
       const uint32_t* u = a.links + (size_t)site * 96;
+      if constexpr (SH::LINKS_SMEM) {
+        if (lane < 24)
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(link_words + 4 * lane)),
+                       "l"(u + 4 * lane)
+                       : "memory");
+      } else {
 #pragma unroll
-      for (int mu = 0; mu < 4; ++mu) {
-        wr[2 * mu] = __ldg(u + L.wf + 24 * mu);
-        wr[2 * mu + 1] = __ldg(u + L.wb + 24 * mu + 12);
+        for (int mu = 0; mu < 4; ++mu) {
+          wr[2 * mu] = __ldg(u + L0.wf + 24 * mu);
+          wr[2 * mu + 1] = __ldg(u + L0.wb + 24 * mu + 12);
+        }
       }
     };
     MmaTile tl(a.tl, blockIdx.y);
@@ -458,23 +484,41 @@ __global__ void __launch_bounds__(MMA_NT, 1) mma_hop_kernel(const MmaHopArgs a, 
     // chunk offsets in a stage that do not depend on the tile
     MmaSlots sl;
     {
-      const int iy = ((r ^ 1) * 6 + dx + 1) * MMA_CHUNKS, iz = ((r ^ 2) * 6 + dx + 1) * MMA_CHUNKS;   // inside the tile
-      const int ey = (MMA_SLOT_Y + yy * 8 + zz * 4 + dx) * MMA_CHUNKS, ez = (MMA_SLOT_Z + zz * 8 + yy * 4 + dx) * MMA_CHUNKS;
+      const int iy = ((r ^ 1) * (W + 2) + dx + 1) * MMA_CHUNKS, iz = ((r ^ 2) * (W + 2) + dx + 1) * MMA_CHUNKS;   // inside the tile
+      const int ey = (SH::Y + (2 * yy + zz) * W + dx) * MMA_CHUNKS, ez = (SH::Z + (2 * zz + yy) * W + dx) * MMA_CHUNKS;
       sl.yf = yy ? ey : iy;
       sl.yb = yy ? iy : ey;
       sl.zf = zz ? ez : iz;
       sl.zb = zz ? iz : ez;
-      sl.t = (MMA_SLOT_T + r * 4 + dx) * MMA_CHUNKS;
+      sl.t = (SH::T + r * W + dx) * MMA_CHUNKS;
     }
-    const int own = (r * 6 + dx) * MMA_CHUNKS, wrap = (MMA_SLOT_WRAP + r) * MMA_CHUNKS;
+    const int own = (r * (W + 2) + dx) * MMA_CHUNKS, wrap = (SH::WRAP + r) * MMA_CHUNKS;
     for (int tile = blockIdx.y; tile < ntile; tile += gridDim.y) {
       const bool more = tile + (int)gridDim.y < ntile;
       const int s = (a.parity + yy + zz + tl.t) & 1;
       uint32_t B[4][2], BL[4][2];
-      make_b<DAG, 0>(L, wr[0], wr[1], B[0], BL[0]);
-      make_b<DAG, 1>(L, wr[2], wr[3], B[1], BL[1]);
-      make_b<DAG, 2>(L, wr[4], wr[5], B[2], BL[2]);
-      make_b<DAG, 3>(L, wr[6], wr[7], B[3], BL[3]);
+      auto make = [&](const MmaLane& L) {
+        make_b<DAG, 0>(L, wr[0], wr[1], B[0], BL[0]);
+        make_b<DAG, 1>(L, wr[2], wr[3], B[1], BL[1]);
+        make_b<DAG, 2>(L, wr[4], wr[5], B[2], BL[2]);
+        make_b<DAG, 3>(L, wr[6], wr[7], B[3], BL[3]);
+      };
+      if constexpr (SH::LINKS_SMEM) {
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncwarp();
+        int ln = lane;
+        asm volatile("" : "+r"(ln));   // the lane constants are formed again: registers are short
+        const MmaLane L(ln);
+#pragma unroll
+        for (int mu = 0; mu < 4; ++mu) {
+          wr[2 * mu] = link_words[L.wf + 24 * mu];
+          wr[2 * mu + 1] = link_words[L.wb + 24 * mu + 12];
+        }
+        make(L);
+        __syncwarp();   // the words are read
+      } else {
+        make(L0);
+      }
       const int xh = tl.tx * a.tl.W + dx;
       sl.xf = s && xh + 1 == a.tl.Lxh ? wrap : own + (1 + s) * MMA_CHUNKS;
       sl.xb = !s && xh == 0 ? wrap : own + s * MMA_CHUNKS;
@@ -498,13 +542,13 @@ __global__ void __launch_bounds__(MMA_NT, 1) mma_hop_kernel(const MmaHopArgs a, 
         float acc[8];
         uint4 cw, pw, rw, xw;
         if (active) {
-          mma_site<DAG>(nb, sl, B, BL, acc);
-          const uint4* f = nb + (MMA_SLOT_F + r * 4 + dx) * MMA_CHUNKS;
+          mma_site<DAG, W>(nb, sl, B, BL, acc);
+          const uint4* f = nb + (SH::F + r * W + dx) * MMA_CHUNKS;
           if constexpr (CENTER) cw = f[0];
           if constexpr (UPD) {
-            pw = f[16 * MMA_CHUNKS];
-            rw = f[32 * MMA_CHUNKS];
-            xw = f[48 * MMA_CHUNKS];
+            pw = f[4 * W * MMA_CHUNKS];
+            rw = f[8 * W * MMA_CHUNKS];
+            xw = f[12 * W * MMA_CHUNKS];
           }
         }
         __syncwarp();
@@ -582,7 +626,7 @@ __global__ void __launch_bounds__(MMA_NT, 1) mma_hop_kernel(const MmaHopArgs a, 
     if (threadIdx.x < 64 && ((mask >> threadIdx.x) & 1ull)) {
       double s = 0.0;
 #pragma unroll
-      for (int w = 0; w < MMA_WARPS; ++w) s += s_sum[w][threadIdx.x >> 3][threadIdx.x & 7];
+      for (int w = 0; w < SH::WARPS; ++w) s += s_sum[w][threadIdx.x >> 3][threadIdx.x & 7];
       a.red.partials[(size_t)threadIdx.x * a.red.stride + blockIdx.y] = s;
       __threadfence();
     }

@@ -17,14 +17,14 @@ inline int groups_of(int nrhs) { return (nrhs + 7) / 8; }
 // tiles of the lattice and the persistent grid: one block per SM, never more
 // than there are tiles or partial slots (the grid fixes the reduction order, so
 // it depends on the lattice and the device alone)
-MmaHopArgs mma_args(const Ctx& c, int p_out, dim3* grid) {
+MmaHopArgs mma_args(const Ctx& c, int p_out, int w, dim3* grid) {
   MmaHopArgs m{};
   MmaTiles& t = m.tl;
   t.Lxh = c.g.Lxh;
   t.Ly = c.g.L[1];
   t.Lz = c.g.L[2];
   t.T = c.g.L[3];
-  t.ntx = blocks_for(t.Lxh, MMA_W);
+  t.ntx = blocks_for(t.Lxh, w);
   t.W = blocks_for(t.Lxh, t.ntx);
   t.nyp = t.Ly / 2;
   t.nzp = t.Lz / 2;
@@ -48,7 +48,9 @@ MmaHopArgs mma_args(const Ctx& c, int p_out, dim3* grid) {
 
 // tensor map of a grouped field: [T * groups][Lz][Ly][Lxh] sites of 384 bytes
 // (48 elements of 8), read in boxes of whole sites, zeros outside
-int make_map(const Ctx& c, CUtensorMap* m, const void* base, const int box[3]) {
+int make_map(const Ctx& c, CUtensorMap* m, const void* base, int kind, int w) {
+  int box[3];
+  mma_box(kind, w, box);
   PFN_cuTensorMapEncodeTiled_v12000 fn = tensor_map_encoder();
   const cuuint64_t dims[5] = {48, (cuuint64_t)c.g.Lxh, (cuuint64_t)c.g.L[1], (cuuint64_t)c.g.L[2],
                               (cuuint64_t)c.g.L[3] * MMA_GROUPS};
@@ -67,18 +69,33 @@ int make_map(const Ctx& c, CUtensorMap* m, const void* base, const int box[3]) {
   return TSM_OK;
 }
 
-int in_maps(const Ctx& c, MmaMaps* m, const void* in) {
-  for (int k = 0; k < MMA_BOXES; ++k) TSM_TRY(make_map(c, &m->in[k], in, kMmaBox[k]));
+int in_maps(const Ctx& c, MmaMaps* m, const void* in, int w) {
+  for (int k = 0; k < MMA_BOXES; ++k) TSM_TRY(make_map(c, &m->in[k], in, k, w));
   return TSM_OK;
 }
 
-template <int DAG, int MODE>
+template <int DAG, int MODE, int W>
 int mma_launch(Ctx& c, const MmaHopArgs& m, const MmaMaps& maps, dim3 grid) {
-  constexpr int smem = MmaStage<MODE>::BYTES * MmaStage<MODE>::COUNT;
-  TSM_CUDA(cudaFuncSetAttribute(mma_hop_kernel<DAG, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  (void)launch_pdl(c, mma_hop_kernel<DAG, MODE>, grid, dim3(MMA_NT), smem, m, maps);
+  using SH = MmaShape<W>;
+  constexpr int smem = MmaStage<MODE, SH>::SMEM;
+  TSM_CUDA(cudaFuncSetAttribute(mma_hop_kernel<DAG, MODE, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  (void)launch_pdl(c, mma_hop_kernel<DAG, MODE, W>, grid, dim3(SH::NT), smem, m, maps);
   c.launches++;
   return check_launch(c, "mma_hop_kernel");
+}
+
+// width of the hops' tiles in half-sites: 6, with 24 warps, where its tiles cover a
+// row with no more idle warps than those of 4 (Lx / 2 = 5, 6, 9 .. 12, ...), else 4,
+// with 16 (24^3x48 K1 349 against 370 us, 12^3x24 35.0 against 42.8; Lx / 2 = 8 would
+// leave a third of the warps idle).  The update (K4), bound by HBM, keeps 4: four
+// fields of a stage of 6 leave two stages, and its epilogue needs the registers.
+int mma_width(const Ctx& c) {
+  return 6 * blocks_for(c.g.Lxh, 6) <= 4 * blocks_for(c.g.Lxh, 4) ? 6 : 4;
+}
+
+template <int DAG, int MODE>
+int mma_hop(Ctx& c, const MmaHopArgs& m, const MmaMaps& maps, dim3 grid, int w) {
+  return w == 6 ? mma_launch<DAG, MODE, 6>(c, m, maps, grid) : mma_launch<DAG, MODE, 4>(c, m, maps, grid);
 }
 
 }  // namespace
@@ -93,12 +110,13 @@ int launch_hop<F16G>(Ctx& c, const HopArgs<F16G>& a0, int dag, int mode, int pro
     return TSM_ERR_ARG;
   }
   dim3 grid;
-  MmaHopArgs m = mma_args(c, a.p_out, &grid);
+  const int w = mma_width(c);
+  MmaHopArgs m = mma_args(c, a.p_out, w, &grid);
   m.in = a.in;
   m.out = a.out;
   MmaMaps maps;
-  TSM_TRY(in_maps(c, &maps, a.in));
-  if (mode & HOP_CENTER) TSM_TRY(make_map(c, &maps.f[0], a.center, kMmaBox[MMA_BOX_TILE]));
+  TSM_TRY(in_maps(c, &maps, a.in, w));
+  if (mode & HOP_CENTER) TSM_TRY(make_map(c, &maps.f[0], a.center, MMA_BOX_TILE, w));
   m.fto_ah = a.fto_ah;
   m.fto_tc_ac = a.fto_tc_ac;
   m.fts = a.fts;
@@ -112,11 +130,11 @@ int launch_hop<F16G>(Ctx& c, const HopArgs<F16G>& a0, int dag, int mode, int pro
   const double sb = spinor_site_bytes(F16::id), lb = link_site_bytes(F16::id);
   TimedLaunch tl(c, 4 * F16::id + kind, (double)a.g.Vh * (lb + nrhs * sb * (2 + ((mode & HOP_CENTER) ? 1 : 0))));
   int rc;
-  if (dag == 0 && mode == 0) rc = mma_launch<0, MMA_HOP>(c, m, maps, grid);
-  else if (dag == 0 && mode == HOP_CENTER) rc = mma_launch<0, MMA_HOP_CENTER>(c, m, maps, grid);
-  else if (dag == 0 && mode == (HOP_CENTER | HOP_NORM)) rc = mma_launch<0, MMA_HOP_CENTER_NORM>(c, m, maps, grid);
-  else if (dag == 1 && mode == 0) rc = mma_launch<1, MMA_HOP>(c, m, maps, grid);
-  else if (dag == 1 && mode == (HOP_CENTER | HOP_NORM)) rc = mma_launch<1, MMA_HOP_CENTER_NORM>(c, m, maps, grid);
+  if (dag == 0 && mode == 0) rc = mma_hop<0, MMA_HOP>(c, m, maps, grid, w);
+  else if (dag == 0 && mode == HOP_CENTER) rc = mma_hop<0, MMA_HOP_CENTER>(c, m, maps, grid, w);
+  else if (dag == 0 && mode == (HOP_CENTER | HOP_NORM)) rc = mma_hop<0, MMA_HOP_CENTER_NORM>(c, m, maps, grid, w);
+  else if (dag == 1 && mode == 0) rc = mma_hop<1, MMA_HOP>(c, m, maps, grid, w);
+  else if (dag == 1 && mode == (HOP_CENTER | HOP_NORM)) rc = mma_hop<1, MMA_HOP_CENTER_NORM>(c, m, maps, grid, w);
   else {
     set_error("grouped FP16 hop variant dag=%d mode=%d not built", dag, mode);
     return TSM_ERR_ARG;
@@ -129,12 +147,13 @@ template <>
 int launch_cg_update<F16G, F16G>(Ctx& c, const CGUpdArgs<F16G, F16G>& a, int nrhs) {
   if (a.g.Vh == 0 || nrhs == 0) return TSM_OK;
   dim3 grid;
-  MmaHopArgs m = mma_args(c, 0, &grid);
+  constexpr int w = 4;
+  MmaHopArgs m = mma_args(c, 0, w, &grid);
   m.in = a.t;
   MmaMaps maps;
-  TSM_TRY(in_maps(c, &maps, a.t));
+  TSM_TRY(in_maps(c, &maps, a.t, w));
   const void* fields[4] = {a.w, a.p, a.r, a.x};
-  for (int k = 0; k < 4; ++k) TSM_TRY(make_map(c, &maps.f[k], fields[k], kMmaBox[MMA_BOX_TILE]));
+  for (int k = 0; k < 4; ++k) TSM_TRY(make_map(c, &maps.f[k], fields[k], MMA_BOX_TILE, w));
   m.r = a.r;
   m.x = a.x;
   m.fto_tc_ac = to_float(a.tw);
@@ -147,7 +166,7 @@ int launch_cg_update<F16G, F16G>(Ctx& c, const CGUpdArgs<F16G, F16G>& a, int nrh
   m.red = a.red;
   const double sb = spinor_site_bytes(F16::id), lb = link_site_bytes(F16::id);
   TimedLaunch tl(c, 4 * F16::id + PK_HOP_UPDATE, (double)a.g.Vh * (lb + nrhs * 7 * sb));
-  const int rc = mma_launch<1, MMA_UPDATE>(c, m, maps, grid);
+  const int rc = mma_launch<1, MMA_UPDATE, w>(c, m, maps, grid);
   tl.done();
   return rc;
 }

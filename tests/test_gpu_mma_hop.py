@@ -52,3 +52,11 @@ def test_wide_batches_equal_single_solves(ctx, nrhs):
     for r in (0, 8, nrhs // 2, nrhs - 1):
         one, it, _, _ = ctx.solve(b[r], stop)
         assert it[0] == iters[r] and np.array_equal(one, s[r]), r
+
+
+@pytest.mark.parametrize("dims,nrhs,apbc", [
+    ((12, 2, 4, 4), 9, True), ((12, 4, 2, 2), 17, False), ((22, 2, 2, 4), 2, True), ((24, 4, 4, 2), 5, True)])
+def test_six_wide_tiles_match_oracle(ctx, dims, nrhs, apbc):
+    """Rows of 6, 11 and 12 half-sites: the hops' tiles are 6 wide (6, 6 + 5 and
+    6 + 6), the update's 3 and 4.  Bounds as above."""
+    test_truncated_solves_match_oracle(ctx, dims, nrhs, apbc)
