@@ -244,8 +244,12 @@ int Net::forward(Ctx& c, const float* X0, int nb, float** out) {
     const NetLayer& l = layers[li];
     const int K2 = 72 * l.cin, N2 = 8 * l.cout;
     // fused up to one tile of 256 columns (figures at pt_layer_kernel); wider
-    // layers gather Z once and multiply it tile by tile
-    if (l.Bs != nullptr) {
+    // layers gather Z once and multiply it tile by tile, and so do lattices of
+    // few blocks, where the fused kernel's chain of stages is the longer one
+    // (98 blocks, 4096 sites: 86 against 91 us at 12 channels, 110 against 104 at
+    // 24; 147 blocks: 87 against 98, 110 against 117; 13 blocks: 87 against 79, 109
+    // against 87).  By the lattice alone: a result does not depend on its batch.
+    if (l.Bs != nullptr && grid1(V, PT_SITES) >= PT_MIN_BLOCKS) {
       TSM_TRY(launch_layer(c, ng, l, X, nb, acts[li + 1], d_err));
     } else {
       pt_gather_kernel<<<dim3(grid1((long long)V * PT_PATHS * l.cin, NET_NT), nb), NET_NT, 0, c.stream>>>(

@@ -8,6 +8,7 @@
 
 namespace tsm {
 
+constexpr int PT_MIN_BLOCKS = 120;           // fewest blocks of a lattice that the fused layer is taken for
 constexpr int PT_SITES = 42;                 // sites of a CTA: 126 of the MMA's 128 rows (3 colours each)
 constexpr int PT_CORE = 144;                 // bytes from a core matrix to the next in K: 128 + 16, so that the
                                              // stores of neighbouring channels fall into different banks

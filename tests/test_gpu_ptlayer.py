@@ -32,3 +32,13 @@ def test_forward_matches_oracle(ctx, channels, dims):
     for b in range(2):
         want = ptnet.net_forward(U, ws, x[b], dims)[-1]
         assert np.linalg.norm(y[b] - want) <= 4 * L * U_BF16 * np.linalg.norm(want)
+
+
+@pytest.mark.parametrize("channels,dims", [
+    ([1, 1], (8, 6, 10, 12)), ([1, 5, 2, 1], (6, 14, 10, 6)), ([1, 9, 16, 1], (8, 6, 10, 12)),
+    ([1, 24, 17, 1], (8, 6, 10, 12)), ([1, 32, 1], (6, 14, 10, 6)), ([1, 40, 1], (8, 6, 10, 12)),
+    ([1, 12, 1], (14, 10, 6, 6)), ([1, 12, 1], (6, 10, 14, 4))])
+def test_fused_lattices_match_oracle(ctx, channels, dims):
+    """The same at the fewest blocks (120) the fused kernel is taken for, with whole
+    and part-filled last blocks, and just below.  Bound as above."""
+    test_forward_matches_oracle(ctx, channels, dims)
