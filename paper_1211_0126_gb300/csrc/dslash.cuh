@@ -147,34 +147,6 @@ __device__ __forceinline__ void su3_mul(const cx<R> r[9], const cx<R> h[6], cx<R
   }
 }
 
-// u = u0 + U h or u0 + U^dag h: the products' chains start from u0
-template <bool DAGU, class R>
-__device__ __forceinline__ void su3_mul_add(const cx<R> r[9], const cx<R> h[6], const cx<R> u0[6], cx<R> u[6]) {
-#pragma unroll
-  for (int s = 0; s < 2; ++s)
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      cx<R> v = u0[3 * s + i];
-#pragma unroll
-      for (int k = 0; k < 3; ++k)
-        v = DAGU ? cjmac(v, r[3 * k + i], h[3 * s + k]) : cmac(v, r[3 * i + k], h[3 * s + k]);
-      u[3 * s + i] = v;
-    }
-}
-
-// the upper components of a direction's two hops, sum, and the lower ones, the
-// reconstruction (spin matrix of (1 + SG gamma_MU)) of diff
-template <int MU, int SG, bool FIRST, class R>
-__device__ __forceinline__ void accumulate_pair(cx<R> acc[12], const cx<R> sum[6], const cx<R> diff[6]) {
-  cx<R> low[12];
-  accumulate<MU, SG, true>(low, diff);
-#pragma unroll
-  for (int k = 0; k < 6; ++k) {
-    acc[k] = FIRST ? sum[k] : acc[k] + sum[k];
-    acc[6 + k] = FIRST ? low[6 + k] : acc[6 + k] + low[6 + k];
-  }
-}
-
 // One direction of the stencil at output site (c, ih) of parity p.
 // links(h, nb, r) fills r[0..8] with the three rows of the link of hop h
 // (2 MU forward at x, 2 MU + 1 backward at x - mu, neighbour index nb).
@@ -184,11 +156,6 @@ __device__ __forceinline__ void hop_dir(const Geom& g, const int c[4], const typ
   using R = typename S::real;
   constexpr int SF = DAG ? +1 : -1;   // forward hop: (1 + SF gamma_mu)
   constexpr int SB = -SF;             // backward hop
-  // FP64, bound by its pipe: the backward product's chains start from the
-  // forward product u_f, whose upper components then need one addition for both
-  // hops, and the lower ones (opposite projector signs) get u_f - u_b = 2 u_f -
-  // sum with one multiply-add: 204 instead of 216 FP64 instructions per direction
-  constexpr bool PAIR = sizeof(R) == 8;
   cx<R> h[6], u[6], r[9];
   // forward neighbour x + mu
   {
@@ -207,7 +174,7 @@ __device__ __forceinline__ void hop_dir(const Geom& g, const int c[4], const typ
     }
     links(2 * MU, -1, r);
     su3_mul<false>(r, h, u);
-    if constexpr (!PAIR) accumulate<MU, SF, MU == 0>(acc, u);   // the site's first hop assigns
+    accumulate<MU, SF, MU == 0>(acc, u);   // the site's first hop assigns
   }
   // backward neighbour x - mu
   {
@@ -225,17 +192,8 @@ __device__ __forceinline__ void hop_dir(const Geom& g, const int c[4], const typ
       }
     }
     links(2 * MU + 1, nb, r);
-    if constexpr (PAIR) {
-      cx<R> sum[6];
-      su3_mul_add<true>(r, h, u, sum);          // u_f + u_b
-#pragma unroll
-      for (int k = 0; k < 6; ++k)               // u_f - u_b
-        u[k] = {fma((R)2, u[k].re, -sum[k].re), fma((R)2, u[k].im, -sum[k].im)};
-      accumulate_pair<MU, SF, MU == 0>(acc, sum, u);
-    } else {
-      su3_mul<true>(r, h, u);
-      accumulate<MU, SB, false>(acc, u);
-    }
+    su3_mul<true>(r, h, u);
+    accumulate<MU, SB, false>(acc, u);
   }
 }
 
@@ -459,7 +417,7 @@ __global__ void __launch_bounds__(128)
 // Squared norms of b - D_tm s and of b for a batch of sources, in FP64 from
 // fields of storage S (FP32 or FP64): one pass over both parities
 // (blockIdx.z), no widened copies, no stored residual.  Bound by the FP64 pipe:
-// 912 FP64 instructions per site (the hop kernel with its epilogue, the norm
+// 960 FP64 instructions per site (the hop kernel with its epilogue, the norm
 // kernel and the conversions took about 1150), the widening of FP32 components
 // is integer work beside them.  Partials: [2 parity + {residual, source}]
 // [source][block], added by residual_sum_kernel.
