@@ -40,6 +40,26 @@ template <class R> __device__ __forceinline__ cx<R> cmac(cx<R> acc, cx<R> a, cx<
 template <class R> __device__ __forceinline__ cx<R> cjmac(cx<R> acc, cx<R> a, cx<R> b) {
   return {fma(a.im, b.im, fma(a.re, b.re, acc.re)), fma(-a.im, b.re, fma(a.re, b.im, acc.im))};
 }
+// a0 b0 + a1 b1 + a2 b2 and conj(a0) b0 + conj(a1) b1 + conj(a2) b2: each part as
+// two chains of three multiply-adds and one addition, seven instructions instead
+// of eight for a sum of three products, with rounding errors of 2 (1 + 2 + 3) + 6 =
+// 18 instead of 3 (1 + 2) + 4 + 6 = 19 in units of one product's variance (one
+// chain of six: 21).  The terms with a's real parts come late: a link near the
+// identity rounds at its large term 7/3 times on average (sum of products 8/3).
+template <class R> __device__ __forceinline__ cx<R> cdot3(cx<R> a0, cx<R> b0, cx<R> a1, cx<R> b1, cx<R> a2, cx<R> b2) {
+  return {fma(a0.re, b0.re, fma(a1.re, b1.re, -a0.im * b0.im)) + fma(a2.re, b2.re, fma(-a2.im, b2.im, -a1.im * b1.im)),
+          fma(a0.re, b0.im, fma(a1.re, b1.im, a0.im * b0.re)) + fma(a2.re, b2.im, fma(a2.im, b2.re, a1.im * b1.re))};
+}
+template <class R> __device__ __forceinline__ cx<R> cjdot3(cx<R> a0, cx<R> b0, cx<R> a1, cx<R> b1, cx<R> a2, cx<R> b2) {
+  return cdot3(cconj(a0), b0, cconj(a1), b1, cconj(a2), b2);
+}
+// the same as one chain of six (FP64, whose pipe counts every instruction)
+template <class R> __device__ __forceinline__ cx<R> cdot3_chain(cx<R> a0, cx<R> b0, cx<R> a1, cx<R> b1, cx<R> a2, cx<R> b2) {
+  const R re = fma(-a2.im, b2.im, fma(-a1.im, b1.im, -a0.im * b0.im));
+  const R im = fma(a2.im, b2.re, fma(a1.im, b1.re, a0.im * b0.re));
+  return {fma(a2.re, b2.re, fma(a1.re, b1.re, fma(a0.re, b0.re, re))),
+          fma(a2.re, b2.im, fma(a1.re, b1.im, fma(a0.re, b0.im, im)))};
+}
 template <class R> __device__ __forceinline__ cx<R> times_i(cx<R> a) { return {-a.im, a.re}; }
 template <class R> __device__ __forceinline__ R norm2(cx<R> a) { return a.re * a.re + a.im * a.im; }
 

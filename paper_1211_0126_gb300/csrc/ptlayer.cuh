@@ -155,13 +155,13 @@ __global__ void __launch_bounds__(256, BN <= 128 ? 2 : 1)
               for (int s2 = 0; s2 < 4; ++s2)
 #pragma unroll
                 for (int a = 0; a < 3; ++a)
-                  out[s2][a] = cmac(cmac(u[3 * a] * v[s2][0], u[3 * a + 1], v[s2][1]), u[3 * a + 2], v[s2][2]);
+                  out[s2][a] = cdot3(u[3 * a], v[s2][0], u[3 * a + 1], v[s2][1], u[3 * a + 2], v[s2][2]);
             } else {
 #pragma unroll
               for (int s2 = 0; s2 < 4; ++s2)
 #pragma unroll
                 for (int a = 0; a < 3; ++a)
-                  out[s2][a] = cjmac(cjmac(cjmul(u[a], v[s2][0]), u[3 + a], v[s2][1]), u[6 + a], v[s2][2]);
+                  out[s2][a] = cjdot3(u[a], v[s2][0], u[3 + a], v[s2][1], u[6 + a], v[s2][2]);
             }
           }
         } else {

@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(NET_NT) pt_gather_kernel(NetGeom ng, const flo
     for (int s2 = 0; s2 < 4; ++s2)
 #pragma unroll
       for (int a = 0; a < 3; ++a)
-        out[s2][a] = cmac(cmac(w[3 * a] * v[s2][0], w[3 * a + 1], v[s2][1]), w[3 * a + 2], v[s2][2]);
+        out[s2][a] = cdot3(w[3 * a], v[s2][0], w[3 * a + 1], v[s2][1], w[3 * a + 2], v[s2][2]);
   }
   const int j8 = (p * C + ch) * 8;
 #pragma unroll
@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(NET_NT) pt_gather_adjoint_kernel(NetGeom ng, c
       for (int s2 = 0; s2 < 4; ++s2)
 #pragma unroll
         for (int a = 0; a < 3; ++a)
-          acc[s2][a] = cmac(cmac(cmac(acc[s2][a], w[3 * a], v[s2][0]), w[3 * a + 1], v[s2][1]), w[3 * a + 2], v[s2][2]);
+          acc[s2][a] = acc[s2][a] + cdot3(w[3 * a], v[s2][0], w[3 * a + 1], v[s2][1], w[3 * a + 2], v[s2][2]);
     }
   }
   const int w = 8 * C;
