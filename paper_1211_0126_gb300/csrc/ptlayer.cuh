@@ -84,9 +84,14 @@ __global__ void __launch_bounds__(256, BN <= 128 ? 2 : 1)
                  "r"(TMEM_COLS));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
-  // rows that no site fills stay zero
-  for (uint32_t o = tid * 16; o < 2 * stage_bytes; o += 256 * 16)
-    asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(ring + o), "r"(0u) : "memory");
+  // rows of Z that no site fills stay zero (each thread's proxy fence in the loop
+  // orders these stores before the MMAs).  The weight parts are left to the bulk
+  // copies, which write every byte of them: nothing orders a generic store here
+  // before a copy of the async proxy to the same bytes
+  for (uint32_t o = tid * 16; o < 2 * a_bytes; o += 256 * 16)
+    asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(ring + o + (o < a_bytes ? 0u : stage_bytes - a_bytes)),
+                 "r"(0u)
+                 : "memory");
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
