@@ -374,6 +374,8 @@ int check_timeout(Net& n, cudaStream_t s) {
   TSM_CUDA(cudaMemcpyAsync(&herr, n.d_err, sizeof(int), cudaMemcpyDeviceToHost, s));
   TSM_CUDA(cudaStreamSynchronize(s));
   if (herr) {
+    TSM_CUDA(cudaMemsetAsync(n.d_err, 0, sizeof(int), s));   // reported once: the next call starts clean
+    TSM_CUDA(cudaStreamSynchronize(s));
     set_error("a tensor-core wait of the network timed out");
     return TSM_ERR_TIMEOUT;
   }

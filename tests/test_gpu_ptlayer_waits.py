@@ -30,3 +30,28 @@ def test_weights_survive_the_zero_fill(ctx, channels, dims):
         if k % 10 == 0:
             ctx.dslash(x[0, 0], tsm.TM_OP_FULL, False, tsm.TSM_F64)
         assert np.array_equal(net.forward(ctx, x), y), k
+
+TIMEOUT = -6   # TSM_ERR_TIMEOUT
+
+
+def _timeout_and_recovery(ctx, channels, dims):
+    U = S.gauge_field(dims, 0.3, 3)
+    ctx.load_gauge(U, dims, 0.124, 0.01)
+    net = tsm.Network(channels, seed=1, init_scale=1.0)
+    x = S.random_spinor(dims, 5, batch=(1, 1))
+    y = net.forward(ctx, x)
+    tsm.tsm_umma_inject_timeout(True)
+    try:
+        with pytest.raises(tsm.TsmError) as e:
+            net.forward(ctx, x)
+        assert e.value.status == TIMEOUT
+    finally:
+        tsm.tsm_umma_inject_timeout(False)
+    assert np.array_equal(net.forward(ctx, x), y)
+
+
+def test_timeout_of_the_gemm_is_reported_once(ctx):
+    """Operand copies withheld on the host's request (nothing is in flight, every
+    wait ends): the call on a lattice of few blocks, gather and GEMM, reports
+    TSM_ERR_TIMEOUT and the next one computes again."""
+    _timeout_and_recovery(ctx, [1, 5, 1], (4, 4, 4, 4))
