@@ -217,7 +217,7 @@ int layer_launch(Ctx& c, const NetGeom& ng, const NetLayer& l, const float* X, i
   const int gj = pt_groups(l.cin), steps = pt_steps(l.cin), smem = pt_layer_smem<BN>(gj);
   TSM_CUDA(cudaFuncSetAttribute(pt_layer_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   pt_layer_kernel<BN><<<dim3(grid1(c.g.V, PT_SITES), nb), 256, smem, c.stream>>>(ng, X, l.cin, l.Bs, 8 * l.cout, Y, gj,
-                                                                                 steps, err);
+                                                                                 steps, err, g_umma_withhold.load());
   return check_net_launch(c, "pt_layer_kernel");
 }
 

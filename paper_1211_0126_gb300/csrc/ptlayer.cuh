@@ -51,7 +51,10 @@ __global__ void __launch_bounds__(256) pt_pack_stages_kernel(const __nv_bfloat16
 // once), rebuilds the link once for both, transports in FP32 and stores three
 // 16-byte core-matrix rows per group; a stage of B is one bulk copy of weights
 // packed in its layout.  One thread issues the stage's MMAs, which run while the
-// next stage is computed.  Every wait is bounded as in umma.cuh.
+// next stage is computed.  Every wait is bounded; a thread whose wait ran out
+// says so at the stage's barrier, where all leave the loop together, the MMAs and
+// copies in flight are waited for (bounded), TMEM is freed and the error is
+// recorded.  withhold: fault injection as in umma.cuh (no weight copies).
 // 12 -> 12 channels at 16^3x32: 346 us against 310 (gather, 680 MB of Z written)
 // + 170 (GEMM); 12 -> 1: 267 against 310 + 108.  Bound by the latency of the
 // neighbour loads (16 warps of 120 registers per SM, 36 % issue; the ring leaves
@@ -59,12 +62,11 @@ __global__ void __launch_bounds__(256) pt_pack_stages_kernel(const __nv_bfloat16
 template <int BN>
 __global__ void __launch_bounds__(256, BN <= 128 ? 2 : 1)
     pt_layer_kernel(NetGeom ng, const float* __restrict__ X, int C, const uint8_t* __restrict__ B, int N,
-                    float* __restrict__ Y, int GJ, int steps, int* __restrict__ error) {
+                    float* __restrict__ Y, int GJ, int steps, int* __restrict__ error, int withhold) {
   constexpr int TMEM_COLS = BN <= 32 ? 32 : (BN <= 64 ? 64 : (BN <= 128 ? 128 : 256));
   extern __shared__ uint8_t pt_dyn[];
   __shared__ __align__(8) uint64_t bar[2], wbar[2];   // a stage's MMAs, its weights
   __shared__ uint32_t tmem_slot;
-  __shared__ int timed_out;
   __shared__ int s_nbr[PT_SITES][8];   // neighbour of path p = 1 .. 8, its complement if the hop changes sign
   const uint32_t ring = (smem_u32(pt_dyn) + 127u) & ~127u;
   const uint32_t a_bytes = 16u * GJ * PT_CORE, stage_bytes = a_bytes + (uint32_t)(BN / 8) * GJ * PT_CORE;
@@ -76,7 +78,6 @@ __global__ void __launch_bounds__(256, BN <= 128 ? 2 : 1)
     mbar_init(&bar[1], 1);
     mbar_init(&wbar[0], 1);
     mbar_init(&wbar[1], 1);
-    timed_out = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
@@ -117,13 +118,16 @@ __global__ void __launch_bounds__(256, BN <= 128 ? 2 : 1)
     }
   }
   __syncthreads();
-  int wcopies = 0;   // thread 0: weight copies issued
-  for (int k = 0; k < steps; ++k) {
+  const long long limit = withhold ? UMMA_INJECT_LIMIT : MBAR_SPIN_LIMIT;
+  bool failed = false;   // a wait of this thread ran out; all threads learn of it at the stage's barrier
+  int wcopies = 0;       // thread 0: weight copies issued
+  int k = 0;             // stages whose MMAs were issued
+  for (; k < steps; ++k) {
     const int s = k & 1;
     const uint32_t sa = ring + s * stage_bytes, sb = sa + a_bytes;
     // the stage's previous MMAs are done
-    if (k >= 2 && !mbar_wait(&bar[s], (uint32_t)((k / 2 - 1) & 1))) *reinterpret_cast<volatile int*>(&timed_out) = 1;
-    if (tid == 0 && !*reinterpret_cast<volatile int*>(&timed_out)) {
+    if (k >= 2) failed = !mbar_wait(&bar[s], (uint32_t)((k / 2 - 1) & 1), limit);
+    if (tid == 0 && !failed && !withhold) {
       mbar_expect_tx(&wbar[s], b_bytes);
       bulk_load(sb, B + (size_t)k * b_bytes, b_bytes, &wbar[s]);
       wcopies = k + 1;
@@ -191,10 +195,9 @@ __global__ void __launch_bounds__(256, BN <= 128 ? 2 : 1)
       }
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic stores -> tensor core
-    __syncthreads();
-    if (*reinterpret_cast<volatile int*>(&timed_out)) break;
+    if (tid == 0 && !failed) failed = !mbar_wait(&wbar[s], (uint32_t)((k / 2) & 1), limit);
+    if (__syncthreads_or(failed)) break;   // the same iteration for every thread
     if (tid == 0) {
-      if (!mbar_wait(&wbar[s], (uint32_t)((k / 2) & 1))) *reinterpret_cast<volatile int*>(&timed_out) = 1;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       for (int kk = 0; kk < pairs; ++kk) {
         const uint64_t da = umma_desc(sa + kk * 2 * PT_CORE, PT_CORE, group_rows);
@@ -210,10 +213,10 @@ __global__ void __launch_bounds__(256, BN <= 128 ? 2 : 1)
                    : "memory");
     }
   }
-  // the last commit covers every earlier MMA
-  const int last = steps - 1;
-  if (!mbar_wait(&bar[last & 1], (uint32_t)((last / 2) & 1))) *reinterpret_cast<volatile int*>(&timed_out) = 1;
-  __syncthreads();
+  // the last commit covers every earlier MMA (after a timeout: of the stages issued)
+  failed = k < steps;
+  if (k > 0 && !mbar_wait(&bar[(k - 1) & 1], (uint32_t)(((k - 1) / 2) & 1))) failed = true;
+  const bool timed_out = __syncthreads_or(failed);
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (!timed_out) {
     // warp w: accumulator lanes (rows) 32 (w % 4) .., columns of half w / 4
@@ -234,10 +237,9 @@ __global__ void __launch_bounds__(256, BN <= 128 ? 2 : 1)
       }
     }
   } else {
-    // a second bounded wait for MMAs and copies in flight before the memory is released
-    mbar_wait(&bar[0], 0);
+    // the MMAs in flight were waited for above, now the copies, before the memory is released
     if (tid == 0) {
-      for (int k = max(0, wcopies - 2); k < wcopies; ++k) mbar_wait(&wbar[k & 1], (uint32_t)((k / 2) & 1));
+      for (int c = max(0, wcopies - 2); c < wcopies; ++c) mbar_wait(&wbar[c & 1], (uint32_t)((c / 2) & 1));
       if (error != nullptr) atomicExch(error, 1);
     }
   }

@@ -55,3 +55,11 @@ def test_timeout_of_the_gemm_is_reported_once(ctx):
     wait ends): the call on a lattice of few blocks, gather and GEMM, reports
     TSM_ERR_TIMEOUT and the next one computes again."""
     _timeout_and_recovery(ctx, [1, 5, 1], (4, 4, 4, 4))
+
+
+@pytest.mark.parametrize("channels", [[1, 5, 1], [1, 24, 17, 1]])
+def test_timeout_of_the_fused_layer(ctx, channels):
+    """The same on a lattice of 138 blocks of the fused layer, one and two blocks
+    per SM: the first stage's weights never come, every thread leaves the loop at
+    that stage, tensor memory is freed."""
+    _timeout_and_recovery(ctx, channels, (8, 6, 10, 12))
