@@ -175,20 +175,19 @@ static __global__ void __launch_bounds__(SITE_NT) pack_links_kernel(Geom g, cons
     store_link<F32>(l32 + off32, lstride, mu, ih, rf);
     store_link<F16>(l16 + off32, lstride, mu, ih, rf);
     store_link<BF16>(lbf + off32, lstride, mu, ih, rf);
-    // tensor-core stencil: rows 0, 1 in FP16, row 2 = conj(row0 x row1) of those in FP32, kept as FP16 hi + lo
-    uint32_t w12[12];
-    cx<float> q[6], w2[3];
+    // tensor-core stencil: rows 0, 1 in FP16, row 2 = conj(row0 x row1) of those as FP16 hi + lo
+    uint32_t w12[12], wlo[3];   // wlo: the scaled remainders of a forward link
+    cx<float> q[6], lo[3];
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
       w12[k] = Pack16<F16>::pack(rf[k]);
       q[k] = Pack16<F16>::unpack(w12[k]);
     }
-    third_row(q, w2);
+    third_row_pair(q, w12 + 6, lo);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      w12[6 + k] = Pack16<F16>::pack(w2[k]);
-      const cx<float> hi = Pack16<F16>::unpack(w12[6 + k]);
-      w12[9 + k] = Pack16<F16>::pack(w2[k] - hi);
+      w12[9 + k] = Pack16<F16>::pack(lo[k]);
+      wlo[k] = Pack16<F16>::pack(F16G::LO_SCALE * lo[k]);
     }
     // [site][hop][12]: forward hop of this site, backward hop of x + mu, with the sign of an antiperiodic boundary
     bool wraps = false;
@@ -205,7 +204,7 @@ static __global__ void __launch_bounds__(SITE_NT) pack_links_kernel(Geom g, cons
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       const uint4 v = make_uint4(w12[4 * k] ^ sign, w12[4 * k + 1] ^ sign, w12[4 * k + 2] ^ sign, w12[4 * k + 3] ^ sign);
-      own[k] = v;
+      own[k] = k < 2 ? v : make_uint4(v.x, wlo[0] ^ sign, wlo[1] ^ sign, wlo[2] ^ sign);
       fwd[k] = v;
     }
   }

@@ -21,10 +21,15 @@
 // [source][colour] chunks of four spins; a warp's load of one neighbour is 384
 // contiguous bytes.
 //
-// Row 2 of a link, conj(row0 x row1) in FP32, is kept as an FP16 pair hi + lo
-// (22 bits): the lo part of a forward link sits in columns 6, 7 (added to
-// colour 2 afterwards), that of a backward link in k slot 3, which carries
-// colour 2 of the half spinor a second time.  Products are exact, sums FP32.
+// Row 2 of a link, conj(row0 x row1), is kept as an FP16 pair hi + lo of its exact
+// value: the lo part of a forward link, scaled by 2^11, sits in columns 6, 7 (added
+// to colour 2 afterwards), that of a backward link in k slot 3, which carries
+// colour 2 of the half spinor a second time.  Products are exact, sums FP32: the 16
+// products of a direction on the tensor cores, which round towards zero, the four
+// directions by additions.  Rounding error of H psi against 64 bits on the same FP16
+// fields and links, relative rms: 6.97e-8 on random links (9.98e-8 with one
+// accumulator over the directions and the pair of an FP32 row; FP32 sums of products
+// with row 2 in FP32 7.03e-8), 0.978 of the FP32 products' near the identity.
 //
 // The lower spin components are the same products times a phase and in one
 // of two orders: the MMA of a direction is issued a second time with the
@@ -143,10 +148,12 @@ __device__ __forceinline__ bool mma_wait_failed(uint64_t* bar, uint32_t parity) 
   return !mbar_try(bar, parity) && !mbar_wait(bar, parity, MMA_SPIN_LIMIT);
 }
 
+// d = a b (no accumulator: the tensor cores round a sum towards zero, so that only
+// the 16 products of one direction are added there)
 __device__ __forceinline__ void mma_f16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+      : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
 }
 __device__ __forceinline__ uint32_t h2_fma(uint32_t a, uint32_t b, uint32_t c) {
   uint32_t d;
@@ -231,41 +238,49 @@ template <int DAG, int W>
 __device__ __forceinline__ void mma_site(const uint4* nb, const MmaSlots& sl, const uint32_t (&B)[4][2],
                                          const uint32_t (&BL)[4][2], float (&acc)[8]) {
   constexpr int SF = DAG ? +1 : -1;
-  float up[4] = {0.f, 0.f, 0.f, 0.f}, ya[4] = {0.f, 0.f, 0.f, 0.f}, yb[4] = {0.f, 0.f, 0.f, 0.f};
   uint32_t a[4];
+  float d[4], e[4];   // a direction's upper and lower components
   project_word<0, SF>(nb[sl.xf], a[0], a[1]);
   project_word<0, -SF>(nb[sl.xb], a[2], a[3]);
-  mma_f16(up, a, B[0][0], B[0][1]);
-  mma_f16(ya, a, BL[0][0], BL[0][1]);      // rows: spin 3 | spin 2
-  ya[0] = -ya[0];
-  ya[1] = -ya[1];
+  mma_f16(d, a, B[0][0], B[0][1]);
+  mma_f16(e, a, BL[0][0], BL[0][1]);       // rows: spin 3 | spin 2
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    acc[k] = d[k];
+    acc[4 + k] = e[k ^ 2];
+  }
   project_word<1, SF>(nb[sl.yf], a[0], a[1]);
   project_word<1, -SF>(nb[sl.yb], a[2], a[3]);
-  mma_f16(up, a, B[1][0], B[1][1]);
-  mma_f16(ya, a, BL[1][0], BL[1][1]);      // rows: -spin 3 | spin 2
+  mma_f16(d, a, B[1][0], B[1][1]);
+  mma_f16(e, a, BL[1][0], BL[1][1]);       // rows: -spin 3 | spin 2
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    acc[k] += d[k];
+    acc[4 + k] += k < 2 ? e[k ^ 2] : -e[k ^ 2];
+  }
   project_word<2, SF>(nb[sl.zf], a[0], a[1]);
   project_word<2, -SF>(nb[sl.zb], a[2], a[3]);
-  mma_f16(up, a, B[2][0], B[2][1]);
-  mma_f16(yb, a, BL[2][0], BL[2][1]);      // rows: spin 2 | -spin 3
-  yb[2] = -yb[2];
-  yb[3] = -yb[3];
+  mma_f16(d, a, B[2][0], B[2][1]);
+  mma_f16(e, a, BL[2][0], BL[2][1]);       // rows: spin 2 | -spin 3
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    acc[k] += d[k];
+    acc[4 + k] += k < 2 ? e[k] : -e[k];
+  }
   project_word<3, SF>((nb + sl.t)[4 * W * MMA_CHUNKS], a[0], a[1]);
   project_word<3, -SF>(nb[sl.t], a[2], a[3]);
-  mma_f16(up, a, B[3][0], B[3][1]);
-  mma_f16(yb, a, BL[3][0], BL[3][1]);      // rows: spin 2 | spin 3
-  acc[0] = up[0];
-  acc[1] = up[1];
-  acc[2] = up[2];
-  acc[3] = up[3];
-  acc[4] = ya[2] + yb[0];
-  acc[5] = ya[3] + yb[1];
-  acc[6] = yb[2] - ya[0];
-  acc[7] = yb[3] - ya[1];
+  mma_f16(d, a, B[3][0], B[3][1]);
+  mma_f16(e, a, BL[3][0], BL[3][1]);       // rows: spin 2 | spin 3
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    acc[k] += d[k];
+    acc[4 + k] += e[k];
+  }
   const int lane = threadIdx.x & 31;
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     const float lo = __shfl_sync(0xffffffffu, acc[k], lane | 3);
-    if ((lane & 3) == 2) acc[k] += lo;
+    if ((lane & 3) == 2) acc[k] = fmaf(lo, 1.f / F16G::LO_SCALE, acc[k]);
   }
 }
 
@@ -309,7 +324,9 @@ __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap* map
 // (24 + 4 warps at 72 registers: the next link words wait in shared memory, the lane
 // constants are formed per tile) and fewer neighbour sites per output site (5.5
 // against 5.75).  24^3x48, 32 sources: K1 370 -> 349 us, K2 473 -> 463; 12^3x24 (3
-// half-sites of a W = 4 tile used): K1 42.8 -> 35.0, K2 56.6 -> 48.6.  Against
+// half-sites of a W = 4 tile used): K1 42.8 -> 35.0, K2 56.6 -> 48.6.  With the
+// directions added outside the tensor cores (24 additions a lane for 8): K1 357, K2
+// 484, K3 353, K4 621 at 24^3x48 x 32, 34.7 / 50.1 / 33.9 / 66.6 at 12^3x24 x 32.  Against
 // the FP32 FMA stencil that these kernels replaced (1727 thread instructions per
 // source-site), 24^3x48, 32 sources: K1 575, K2 690, K3 574, K4 849 -> 614 (5.9
 // TB/s); with one group of 8: K1 152 -> 139, K2 199 -> 171, K4 233 -> 194.  A group
