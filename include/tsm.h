@@ -81,10 +81,13 @@ typedef enum {
  *   TSM_BF16, TSM_F16  16-bit storage of links and Krylov/operator vectors,
  *            FP32 arithmetic.  TSM_F16 keeps the CG residual and iterate in
  *            FP16 as well (relative precision 2^-11, below the truncation of
- *            an LP solve) and solves in groups of 8 sources on the tensor
- *            cores (FP16 products, FP32 sums): a group costs the same however
- *            few of its sources are used, so batches of a multiple of 8 pay
- *            most; TSM_BF16 keeps them in FP32.  Sources and solutions
+ *            an LP solve); TSM_BF16 keeps them in FP32.  TSM_F16 solves run
+ *            in groups of 8 sources on the tensor cores (FP16 products, FP32
+ *            sums) inside tsm_loops / tsm_loops_graph (up to 2^25 sites) and,
+ *            on lattices of up to 108 sites per SM, in tm_solve_batch; the
+ *            lattice alone decides, so that a source's bits do not depend on
+ *            its batch.  A group costs the same, and holds the fields of 8
+ *            sources, however few of its sources are used.  Sources and solutions
  *            are exchanged in FP32 for both through tm_solve_batch; inside
  *            tsm_loops / tsm_loops_graph the TSM_F16 tier also keeps its noise
  *            source, Schur source and solution in FP16 (the solution is FP16
@@ -346,8 +349,8 @@ int tsm_tune(tsm_ctx* ctx, const tm_stop* stop, int* best_batch, int* best_tile,
 /* Set the block shape of the link-sharing stencil of tier prec (TSM_F16,
  * TSM_BF16 or TSM_F32) for this context's later solves, as tsm_tune does:
  * tile_sources 2, 4 or 8 sources per block, max_regs 80 (or 96 with 4
- * sources); 4 and 80 by default.  TSM_F16 accepts the call and is unaffected
- * by it.  TSM_ERR_ARG for other tiers or values. */
+ * sources); 4 and 80 by default.  TSM_F16: for the solves that do not run in
+ * groups of 8 (see tsm_prec).  TSM_ERR_ARG for other tiers or values. */
 int tsm_set_tile(tsm_ctx* ctx, int prec, int tile_sources, int max_regs);
 
 

@@ -212,7 +212,7 @@ int prepare_run(Ctx& c, const tsm_params* p, TsmRun* run, bool branch = false) {
   }
   run->n_hp = (int)(p->hp_end - p->hp_begin);
   run->n_lp = (int)(p->lp_end - p->lp_begin);
-  run->sp_lp = loop_solution_prec(p->lp);
+  run->sp_lp = loop_solution_prec(c, p->lp);
   run->sp_hp = solution_prec(p->hp);
   run->cp_lp = run->sp_lp == F16G::id ? TSM_F16 : run->sp_lp;
   run->fp64_path = (p->lp.prec == TSM_F64 && p->hp.prec == TSM_F64);
@@ -548,17 +548,20 @@ int tsm_load_gauge(tsm_ctx* h, const tm_lattice* lat, const double* U, int on_de
     if (c.links_base) cudaFree(c.links_base);
     c.links_base = nullptr;
     const size_t vh = (size_t)c.g.Vh;
-    // the links of every storage in one allocation
+    // the links of every storage in one allocation (those of the tensor-core
+    // stencil only for lattices that it is used on)
     const size_t per_site[5] = {4 * F64::LN * sizeof(double2), 4 * F32::LN * sizeof(float4),
                                 4 * BF16::LN * sizeof(uint2), 4 * F16::LN * sizeof(uint2),
                                 4 * F16G::LN * sizeof(uint32_t)};
     size_t off[5], total = 0;
-    for (int k = 0; k < 5; ++k) {
+    const int kinds = f16_grouped_loops(c) || f16_grouped_solve(c) ? 5 : 4;
+    for (int k = 0; k < kinds; ++k) {
       off[k] = total;
       total += (2 * vh * per_site[k] + 255) & ~(size_t)255;
     }
+    for (void*& l : c.links) l = nullptr;
     TSM_CUDA(cudaMalloc(&c.links_base, total));
-    for (int k = 0; k < 5; ++k) c.links[k] = static_cast<char*>(c.links_base) + off[k];
+    for (int k = 0; k < kinds; ++k) c.links[k] = static_cast<char*>(c.links_base) + off[k];
     if (c.red.partials) cudaFree(c.red.partials);
     c.red_cap = vh / 32 + 64;   // block partials: up to one per 32 sites (link-sharing stencil)
     c.red.stride = (int)c.red_cap;
@@ -1065,9 +1068,11 @@ int tsm_tune(tsm_ctx* h, const tm_stop* stop, int* best_batch, int* best_tile, i
   const int regs[kShapes] = {80, 80, 80, 96};
   // the link-sharing stencil (BF16; FP32 for its hops without a reduction) has
   // a block shape to choose; FP64 runs one thread per (source, site), FP16 the
-  // tensor-core stencil, whose blocks are fixed (one timing stands for every shape)
-  const bool fixed16 = stop->prec == TSM_F16;
-  const bool tiled = fixed16 || stop->prec == TSM_BF16 || stop->prec == TSM_F32;
+  // tensor-core stencil, whose blocks are fixed (one timing stands for every shape;
+  // but see f16_grouped_loops)
+  const int sp = loop_solution_prec(c, *stop);   // the solves of the loop estimators
+  const bool fixed16 = sp == F16G::id;
+  const bool tiled = stop->prec == TSM_F16 || stop->prec == TSM_BF16 || stop->prec == TSM_F32;
   const int ntile = tiled && !fixed16 ? kShapes : 1;
   auto ib = c.tuned_batch.find(key);
   auto it = c.tuned_rpb.find(key);
@@ -1082,7 +1087,6 @@ int tsm_tune(tsm_ctx* h, const tm_stop* stop, int* best_batch, int* best_tile, i
     }
     return TSM_OK;
   }
-  const int sp = loop_solution_prec(*stop);   // the solves of the loop estimators
   c.batch_cap = std::max(c.batch_cap, cand[3]);
   EOField fb, fs;
   TSM_TRY(eo_fields(c, "tune_b", sp, &fb, c.batch_cap));

@@ -175,37 +175,39 @@ static __global__ void __launch_bounds__(SITE_NT) pack_links_kernel(Geom g, cons
     store_link<F32>(l32 + off32, lstride, mu, ih, rf);
     store_link<F16>(l16 + off32, lstride, mu, ih, rf);
     store_link<BF16>(lbf + off32, lstride, mu, ih, rf);
-    // tensor-core stencil: rows 0, 1 in FP16, row 2 = conj(row0 x row1) of those as FP16 hi + lo
-    uint32_t w12[12], wlo[3];   // wlo: the scaled remainders of a forward link
-    cx<float> q[6], lo[3];
+    if (lmma != nullptr) {
+      // tensor-core stencil: rows 0, 1 in FP16, row 2 = conj(row0 x row1) of those as FP16 hi + lo
+      uint32_t w12[12], wlo[3];   // wlo: the scaled remainders of a forward link
+      cx<float> q[6], lo[3];
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
-      w12[k] = Pack16<F16>::pack(rf[k]);
-      q[k] = Pack16<F16>::unpack(w12[k]);
-    }
-    third_row_pair(q, w12 + 6, lo);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      w12[9 + k] = Pack16<F16>::pack(lo[k]);
-      wlo[k] = Pack16<F16>::pack(F16G::LO_SCALE * lo[k]);
-    }
-    // [site][hop][12]: forward hop of this site, backward hop of x + mu, with the sign of an antiperiodic boundary
-    bool wraps = false;
-#pragma unroll
-    for (int d = 0; d < 4; ++d)
-      if (d == mu) {
-        wraps = c[d] + 1 == g.L[d];
-        c[d] = wraps ? 0 : c[d] + 1;
+      for (int k = 0; k < 6; ++k) {
+        w12[k] = Pack16<F16>::pack(rf[k]);
+        q[k] = Pack16<F16>::unpack(w12[k]);
       }
-    const uint32_t sign = wraps && mu == 3 && g.apbc ? 0x80008000u : 0u;
-    const int fh = half_index(g, c[0], c[1], c[2], c[3]);
-    uint4* own = reinterpret_cast<uint4*>(lmma) + (((size_t)parity * g.Vh + ih) * 8 + 2 * mu) * 3;
-    uint4* fwd = reinterpret_cast<uint4*>(lmma) + (((size_t)(1 - parity) * g.Vh + fh) * 8 + 2 * mu + 1) * 3;
+      third_row_pair(q, w12 + 6, lo);
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const uint4 v = make_uint4(w12[4 * k] ^ sign, w12[4 * k + 1] ^ sign, w12[4 * k + 2] ^ sign, w12[4 * k + 3] ^ sign);
-      own[k] = k < 2 ? v : make_uint4(v.x, wlo[0] ^ sign, wlo[1] ^ sign, wlo[2] ^ sign);
-      fwd[k] = v;
+      for (int k = 0; k < 3; ++k) {
+        w12[9 + k] = Pack16<F16>::pack(lo[k]);
+        wlo[k] = Pack16<F16>::pack(F16G::LO_SCALE * lo[k]);
+      }
+      // [site][hop][12]: forward hop of this site, backward hop of x + mu, with the sign of an antiperiodic boundary
+      bool wraps = false;
+#pragma unroll
+      for (int d = 0; d < 4; ++d)
+        if (d == mu) {
+          wraps = c[d] + 1 == g.L[d];
+          c[d] = wraps ? 0 : c[d] + 1;
+        }
+      const uint32_t sign = wraps && mu == 3 && g.apbc ? 0x80008000u : 0u;
+      const int fh = half_index(g, c[0], c[1], c[2], c[3]);
+      uint4* own = reinterpret_cast<uint4*>(lmma) + (((size_t)parity * g.Vh + ih) * 8 + 2 * mu) * 3;
+      uint4* fwd = reinterpret_cast<uint4*>(lmma) + (((size_t)(1 - parity) * g.Vh + fh) * 8 + 2 * mu + 1) * 3;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const uint4 v = make_uint4(w12[4 * k] ^ sign, w12[4 * k + 1] ^ sign, w12[4 * k + 2] ^ sign, w12[4 * k + 3] ^ sign);
+        own[k] = k < 2 ? v : make_uint4(v.x, wlo[0] ^ sign, wlo[1] ^ sign, wlo[2] ^ sign);
+        fwd[k] = v;
+      }
     }
   }
 #pragma unroll

@@ -331,8 +331,9 @@ __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap* map
 // source-site), 24^3x48, 32 sources: K1 575, K2 690, K3 574, K4 849 -> 614 (5.9
 // TB/s); with one group of 8: K1 152 -> 139, K2 199 -> 171, K4 233 -> 194.  A group
 // costs the same however few of its 8 rows are used (4 sources: K1 83 -> 139 us),
-// but a source's bits must not depend on its batch, so every FP16 solve runs here
-// and the loop estimators fill whole groups.  Tried on the way: neighbours loaded
+// but a source's bits must not depend on its batch: the lattice alone decides which
+// solves run here (f16_grouped_solve, f16_grouped_loops), and the loop estimators
+// fill whole groups.  Tried on the way: neighbours loaded
 // from L2 by each warp one item ahead (K1 560 us, latency-bound at 39 % issue),
 // bulk copies of rows issued by one warp (676 us, the copy warp set the pace) and
 // by four (375 us), all boxes issued by one thread (485 us), W = 6 with two copy

@@ -29,16 +29,16 @@ int launch_hop(Ctx& c, const HopArgs<S>& a0, int dag, int mode, int prof_kind, i
   const double bytes = (double)a.g.Vh *
       (lb + nrhs * sb * (2 + ((mode & HOP_CENTER) ? 1 : 0) + ((mode & HOP_BASE) ? 1 : 0)));
   TimedLaunch tl(c, 4 * S::id + kind, bytes);
-  // BF16: link-sharing blocks of LT_SITES sites x up to RPB sources (RPB =
-  // c.tile_rpb, 2, 4 or 8, and for 4 a register budget of 80 or 96, from the
+  // 16-bit tiers (FP16: where its solves do not run in grouped storage, see
+  // f16_grouped_solve): link-sharing blocks of LT_SITES sites x up to RPB sources
+  // (RPB = c.tile_rpb, 2, 4 or 8, and for 4 a register budget of 80 or 96, from the
   // autotuner; every solve, whatever its batch width, so that a source's
   // iterates do not depend on its batch); the FP32 tier the same for the hops
   // without a reduction (its reducing hop K2 measured slower in tiles; per-site
-  // arithmetic, and so every result, is the same in both kernels); FP64, FP16
-  // (whose batched solves run in grouped storage, F16G) and single-source
-  // operator applications outside the solvers (c.hop_per_site): one thread per
-  // (source, site), blocks of HOP_NT sites
-  constexpr bool TILE16 = S::id == BF16::id;
+  // arithmetic, and so every result, is the same in both kernels); FP64 and
+  // single-source operator applications outside the solvers (c.hop_per_site):
+  // one thread per (source, site), blocks of HOP_NT sites
+  constexpr bool TILE16 = S::id == F16::id || S::id == BF16::id;
   constexpr bool TILE32 = S::id == F32::id;
   // (FP32: only with several sources to share the links; a single field runs
   // faster one thread per site, with the same bits)
@@ -118,7 +118,8 @@ int launch_cg_update(Ctx& c, const CGUpdArgs<S, SA>& a0, int nrhs) {
   TimedLaunch tl(c, 4 * S::id + PK_HOP_UPDATE, (double)a.g.Vh * (lb + nrhs * (3 * sb + 4 * sa)));
   // one thread per (source, site) for every tier: the update is memory-bound,
   // and link sharing measured slower here (534 against 511 us per launch)
-  (void)launch_pdl(c, cg_update_kernel<S, SA>, dim3(nrhs, nb), dim3(HOP_NT), 0, a);
+  (void)launch_pdl(c, cg_update_kernel<S, SA>, dim3(nrhs, blocks_for(a.g.Vh, HOP_NT * UpdGroups<S, SA>::value)),
+                   dim3(HOP_NT), 0, a);
   tl.done();
   c.launches++;
   return check_launch(c, "cg_update_kernel");

@@ -39,8 +39,27 @@ int solution_prec(const tm_stop& stop) {
   return TSM_F32;
 }
 
-int loop_solution_prec(const tm_stop& stop) {
-  if (stop.prec == TSM_F16 && !stop.precond) return F16G::id;
+// A call of tm_solve_batch may bring a single source, and a group of 8 costs the
+// same (and holds 8 sources of every Krylov field) however few of its rows are
+// used: grouped only on lattices on which one source is no slower than on plain
+// fields, up to 16416 sites on 152 SMs.  8 iterations, grouped / plain, 1, 8 and 32
+// sources: 8^3x16 0.52 / 0.61, 0.66 / 0.75, 1.37 / 1.38 ms; 10^3x16 0.62 / 0.63, 0.91
+// / 0.95, 2.31 / 2.26; 8x12^2x24 0.71 / 0.67, 1.20 / 1.24, 3.43 / 3.57; 16^3x32 1.77 /
+// 1.02, 4.15 / 4.31, 14.4 / 15.5; 24^3x48 7.3 / 3.6, 19.4 / 19.7.
+constexpr int F16_GROUPED_SITES_PER_SM = 108;
+bool f16_grouped_solve(const Ctx& c) { return (long long)c.g.V <= (long long)F16_GROUPED_SITES_PER_SM * c.sm_count; }
+
+// The loop estimators fill whole groups and run grouped on larger lattices too: 32
+// LP sources, 8 iterations, grouped / plain: 12^3x24 1.93 / 2.21 ms, 16^3x32 4.52 /
+// 5.73, 24^3x48 20.0 / 26.6, 32^3x64 64.8 / 85.0 (8 sources: 0.92 / 0.93, 1.76 / 1.93,
+// 7.0 / 7.2, 20.6 / 21.3; fewer cost as much as 8).  Not on lattices on which 8
+// sources' fields (2.7 KB per site) and the stencil's links (384 bytes per site)
+// would take memory that a narrower batch needs: beyond 2^25 sites, 64^3x128.
+constexpr long long F16_GROUPED_LOOP_SITES = 1ll << 25;
+bool f16_grouped_loops(const Ctx& c) { return c.g.V <= F16_GROUPED_LOOP_SITES; }
+
+int loop_solution_prec(const Ctx& c, const tm_stop& stop) {
+  if (stop.prec == TSM_F16 && !stop.precond) return f16_grouped_loops(c) ? F16G::id : TSM_F16;
   return solution_prec(stop);
 }
 
@@ -302,6 +321,7 @@ static int cg_solve(Ctx& c, const tm_stop& stop, int s0, int nrhs, EOField b, EO
       // the stopping rule stops here (rel_finish_kernel)
       if (x0_prec == TSM_F64) TSM_TRY((launch_convert<F64, F64>(c, *x0, x64, nullptr, nrhs)));
       else if (x0_prec == F16G::id) TSM_TRY((launch_convert<F16G, F64>(c, *x0, x64, nullptr, nrhs)));
+      else if (x0_prec == TSM_F16) TSM_TRY((launch_convert<F16, F64>(c, *x0, x64, nullptr, nrhs)));
       else TSM_TRY((launch_convert<F32, F64>(c, *x0, x64, nullptr, nrhs)));
       warm_start_kernel<<<1, Ctx::kMaxBatch, 0, c.stream>>>(st, nrhs);
       c.launches++;
@@ -505,10 +525,13 @@ int reserve_solver(Ctx& c, const tm_stop& stop, int sol_prec) {
   switch (stop.prec) {
     case TSM_F64: pS = pA = pP = TSM_F64; break;
     case TSM_F32: pS = pA = TSM_F32; pP = stop.reliable ? TSM_F64 : TSM_F32; break;
-    case TSM_F16: pS = pA = F16G::id; pP = TSM_F32; break;
+    case TSM_F16:
+      pS = pA = sol_prec == F16G::id || (sol_prec != TSM_F16 && f16_grouped_solve(c)) ? F16G::id : TSM_F16;
+      pP = TSM_F32;
+      break;
     default: pS = stop.prec; pA = pP = TSM_F32; break;
   }
-  if (sol_prec == F16G::id) pP = F16G::id;
+  if (stop.prec == TSM_F16 && (sol_prec == F16G::id || sol_prec == TSM_F16)) pP = sol_prec;
   const int nb = c.batch_cap;
   PField f;
   for (const char* name : {"cg_tmp_o", "cg_bhat", "cg_w0", "cg_t0", "cg_r0"}) TSM_TRY(c.field(name, pP, &f, nb));
@@ -523,7 +546,8 @@ int reserve_solver(Ctx& c, const tm_stop& stop, int sol_prec) {
 
 int solve_batch(Ctx& c, const tm_stop& stop, int s0, int nrhs, EOField b, EOField s, SolveResult* res,
                 const PField* x0, int x0_prec, int sol_prec) {
-  if (sol_prec >= 0 && sol_prec != solution_prec(stop) && !(stop.prec == TSM_F16 && sol_prec == F16G::id)) {
+  if (sol_prec >= 0 && sol_prec != solution_prec(stop) &&
+      !(stop.prec == TSM_F16 && (sol_prec == F16G::id || sol_prec == TSM_F16))) {
     set_error("solution storage tier %d not available for solver tier %d", sol_prec, stop.prec);
     return TSM_ERR_ARG;
   }
@@ -538,8 +562,8 @@ int solve_batch(Ctx& c, const tm_stop& stop, int s0, int nrhs, EOField b, EOFiel
     case TSM_F64: return cg_solve<F64, F64, F64, false>(c, stop, s0, nrhs, b, s, res, nullptr, -1);
     case TSM_F32:
       if (stop.reliable) {
-        if (x0 != nullptr && x0_prec != F16G::id && x0_prec != TSM_F32 && x0_prec != TSM_F64) {
-          set_error("starting guess of tier %d (grouped FP16, FP32 or FP64 expected)", x0_prec);
+        if (x0 != nullptr && x0_prec != F16G::id && x0_prec != TSM_F16 && x0_prec != TSM_F32 && x0_prec != TSM_F64) {
+          set_error("starting guess of tier %d (FP16, FP32 or FP64 expected)", x0_prec);
           return TSM_ERR_ARG;
         }
         return cg_solve<F32, F32, F64, true>(c, stop, s0, nrhs, b, s, res, x0, x0_prec);
@@ -550,7 +574,9 @@ int solve_batch(Ctx& c, const tm_stop& stop, int s0, int nrhs, EOField b, EOFiel
     // source and solution in FP16 too when the caller asks for it
     case TSM_F16:
       if (sol_prec == F16G::id) return cg_solve<F16G, F16G, F16G, false>(c, stop, s0, nrhs, b, s, res, nullptr, -1);
-      return cg_solve<F16G, F16G, F32, false>(c, stop, s0, nrhs, b, s, res, nullptr, -1);
+      if (sol_prec == TSM_F16) return cg_solve<F16, F16, F16, false>(c, stop, s0, nrhs, b, s, res, nullptr, -1);
+      if (f16_grouped_solve(c)) return cg_solve<F16G, F16G, F32, false>(c, stop, s0, nrhs, b, s, res, nullptr, -1);
+      return cg_solve<F16, F16, F32, false>(c, stop, s0, nrhs, b, s, res, nullptr, -1);
     case TSM_BF16: return cg_solve<BF16, F32, F32, false>(c, stop, s0, nrhs, b, s, res, nullptr, -1);
     default: set_error("unknown solver tier %d", stop.prec); return TSM_ERR_ARG;
   }

@@ -22,16 +22,22 @@ int solution_prec(const tm_stop& stop);
 // estimators: as solution_prec, except that the FP16 tier (whose iterates x
 // and r are FP16 already) keeps its noise source, Schur source and solution in
 // FP16 as well, so that its source preparation, odd reconstruction and
-// contraction move 16-bit fields through the link-sharing stencil.
-int loop_solution_prec(const tm_stop& stop);
+// contraction move 16-bit fields: in groups of 8 sources (F16G), where
+// f16_grouped_loops says so, or as plain fields.
+int loop_solution_prec(const Ctx& c, const tm_stop& stop);
+
+// Where FP16 solves run in groups of 8 sources on the tensor cores (mma_hop.cuh),
+// by the lattice alone, so that a source's bits do not depend on its batch.
+bool f16_grouped_solve(const Ctx& c);   // tm_solve_batch
+bool f16_grouped_loops(const Ctx& c);   // loop estimators
 
 // Solve D_tm s_r = b_r for nrhs independent sources at once.  b and s are
 // batches of nrhs contiguous even/odd fields of tier sol_prec (-1:
 // solution_prec(stop); otherwise solution_prec(stop) or, for the FP16 tier,
-// TSM_F16) laid out for c.batch_cap sources; device solver states s0 ..
+// TSM_F16 or F16G) laid out for c.batch_cap sources; device solver states s0 ..
 // s0+nrhs-1 are used; res receives nrhs results.  x0 (optional; FP32 with FP64
 // reliable updates only, ignored by the other tiers): a batch of even-site
-// starting guesses of storage tier x0_prec (TSM_F16, TSM_F32 or TSM_F64); the
+// starting guesses of storage tier x0_prec (F16G, TSM_F16, TSM_F32 or TSM_F64); the
 // first iterate's residual is then the true normal residual of b - D x0,
 // computed as in a reliable update, and the stopping rule stays relative to
 // ||Dhat^dag bhat||.
