@@ -508,9 +508,17 @@ enum PostOp {
 
 // stopping rule of the iterated residual: ||r|| < tol ||r0|| (NaN counts as
 // met), on the squares: an FP64 square root is about 20 dependent instructions
-// of 70 cycles at the end of every iteration
+// of 70 cycles at the end of every iteration.  A residual that underflowed to
+// zero is below every positive limit, also below one that did (sources of 1e-154
+// and less); that test is on bits, an FP64 comparison would join the chain.
 __host__ __device__ __forceinline__ bool rule_met(const CGState* st, double rr) {
-  return !(rr >= st->tol * st->tol * st->rr0);
+  const double limit = st->tol * st->tol * st->rr0;
+#ifdef __CUDA_ARCH__
+  const bool zero = __double_as_longlong(rr) == 0 && __double_as_longlong(st->tol) != 0;
+#else
+  const bool zero = rr == 0.0 && st->tol != 0.0;
+#endif
+  return zero || !(rr >= limit);
 }
 
 __device__ __forceinline__ void post_action(CGState* st, int op, double sum) {
