@@ -1142,6 +1142,8 @@ int tsm_tune(tsm_ctx* h, const tm_stop* stop, int* best_batch, int* best_tile, i
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
+  const int wt = c.check_waits();   // of the timed solves' last kernels
+  if (rc == TSM_OK) rc = wt;
   if (rc != TSM_OK) {
     if (tiled) {
       c.tile_rpb[stop->prec] = saved_rpb;

@@ -57,6 +57,7 @@ constexpr int MMA_GROUPS = 8;                        // groups of 8 sources of a
 constexpr int MMA_FLUSH = 8;                         // tiles whose norms add up in FP32 before they join the FP64 sum
 constexpr int MMA_CHUNKS = 24;                       // 16-byte chunks per site of a group
 constexpr long long MMA_SPIN_LIMIT = 1ll << 22;      // polls of a ring wait
+constexpr long long MMA_INJECT_LIMIT = 4096;         // the same where the copies are withheld (tests)
 
 // A tile of 2 x 2 rows of W half-sites: a warp per site and the copy warps (one
 // thread each).  Slots (sites) of a ring stage: the own rows [zz][yy][W + 2] from
@@ -141,11 +142,12 @@ struct MmaHopArgs {
   int post;
   RedSlot red;
   int* err;                    // host-mapped: set when a ring wait ran out
+  int withhold;                // fault injection: no copies, ring waits of MMA_INJECT_LIMIT polls
 };
 
 // ring wait: one try, then the bounded loop; true on timeout
-__device__ __forceinline__ bool mma_wait_failed(uint64_t* bar, uint32_t parity) {
-  return !mbar_try(bar, parity) && !mbar_wait(bar, parity, MMA_SPIN_LIMIT);
+__device__ __forceinline__ bool mma_wait_failed(uint64_t* bar, uint32_t parity, int withhold) {
+  return !mbar_try(bar, parity) && !mbar_wait(bar, parity, withhold ? MMA_INJECT_LIMIT : MMA_SPIN_LIMIT);
 }
 
 // d = a b (no accumulator: the tensor cores round a sum towards zero, so that only
@@ -412,7 +414,7 @@ __global__ void __launch_bounds__(MmaShape<W>::NT, 1) mma_hop_kernel(const MmaHo
       const MmaTiles& g = a.tl;
       MmaTile tl(g, blockIdx.y);
       int stage = 0, round = 0, issued = 0;
-      bool go = true;
+      bool go = !a.withhold;
       for (int tile = blockIdx.y; tile < ntile && go; tile += gridDim.y, tl.next(g)) {
         const int x0 = tl.tx * g.W, w = min(g.W, g.Lxh - x0), y0 = 2 * tl.yp, z0 = 2 * tl.zp, t = tl.t;
         const int ym = y0 == 0 ? g.Ly - 1 : y0 - 1, yp = y0 + 2 == g.Ly ? 0 : y0 + 2;
@@ -420,7 +422,7 @@ __global__ void __launch_bounds__(MmaShape<W>::NT, 1) mma_hop_kernel(const MmaHo
         const int tm = t == 0 ? g.T - 1 : t - 1, tp = t + 1 == g.T ? 0 : t + 1;
         const bool left = x0 == 0, right = x0 + w == g.Lxh;
         for (int j = 0; j < ng && go; ++j) {
-          if (round > 0 && mma_wait_failed(&s_empty[stage], (uint32_t)((round - 1) & 1)))
+          if (round > 0 && mma_wait_failed(&s_empty[stage], (uint32_t)((round - 1) & 1), 0))
             *reinterpret_cast<volatile int*>(&s_timeout) = 1;
           go = *reinterpret_cast<volatile int*>(&s_timeout) == 0;
           if (!go) break;
@@ -547,7 +549,7 @@ __global__ void __launch_bounds__(MmaShape<W>::NT, 1) mma_hop_kernel(const MmaHo
       valid = dx < width(tl);
       if (more && valid) fetch_links(site);
       for (int j = 0; j < ng; ++j) {
-        if (!dead && mma_wait_failed(&s_full[stage], (uint32_t)phase)) {
+        if (!dead && mma_wait_failed(&s_full[stage], (uint32_t)phase, a.withhold)) {
           dead = true;
           *reinterpret_cast<volatile int*>(&s_timeout) = 1;
         }

@@ -67,6 +67,8 @@ int umma_launch_any(cudaStream_t stream, dim3 grid, const __nv_bfloat16* A, cons
 
 }  // namespace
 
+int copies_withheld() { return g_umma_withhold.load(); }
+
 // C (FP32) = A (BF16, rows of length lda) * B (BF16, rows of length ldb)^T over
 // K columns (+ C if beta).  splits > 1: split-K, partial z written to
 // C + z * M * ldc (the caller reduces); *used_splits receives the number of
@@ -217,7 +219,7 @@ int layer_launch(Ctx& c, const NetGeom& ng, const NetLayer& l, const float* X, i
   const int gj = pt_groups(l.cin), steps = pt_steps(l.cin), smem = pt_layer_smem<BN>(gj);
   TSM_CUDA(cudaFuncSetAttribute(pt_layer_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   pt_layer_kernel<BN><<<dim3(grid1(c.g.V, PT_SITES), nb), 256, smem, c.stream>>>(ng, X, l.cin, l.Bs, 8 * l.cout, Y, gj,
-                                                                                 steps, err, g_umma_withhold.load());
+                                                                                 steps, err, copies_withheld());
   return check_net_launch(c, "pt_layer_kernel");
 }
 

@@ -43,6 +43,7 @@ MmaHopArgs mma_args(const Ctx& c, int p_out, int w, dim3* grid) {
   m.parity = p_out;
   m.links = c.links_of<F16G>(p_out);
   m.err = c.h_err;
+  m.withhold = copies_withheld();
   return m;
 }
 

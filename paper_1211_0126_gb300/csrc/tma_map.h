@@ -10,4 +10,7 @@ namespace tsm {
 // null when the driver does not have it
 PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder();
 
+// 1: operand copies are withheld (tsm_umma_inject_timeout)
+int copies_withheld();
+
 }  // namespace tsm
