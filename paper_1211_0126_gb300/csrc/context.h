@@ -221,8 +221,6 @@ int launch_noise(Ctx& c, int parity, const NoiseSpec& n, uint32_t source0, const
 template <class S>
 int launch_twist(Ctx& c, const Twist& f, const PField& in, const PField& out, const CGState* st,
                  const int* active = nullptr, int nrhs = 1);
-template <class S>
-int launch_norm(Ctx& c, const PField& v, CGState* st, int post, const int* active = nullptr, int nrhs = 1);
 template <class Si, class So>
 int launch_convert(Ctx& c, const PField& in, const PField& out, const int* active = nullptr, int nrhs = 1);
 

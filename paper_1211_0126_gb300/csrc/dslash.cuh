@@ -399,10 +399,10 @@ __global__ void __launch_bounds__(HOP_NT, HopMinBlocks<S>::value)
 // each (a warp per direction, so that no warp diverges), then warp s joins the
 // four sums of spin s in shared memory.  A warp-wide FP64 instruction occupies
 // its scheduler for about 70 cycles on GB300, so below one warp per scheduler
-// (152 x 4 warps of 32 sites) a thread per site takes the time of its ~1000
+// (four warps of 32 sites per SM) a thread per site takes the time of its ~1000
 // FP64 instructions, 37 us, however small the lattice; a thread of four issues
 // about 240.
-constexpr int SPLIT_SITES = 152 * 4 * 32;
+constexpr int SPLIT_SITES_PER_SM = 4 * 32;
 
 template <int DAG>
 __global__ void __launch_bounds__(128)

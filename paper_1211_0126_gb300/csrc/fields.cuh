@@ -417,25 +417,6 @@ static __global__ void warm_start_kernel(CGState* st, int n) {
   s.final_check = 1;
 }
 
-// <v, v> per right-hand side with post action (deterministic two-stage sum)
-template <class S>
-__global__ void __launch_bounds__(SITE_NT) norm_kernel(int Vh, const typename S::schunk* __restrict__ v, int sstride,
-                                                       RedSlot red, const int* active, CGState* st, int post) {
-  const int rhs = rhs_slot(active);
-  const int ih = blockIdx.y * SITE_NT + threadIdx.x;
-  double part = 0.0;
-  if (ih < Vh) {
-    cx<typename S::real> w[12];
-    load_spinor<S>(v + rhs_offset<S>(rhs, sstride), sstride, ih, w);
-    typename S::real s = 0;
-#pragma unroll
-    for (int k = 0; k < 12; ++k) s += norm2(w[k]);
-    part = (double)s;
-  }
-  double total;
-  if (grid_sum<SITE_NT>(part, red, rhs, &total) && threadIdx.x == 0) post_action(st + rhs, post, total);
-}
-
 // states 0 .. n-1: fresh solve
 static __global__ void state_init_kernel(CGState* st, int n, double tol, int max_iter, int rel, double delta2) {
   const int k = threadIdx.x + blockIdx.x * blockDim.x;

@@ -92,7 +92,7 @@ template <int MODE, class SH> struct MmaStage {
 // tiles of a lattice: ntx x nyp x nzp x T, x fastest; gx .. gt: the grid's
 // stride in the same mixed radix
 struct MmaTiles {
-  int Lxh, Ly, Lz, T, W, ntx, nyp, nzp, ntiles, apbc;
+  int Lxh, Ly, Lz, T, W, ntx, nyp, nzp, ntiles;
   int gx, gy, gz, gt;
 };
 

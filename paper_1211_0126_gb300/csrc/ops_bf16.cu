@@ -6,6 +6,4 @@ TSM_INSTANTIATE_STORAGE(BF16)
 TSM_INSTANTIATE_PAIR(BF16, F32)
 TSM_INSTANTIATE_CONVERT(F32, BF16)
 TSM_INSTANTIATE_CONVERT(BF16, F32)
-TSM_INSTANTIATE_CONVERT(F64, BF16)
-TSM_INSTANTIATE_CONVERT(BF16, F64)
 TSM_INSTANTIATE_CONVERT(BF16, BF16)

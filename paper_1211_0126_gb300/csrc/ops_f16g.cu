@@ -29,7 +29,6 @@ MmaHopArgs mma_args(const Ctx& c, int p_out, int w, dim3* grid) {
   t.nyp = t.Ly / 2;
   t.nzp = t.Lz / 2;
   t.ntiles = t.ntx * t.nyp * t.nzp * t.T;
-  t.apbc = c.g.apbc;
   const int gy = std::min(std::min(t.ntiles, c.sm_count), (int)c.red_cap);
   int n = gy;
   t.gx = n % t.ntx;

@@ -91,7 +91,7 @@ int launch_full(Ctx& c, const HopArgs<S>& e0, const HopArgs<S>& o0, int dag) {
   hop_factors(&o);
   const double sb = spinor_site_bytes(S::id), lb = link_site_bytes(S::id);
   TimedLaunch tl(c, 4 * S::id + (dag ? PK_HOP_DAG : PK_HOP_XPAY), 2.0 * c.g.Vh * (lb + 3.0 * sb));
-  if (S::id == F64::id && 2 * c.g.Vh < SPLIT_SITES) {
+  if (S::id == F64::id && 2 * c.g.Vh < SPLIT_SITES_PER_SM * c.sm_count) {
     const dim3 grid(blocks_for(c.g.Vh, 32), 1, 2);
     if constexpr (S::id == F64::id) {
       if (dag) split_hop_kernel<1><<<grid, 128, 0, c.stream>>>(e, o);
@@ -172,15 +172,6 @@ int launch_twist(Ctx& c, const Twist& f, const PField& in, const PField& out, co
   return check_launch(c, "twist_kernel");
 }
 
-template <class S>
-int launch_norm(Ctx& c, const PField& v, CGState* st, int post, const int* active, int nrhs) {
-  const int nb = blocks_for(c.g.Vh, SITE_NT);
-  if (nrhs == 0) return TSM_OK;
-  norm_kernel<S><<<dim3(nrhs, nb), SITE_NT, 0, c.stream>>>(c.g.Vh, v.as<S>(), c.sstride, c.red, active, st, post);
-  c.launches++;
-  return check_launch(c, "norm_kernel");
-}
-
 template <class Si, class So>
 int launch_convert(Ctx& c, const PField& in, const PField& out, const int* active, int nrhs) {
   const int nb = blocks_for(c.g.Vh, SITE_NT);
@@ -200,8 +191,7 @@ int launch_convert(Ctx& c, const PField& in, const PField& out, const int* activ
   template int tsm::launch_full<S>(Ctx&, const HopArgs<S>&, const HopArgs<S>&, int);                 \
   template int tsm::launch_noise<S>(Ctx&, int, const NoiseSpec&, uint32_t, const PField&, int);      \
   template int tsm::launch_twist<S>(Ctx&, const Twist&, const PField&, const PField&, const CGState*, \
-                                    const int*, int);                                                \
-  template int tsm::launch_norm<S>(Ctx&, const PField&, CGState*, int, const int*, int);
+                                    const int*, int);
 
 #define TSM_INSTANTIATE_PAIR(S, SA)                                                    \
   template int tsm::launch_cg_update<S, SA>(Ctx&, const CGUpdArgs<S, SA>&, int);      \
