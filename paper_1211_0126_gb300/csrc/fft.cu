@@ -247,12 +247,8 @@ __global__ void __launch_bounds__(FFT_XY_NT, XYMinBlocks<R>::value) fft_xy_kerne
 #pragma unroll
     for (int r = 0; r < 4; ++r)
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        cx<R> acc = cjmul(eta[3 * r], s[3 * c]);
-        acc = cjmac(acc, eta[3 * r + 1], s[3 * c + 1]);
-        acc = cjmac(acc, eta[3 * r + 2], s[3 * c + 2]);
-        S[r][c] = acc;
-      }
+      for (int c = 0; c < 4; ++c)
+        S[r][c] = cjdot3(eta[3 * r], s[3 * c], eta[3 * r + 1], s[3 * c + 1], eta[3 * r + 2], s[3 * c + 2]);
     for (int k = 0; k < gn; ++k) {
       const int gi = g0 + k;
       cx<R> d[4];
