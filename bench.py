@@ -81,9 +81,11 @@ def parse():
                          "1-12-12-12-1) at 16^3x32, timed with CUDA events (a small case for ncu captures of "
                          "the transport and tensor-core GEMM kernels)")
     ap.add_argument("--lp-only", action="store_true",
-                    help="only run one batched LP solve (32 Z4 sources, FP16 storage, 5e-3 or 60 iterations) at "
-                         "16^3x32 (a small case for ncu captures of the batched K1-K4 kernels; its fields exceed "
-                         "L2)")
+                    help="only run one LP batch of the loop estimators (32 Z4 sources, FP16, 3 iterations; a small "
+                         "case for ncu captures of the batched K1-K5 kernels; its fields exceed L2)")
+    ap.add_argument("--lp-lattice", default="16,16,16,32",
+                    help="lattice of --lp-only, Lx,Ly,Lz,T (default 16^3x32, hops in tiles of 4 half-sites; "
+                         "24,16,16,24 has tiles of 6)")
     ap.add_argument("--fft-only", action="store_true",
                     help="only run two all-momenta TSM estimates of 64 LP sources (FP16, batch 32) at 24^3x48 (a "
                          "small case for ncu captures of the FFT projection kernels)")
@@ -125,27 +127,23 @@ def run_net_only():
     ctx.close()
 
 
-def run_lp_only():
+def run_lp_only(dims):
+    """One batch of 32 LP solves of the loop estimators (FP16, 3 iterations), for a profiler."""
     import torch
     from paper_1211_0126_gb300 import build, tsm
     from paper_1211_0126_gb300 import synthetic as S
     if not os.path.exists(tsm.LIB_PATH):
         build.build()
-    dims = (16, 16, 16, 32)
-    stream = torch.cuda.current_stream()
-    ctx = tsm.Context(0, stream.cuda_stream)
+    ctx = tsm.Context(0, torch.cuda.current_stream().cuda_stream)
     ctx.load_gauge(S.gauge_field(dims, EPS, GAUGE_SEED), dims, KAPPA, MU)
-    V = int(np.prod(dims))
-    b = torch.zeros(32, V * 12, dtype=torch.complex128, device="cuda")
-    for j in range(32):
-        tsm.tsm_noise(ctx.h, 77, 4, j, b[j])
-    s = torch.zeros_like(b)
-    lp = tsm.stop(LP_TOL, LP_MAXIT, tsm.TSM_F16)
+    out = torch.zeros((1, 1, dims[3]), dtype=torch.complex128, device="cuda")
+    p = tsm.params(77, 4, (0, 0), (0, 32), tsm.stop(HP_TOL, HP_MAXIT, tsm.TSM_F64), tsm.stop(0.0, 3, tsm.TSM_F16),
+                   [0], [(0, 0, 0)], batch=32)
     torch.cuda.synchronize()
     t0 = time.perf_counter()
-    st, iters, _ = tsm.tm_solve_batch(ctx.h, b, s, lp, 32)
+    tsm.tsm_loops(ctx.h, p, out)
     torch.cuda.synchronize()
-    print(json.dumps({"lp_only": {"lattice": list(dims), "batch": 32, "iters_mean": float(np.mean(iters)),
+    print(json.dumps({"lp_only": {"lattice": list(dims), "batch": 32, "iters": 3,
                                   "ms": (time.perf_counter() - t0) * 1e3}}), flush=True)
     ctx.close()
 
@@ -515,15 +513,21 @@ def tune_table(tsm, times):
 
 def kernel_source_hash():
     h = hashlib.sha256()
-    for f in ("mma_hop.cuh", "common.cuh"):
+    for f in ("mma_hop.cuh", "dslash.cuh", "common.cuh", "mbar.cuh", "ops_f16g.cu"):
         with open(os.path.join(ROOT, "paper_1211_0126_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
 
 
-def ncu_traffic():
-    """DRAM bytes per hop launch from the committed ncu summary, if it was
-    taken on the current kernel source (else None)."""
+def hop_tile_width(lx):
+    """width in half-sites of the FP16 hops' tiles on rows of lx sites (mma_width in ops_f16g.cu)"""
+    h = lx // 2
+    return 6 if 6 * (-(-h // 6)) <= 4 * (-(-h // 4)) else 4
+
+
+def ncu_traffic(dims):
+    """Committed ncu capture of the FP16 LP kernels with the tiles that `dims`
+    runs, if it was taken on the current kernel source (else None)."""
     p = os.path.join(ROOT, "profiles", "hop_traffic.json")
     if not os.path.exists(p):
         return None
@@ -531,7 +535,7 @@ def ncu_traffic():
         d = json.load(f)
     if d.get("source_hash") != kernel_source_hash():
         return None
-    return d
+    return d["captures"].get(str(hop_tile_width(dims[0])))
 
 
 def run_ours(args):
@@ -629,7 +633,7 @@ def run_ours(args):
     dom = slice(12, 16)
     tot_ms, tot_bytes, tot_cnt = float(prof_ms[dom].sum()), float(prof_bytes[dom].sum()), int(prof_cnt[dom].sum())
     achieved = tot_bytes / (tot_ms * 1e-3) / 1e9 if tot_ms > 0 else None
-    traffic = ncu_traffic()
+    traffic = ncu_traffic(DIMS)
     per_kernel = {}
     for b in range(16):
         if prof_cnt[b]:
@@ -655,8 +659,9 @@ def run_ours(args):
                 "frac": (achieved / peak) if achieved else None,
                 "traffic": (traffic["dram_over_algorithmic"] * alg_per_launch
                             if (traffic and alg_per_launch) else None),
-                "traffic_source": ("ncu DRAM/algorithmic ratio of the same kernels at 16^3x32 x 32 sources, "
-                                   "scaled to this launch" if traffic else "no capture for this kernel source"),
+                "traffic_source": ("ncu DRAM/algorithmic ratio of the same kernels and tile width at %s x 32 "
+                                   "sources, scaled to this launch" % "x".join(map(str, traffic["lattice"]))
+                                   if traffic else "no capture for this kernel source and tile width"),
                 "algorithmic_bytes_per_launch": alg_per_launch,
                 "alu": {"flop_per_source_site": 1320, "achieved_tflops": alu_tflops, "peak_tflops": fp32_peak,
                         "frac": (alu_tflops / fp32_peak) if (alu_tflops and fp32_peak) else None,
@@ -1262,7 +1267,7 @@ def main():
     if args.net_only:
         run_net_only()
     elif args.lp_only:
-        run_lp_only()
+        run_lp_only(tuple(int(x) for x in args.lp_lattice.split(",")))
     elif args.fft_only:
         run_fft_only()
     elif args.contract_only:

@@ -55,9 +55,9 @@ __global__ void __launch_bounds__(256) pt_pack_stages_kernel(const __nv_bfloat16
 // says so at the stage's barrier, where all leave the loop together, the MMAs and
 // copies in flight are waited for (bounded), TMEM is freed and the error is
 // recorded.  withhold: fault injection as in umma.cuh (no weight copies).
-// 12 -> 12 channels at 16^3x32: 346 us against 310 (gather, 680 MB of Z written)
+// 12 -> 12 channels at 16^3x32: 340 us against 310 (gather, 680 MB of Z written)
 // + 170 (GEMM); 12 -> 1: 267 against 310 + 108.  Bound by the latency of the
-// neighbour loads (16 warps of 120 registers per SM, 36 % issue; the ring leaves
+// neighbour loads (16 warps of 128 registers per SM, 40 % issue; the ring leaves
 // 30 KB of L1).
 template <int BN>
 __global__ void __launch_bounds__(256, BN <= 128 ? 2 : 1)

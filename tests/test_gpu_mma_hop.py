@@ -12,6 +12,10 @@ u = 2^-11 (p, t, w, t, r, x) and applies four hops whose links are rounded to u,
 all of norm about one here (8 kappa ~ 1), so the solution's relative error is
 at most about 10 n u; 16 n u is required normwise, and 64 n u of the largest
 component at every site (a wrong neighbour is off by about 2 kappa).
+
+(Tiles of 4 half-sites are those of the CG update; the hops of rows of 5, 6 and 9
+to 12 half-sites run in tiles of up to 6.  Each block has one tile here;
+test_gpu_mma_tiles.py has several.)
 """
 import numpy as np
 import pytest
