@@ -341,8 +341,9 @@ int tsm_tune_batch(tsm_ctx* ctx, const tm_stop* stop, int* best, double* times_m
  * per context, lattice and stopping rule.  times_ms (may be NULL): 16 entries,
  * [width k][shape q] = ms per source for widths {8, 16, 32, 64} and shapes
  * {2 sources / 80 registers, 4 / 80, 8 / 80, 4 / 96} (0 where a shape does not
- * apply; TSM_F16, whose blocks are fixed, is timed once per width and reports
- * that time for every shape).  tsm_tune_batch runs the same search and reports, per width, the best
+ * apply; TSM_F16 solves in groups of 8, whose blocks are fixed, are timed once
+ * per width, with that time reported for every shape, and the shape that
+ * tsm_set_tile last set is reported and kept).  tsm_tune_batch runs the same search and reports, per width, the best
  * time over the shapes. */
 int tsm_tune(tsm_ctx* ctx, const tm_stop* stop, int* best_batch, int* best_tile, int* best_regs, double* times_ms);
 

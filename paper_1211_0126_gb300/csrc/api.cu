@@ -1074,10 +1074,14 @@ int tsm_tune(tsm_ctx* h, const tm_stop* stop, int* best_batch, int* best_tile, i
   const bool fixed16 = sp == F16G::id;
   const bool tiled = stop->prec == TSM_F16 || stop->prec == TSM_BF16 || stop->prec == TSM_F32;
   const int ntile = tiled && !fixed16 ? kShapes : 1;
+  // FP16: the shape of the solves on plain fields stays as it is set
+  int set_q = 1;
+  for (int q = 0; q < kShapes; ++q)
+    if (c.tile_rpb[TSM_F16] == tiles[q] && c.tile_regs[TSM_F16] == regs[q]) set_q = q;
   auto ib = c.tuned_batch.find(key);
   auto it = c.tuned_rpb.find(key);
   if (ib != c.tuned_batch.end() && it != c.tuned_rpb.end() && times_ms == nullptr) {
-    const int q = it->second;
+    const int q = fixed16 ? set_q : it->second;
     *best_batch = ib->second;
     if (best_tile) *best_tile = tiled ? tiles[q] : 1;
     if (best_regs) *best_regs = tiled ? regs[q] : 0;
@@ -1114,7 +1118,7 @@ int tsm_tune(tsm_ctx* h, const tm_stop* stop, int* best_batch, int* best_tile, i
       });
     }
     for (int q = 0; q < ntile && rc == TSM_OK; ++q) {
-      if (tiled) {
+      if (tiled && !fixed16) {
         c.tile_rpb[stop->prec] = tiles[q];
         c.tile_regs[stop->prec] = regs[q];
       }
@@ -1134,7 +1138,7 @@ int tsm_tune(tsm_ctx* h, const tm_stop* stop, int* best_batch, int* best_tile, i
       if (per < best_t) {
         best_t = per;
         best_w = w;
-        best_q = fixed16 ? 1 : q;
+        best_q = fixed16 ? set_q : q;
       }
     }
     if (times_ms && !tiled)

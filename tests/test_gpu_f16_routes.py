@@ -70,3 +70,16 @@ def test_one_source_of_a_large_lattice_holds_one_source(libtsm):
         assert used <= V // 2 * (8 * 96 + 5 * 48) + 20 * (2 << 20), used
     finally:
         c.close()
+
+
+def test_tuner_keeps_the_shape_of_plain_solves(ctx):
+    """The estimators' FP16 solves have no block shape to tune; the one set for the
+    solves on plain fields is reported and left as it is, first time and cached."""
+    dims = (4, 4, 4, 4)
+    ctx.load_gauge(S.gauge_field(dims, 0.3, 7), dims, KAPPA, MU)
+    stop = tsm.stop(0.0, 3, tsm.TSM_F16)
+    for shape in ((4, 96), (8, 80)):
+        tsm.tsm_set_tile(ctx.h, tsm.TSM_F16, *shape)
+        for _ in range(2):
+            width, sources, regs, times = tsm.tsm_tune(ctx.h, stop)
+            assert (sources, regs) == shape and np.all(times > 0) and width in (8, 16, 32, 64)
