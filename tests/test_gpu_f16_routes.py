@@ -83,3 +83,56 @@ def test_tuner_keeps_the_shape_of_plain_solves(ctx):
         for _ in range(2):
             width, sources, regs, times = tsm.tsm_tune(ctx.h, stop)
             assert (sources, regs) == shape and np.all(times > 0) and width in (8, 16, 32, 64)
+
+
+HP, LP = tsm.stop(1e-10, 5000, tsm.TSM_F32, reliable=True), tsm.stop(5e-3, 60, tsm.TSM_F16)
+GAM = list(range(16))
+
+
+@pytest.mark.parametrize("kw", [{}, {"estimator": 1}, {"estimator": 2}, {"deriv_mask": 5}, {"hp_warm_start": True}])
+@pytest.mark.parametrize("n_hp,n_lp,batch", [(1, 1, 1), (3, 2, 8), (3, 9, 2), (11, 20, 4), (8, 3, 8)])
+def test_estimates_do_not_depend_on_shared_groups(ctx, kw, n_hp, n_lp, batch):
+    """LP-set sources that fill the HP set's last group of 8 have the values of a call
+    without HP sources, the HP set's those of a call without LP sources."""
+    dims = (4, 4, 2, 4)
+    ctx.load_gauge(S.gauge_field(dims, 0.3, 7), dims, KAPPA, MU)
+    def run(hp, lp):
+        return ctx.loops(9, 4, 0, 0, HP, LP, GAM, S.default_momenta(4), hp_range=hp, lp_range=lp, per_source=True,
+                         batch=batch, **kw)
+    both = run((0, n_hp), (n_hp, n_hp + n_lp))
+    hp_only, lp_only = run((0, n_hp), (n_hp, n_hp)), run((0, 0), (n_hp, n_hp + n_lp))
+    assert np.array_equal(both["per_corr"], hp_only["per_corr"])
+    assert np.array_equal(both["per_lp"], lp_only["per_lp"])
+    assert both["stats"]["lp_iters"] == hp_only["stats"]["lp_iters"] + lp_only["stats"]["lp_iters"]
+    comb = ctx.combine(both["per_corr"], both["per_lp"])
+    assert np.array_equal(comb["loops"], both["loops"]) and np.array_equal(comb["err"], both["err"])
+
+
+@pytest.mark.parametrize("n_hp,n_lp", [(2, 9), (9, 40)])
+def test_all_momenta_with_shared_groups(ctx, n_hp, n_lp):
+    """The running moments of both sets against the direct projection (bounds of
+    test_gpu_fft.py's mixed tier)."""
+    dims = (4, 6, 2, 4)
+    ctx.load_gauge(S.gauge_field(dims, 0.3, 5), dims, KAPPA, MU)
+    moms = [(0, 0, 0), (1, 0, 0), (-1, 2, 1)]
+    direct = ctx.loops(13, 4, n_hp, n_lp, HP, LP, GAM, moms, batch=4)
+    allq = ctx.loops(13, 4, n_hp, n_lp, HP, LP, GAM, None, batch=4, all_momenta=True)
+    for k, (nx, ny, nz) in enumerate(moms):
+        i = (slice(None), slice(None), nz % dims[2], ny % dims[1], nx % dims[0])
+        for name, tol in (("loops", 1e-5), ("err", 1e-4)):
+            scale = np.abs(direct[name][:, k, :]).max()
+            assert np.abs(allq[name][i] - direct[name][:, k, :]).max() < tol * scale, name
+
+
+def test_few_lp_sources_share_the_group_of_the_hp_set(ctx):
+    """1 HP source and up to 7 LP sources are one group: LP sources add no solve, a few
+    launches for their noise and contraction."""
+    dims = (4, 4, 4, 4)
+    ctx.load_gauge(S.gauge_field(dims, 0.3, 7), dims, KAPPA, MU)
+    fixed = tsm.stop(0.0, 8, tsm.TSM_F16)
+    def launches(n_lp):
+        a = tsm.tsm_launch_count(ctx.h)
+        ctx.loops(9, 4, 1, n_lp, HP, fixed, GAM, S.default_momenta(4), batch=8)
+        return tsm.tsm_launch_count(ctx.h) - a
+    base = launches(0)
+    assert launches(1) <= base + 6 and launches(7) <= base + 6
