@@ -397,11 +397,12 @@ int record_run(Ctx& c, const tsm_params* p, TsmRun& run, tsm_loop_stats* st) {
   uint32_t lp_next = p->lp_begin;
   for (uint32_t l0 = p->hp_begin; l0 < p->hp_end; l0 += BH) {
     const int nl = (int)std::min<uint32_t>(BH, p->hp_end - l0);
-    // a group of 8 costs the same however few of its rows are used: the first
-    // sources of the LP set fill the last one (24^3x48, 1 HP and 1 LP source: 32.1
-    // -> 26.0 ms, 1 and 4: 32.4 -> 26.3)
+    // a group of 8 costs the same however few of its rows are used: sources of the LP
+    // set that would leave one part-filled take the rows that are left here, if there
+    // are enough (24^3x48, 1 HP and 1 LP source: 32.1 -> 26.0 ms, 1 and 4: 32.4 -> 26.3)
     const int fill = sp_lp == F16G::id && !c.capturing ? ((nl + 7) & ~7) - nl : 0;
-    const int nx = (int)std::min<uint32_t>(fill, p->lp_end - lp_next);
+    const int odd = (int)((p->lp_end - lp_next) % 8);
+    const int nx = odd <= fill ? odd : 0;
     TSM_TRY(gen(sp_lp, l0, run.b_lp, nl));
     if (nx > 0) {
       const size_t row = rhs_offset<F16G>(nl, c.sstride);   // the rows left of the last group

@@ -92,7 +92,7 @@ GAM = list(range(16))
 @pytest.mark.parametrize("kw", [{}, {"estimator": 1}, {"estimator": 2}, {"deriv_mask": 5}, {"hp_warm_start": True}])
 @pytest.mark.parametrize("n_hp,n_lp,batch", [(1, 1, 1), (3, 2, 8), (3, 9, 2), (11, 20, 4), (8, 3, 8)])
 def test_estimates_do_not_depend_on_shared_groups(ctx, kw, n_hp, n_lp, batch):
-    """LP-set sources that fill the HP set's last group of 8 have the values of a call
+    """LP-set sources that share the HP set's last group of 8 have the values of a call
     without HP sources, the HP set's those of a call without LP sources."""
     dims = (4, 4, 2, 4)
     ctx.load_gauge(S.gauge_field(dims, 0.3, 7), dims, KAPPA, MU)
